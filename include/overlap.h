@@ -88,8 +88,9 @@ typedef struct {
   int    wilson_variant;/* Wilson-kernel launch shape: -1 autotune at create (default), 0 one
                            thread per site, 1 four threads per site (one per direction), 2 one
                            thread per site on 8x4x4x2 tiles (needs extents divisible by those),
-                           3 two threads per site, one per half spinor (double-float only; the
-                           other precisions use 0)                                           */
+                           3 as 0. Double-float (two threads per pair of sites, one per half
+                           spinor): 0, 3, 2, 1 share the eight hops of a pair among 1, 2, 4, 8
+                           groups of threads; -1 takes the number by the size of each launch  */
   int    use_graphs;    /* 1 (default): run the multi-shift CG iterations as cached CUDA graphs
                            (not while profiling); 0: launch every kernel on the stream        */
   int    verify;        /* 1: after a solve, recompute ||b - D x|| / ||b|| with an FP64 sign at

@@ -70,20 +70,22 @@ static void convert_links(const double* links, const int L[4], int bc_t, std::ve
   const int V = L[0] * L[1] * L[2] * L[3];
   // canonical [site][mu][row][col] complex -> [mu][chunk][V] keeping rows 0, 1.
   // The double-float copy holds, for each site x, the matrix of each of the eight hops
-  // in slot n = 2 mu + b: b = 0 U_mu(x), b = 1 U_mu(x - mu)^dag, all 9 entries
-  // ([n][chunk][V]), with the antiperiodic-t sign of the hops that cross the boundary
-  // folded in.
+  // in slot n = 2 mu + b: b = 0 U_mu(x), b = 1 U_mu(x - mu)^dag, all 9 entries, in the
+  // pair layout ([i / 32][n][2 e + r][i % 32] of (hi, hi', lo, lo') for the sites i, i + V/2), with
+  // the antiperiodic-t sign of the hops that cross the boundary folded in.
   l64.assign((size_t)4 * 6 * V * 2, 0.0);
   l32.assign((size_t)4 * 3 * V * 4, 0.f);
   l16.assign((size_t)4 * 3 * V * 4, __float2half(0.f));
-  l64e.assign((size_t)8 * 9 * V * 4, 0.f);
+  l64e.assign((size_t)df_blocks(V) * 8 * 18 * 32 * 4, 0.f);
   auto put_df = [&](int n, int e, int s, double re, double im) {
     const float rh = (float)re, ih = (float)im;
-    float* d = &l64e[(((size_t)n * 9 + e) * V + s) * 4];
+    const int h = s >= V / 2 ? 1 : 0;
+    const int i = s - h * (V / 2);
+    float* d = &l64e[((((size_t)(i / 32) * 8 + n) * 18 + 2 * e) * 32 + i % 32) * 4 + h];
     d[0] = rh;
-    d[1] = (float)(re - (double)rh);
-    d[2] = ih;
-    d[3] = (float)(im - (double)ih);
+    d[2] = (float)(re - (double)rh);
+    d[128] = ih;
+    d[130] = (float)(im - (double)ih);
   };
   const int str[4] = {1, L[0], L[0] * L[1], L[0] * L[1] * L[2]};
   for (int s = 0; s < V; ++s) {
@@ -118,7 +120,7 @@ static void convert_links(const double* links, const int L[4], int bc_t, std::ve
 }
 
 // Create-time autotuner: the Wilson-kernel launch shapes (thread per site, direction split,
-// 4D tiles when the lattice divides into them, and for double-float the lane-pair form)
+// 4D tiles when the lattice divides into them; for double-float 1, 8, 4 and 2 thread groups)
 // timed for every storage precision on this lattice (random input), once with one system
 // and once with a batch (min(12, batch_max) systems; 4 in double-float), and the fastest
 // kept for each (another shape must beat the thread-per-site one by 5%).
@@ -174,6 +176,9 @@ static ovl_status autotune_wilson(ovl_ctx* c) {
       int best = 0;
       for (int v = 1; v < nv; ++v)
         if (wt[v] > 0.f && wt[v] < 0.95f * wt[0] && wt[v] < wt[best]) best = v;
+      // the double-float kernel takes its shape from each launch's size (wilson_df_variant); its
+      // timings are kept for ovl_wilson_tuning
+      if (p == P64E) best = wilson_df_variant(c->V, ns);
       (bucket == 0 ? c->wvar[p] : c->wvar_multi[p]) = best;
     }
     free_field(c->ws["at_in"]);
@@ -771,7 +776,7 @@ static ovl_status defl_alloc(ovl_ctx* c, ovl_defl* d, int prec, int cap) {
     f.prec = prec;
     f.V = c->V;
     f.n = cap;
-    if (cudaMalloc(&f.data, (size_t)spinor_site_bytes(prec) * c->V * cap) != cudaSuccess) {
+    if (cudaMalloc(&f.data, field_bytes(prec, c->V) * cap) != cudaSuccess) {
       cudaGetLastError();
       f.data = nullptr;
       return set_err(c, OVL_ENOMEM, "cudaMalloc failed for the deflation space");

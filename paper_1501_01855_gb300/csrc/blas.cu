@@ -231,7 +231,7 @@ void launch_gamma5(int p, SpinorRef x, int nrhs, int V, cudaStream_t st) {
   else gamma5_kernel<P16><<<sh.grid(), sh.block(), 0, st>>>(x, nrhs, V, sh.ngr);
 }
 void launch_zero(int p, SpinorRef x, int nrhs, int V, cudaStream_t st) {
-  const size_t per = (size_t)V * spinor_site_bytes(p);
+  const size_t per = field_bytes(p, V);
   cudaMemsetAsync(x.data, 0, per * nrhs, st);
   if (p == P16 && x.norm) cudaMemsetAsync(x.norm, 0, sizeof(float) * V * nrhs, st);
 }

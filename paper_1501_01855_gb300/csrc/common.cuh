@@ -7,7 +7,10 @@
 // site s at [c*V + s], so that a warp reading chunk c of 32 consecutive sites
 // issues one fully coalesced 512-byte transaction:
 //   F64:  12 chunks of double2 (1 complex)                       192 B/site
-//   F64E: 12 chunks of float4 (re.hi, re.lo, im.hi, im.lo)        192 B/site
+//   F64E: 24 chunks per pair of sites (i, i + V/2), chunk 2 k + r the real (r = 0) or
+//         imaginary part of component k, in blocks of 32 pairs (the last one padded):
+//         [i / 32][2 k + r][i % 32] float4 (hi_i, hi_i+V/2, lo_i, lo_i+V/2), so
+//         that the chunks of a pair lie at constant distances      192 B/site
 //         = the same number as a double, held as an unevaluated sum hi + lo
 //         of two floats (double-float, ~48-bit significand)
 //   F32:   6 chunks of float4  (2 complex)                         96 B/site
@@ -17,8 +20,12 @@
 //
 // Links keep only rows 1 and 2 of each SU(3) matrix (12 reals); row 3 is
 // rebuilt in registers as conj(row1 x row2). Layout [mu][chunk][V]:
-//   F64: 6 chunks double2, F64E: 6 chunks float4, F32: 3 chunks float4,
-//   F16: 3 chunks of 4 halves.
+//   F64: 6 chunks double2, F32: 3 chunks float4, F16: 3 chunks of 4 halves.
+// F64E links: eight slots per site, one per hop (slot n = 2 mu + b holds U_mu(x) for b = 0 and
+// U_mu(x - mu)^dag for b = 1, with the antiperiodic sign folded in), all 9 entries, in pairs
+// of sites like the spinors: [i / 32][n][2 e + r][i % 32] float4. The double-float kernel is bound by
+// FP32 arithmetic, not bytes: rebuilding row 3 would cost a fifth of it, and transposed
+// backward links let one loop body serve all eight neighbours.
 #pragma once
 #include <cuda_runtime.h>
 #include <cuda_fp16.h>
@@ -113,6 +120,12 @@ template <> struct Real<P64> { using T = double; };
 template <> struct Real<P64E> { using T = df; };
 
 __host__ __device__ constexpr int spinor_site_bytes(int p) { return p == P32 ? 96 : p == P16 ? 48 : 192; }
+// double-float: blocks of 32 pairs of sites, the last one padded
+__host__ __device__ constexpr int df_blocks(int V) { return (V / 2 + 31) / 32; }
+// bytes of one spinor field (F16: without its scales)
+__host__ __device__ constexpr size_t field_bytes(int p, int V) {
+  return p == P64E ? (size_t)df_blocks(V) * 24 * 32 * 16 : (size_t)V * spinor_site_bytes(p);
+}
 
 // ------------------------------------------------------------------ spinors
 // A batch of spinor fields in device memory.
@@ -150,20 +163,31 @@ struct SpinorIO<P64, RO> {
     for (int c = 0; c < 12; ++c) p[(size_t)c * f.V] = make_double2(v[c].r, v[c].i);
   }
 };
+// one site of the pair layout (conversions and rare paths; the kernels of dfpair.cuh take pairs)
 template <bool RO>
 struct SpinorIO<P64E, RO> {
+  static __device__ __forceinline__ size_t at(const SpinorRef& f, int rhs, int s) {
+    const int Vh = f.V >> 1, h = s >= Vh ? 1 : 0, i = s - h * Vh;
+    return (((size_t)rhs * df_blocks(f.V) + (i >> 5)) * 768 + (i & 31)) * 4 + h;
+  }
   static __device__ __forceinline__ void load(const SpinorRef& f, int rhs, int s, cpx<df> v[12]) {
-    const float4* p = reinterpret_cast<const float4*>(f.data) + (size_t)rhs * 12 * f.V + s;
+    const float* p = reinterpret_cast<const float*>(f.data) + at(f, rhs, s);
+    constexpr int st = 128;   // floats from one real number of a pair to the next
 #pragma unroll
-    for (int c = 0; c < 12; ++c) {
-      float4 w = ldc<RO>(p + (size_t)c * f.V);
-      v[c] = cmk(df(w.x, w.y), df(w.z, w.w));
-    }
+    for (int c = 0; c < 12; ++c)
+      v[c] = cmk(df(ldc<RO>(p + 2 * c * st), ldc<RO>(p + 2 * c * st + 2)),
+                 df(ldc<RO>(p + (2 * c + 1) * st), ldc<RO>(p + (2 * c + 1) * st + 2)));
   }
   static __device__ __forceinline__ void store(const SpinorRef& f, int rhs, int s, const cpx<df> v[12]) {
-    float4* p = reinterpret_cast<float4*>(f.data) + (size_t)rhs * 12 * f.V + s;
+    float* p = reinterpret_cast<float*>(f.data) + at(f, rhs, s);
+    constexpr int st = 128;
 #pragma unroll
-    for (int c = 0; c < 12; ++c) p[(size_t)c * f.V] = make_float4(v[c].r.hi, v[c].r.lo, v[c].i.hi, v[c].i.lo);
+    for (int c = 0; c < 12; ++c) {
+      p[2 * c * st] = v[c].r.hi;
+      p[2 * c * st + 2] = v[c].r.lo;
+      p[(2 * c + 1) * st] = v[c].i.hi;
+      p[(2 * c + 1) * st + 2] = v[c].i.lo;
+    }
   }
 };
 template <bool RO>
@@ -278,7 +302,8 @@ __device__ __forceinline__ void store_spinor_any(const SpinorRef& f, int rhs, in
 struct LinkRef {
   const void* data;  // [mu][chunk][V]
   int V;
-  int variant;       // Wilson-kernel variant chosen for this field (0 thread per site, 1 split)
+  int variant;       // Wilson-kernel variant chosen for this field (0 thread per site, 1 split, 2 tiles;
+                     // double-float: 0, 3, 2, 1 for 1, 2, 4, 8 thread groups, -1 by launch size)
   int variant_multi; // the variant chosen for launches of 4 or more systems
 };
 
@@ -293,7 +318,6 @@ __device__ __forceinline__ void reconstruct_row3(cpx<T> u[9]) {
 template <int P> struct LinkIO;
 template <>
 struct LinkIO<P64> {
-  static constexpr bool full = false;
   static __device__ __forceinline__ void load(const LinkRef& L, int mu, int s, cpx<double> u[9]) {
     const double2* p = reinterpret_cast<const double2*>(L.data) + (size_t)mu * 6 * L.V + s;
 #pragma unroll
@@ -303,26 +327,8 @@ struct LinkIO<P64> {
     }
   }
 };
-// Double-float links: eight slots per site, one per hop (slot n = 2 mu + b holds U_mu(x)
-// for b = 0 and U_mu(x - mu)^dag for b = 1), all 9 entries ([n][9 chunks][V] float4
-// chunks). The double-float kernel is bound by FP32 instruction issue, not bytes:
-// rebuilding row 3 would cost ~20% of its instructions, and pre-transposed backward
-// links let one loop body serve all eight neighbours.
-template <>
-struct LinkIO<P64E> {
-  static constexpr bool full = true;
-  static __device__ __forceinline__ void load(const LinkRef& L, int slot, int s, cpx<df> u[9]) {
-    const float4* p = reinterpret_cast<const float4*>(L.data) + (size_t)slot * 9 * L.V + s;
-#pragma unroll
-    for (int c = 0; c < 9; ++c) {
-      float4 w = __ldg(p + (size_t)c * L.V);
-      u[c] = cmk(df(w.x, w.y), df(w.z, w.w));
-    }
-  }
-};
 template <>
 struct LinkIO<P32> {
-  static constexpr bool full = false;
   static __device__ __forceinline__ void load(const LinkRef& L, int mu, int s, cpx<float> u[9]) {
     const float4* p = reinterpret_cast<const float4*>(L.data) + (size_t)mu * 3 * L.V + s;
 #pragma unroll
@@ -335,7 +341,6 @@ struct LinkIO<P32> {
 };
 template <>
 struct LinkIO<P16> {
-  static constexpr bool full = false;
   static __device__ __forceinline__ void load(const LinkRef& L, int mu, int s, cpx<float> u[9]) {
     const uint2* p = reinterpret_cast<const uint2*>(L.data) + (size_t)mu * 3 * L.V + s;
 #pragma unroll
@@ -354,7 +359,7 @@ template <int P, typename T>
 __device__ __forceinline__ void load_link(const LinkRef& L, int mu, int s, cpx<T> u[9]) {
   static_assert(std::is_same<T, typename Real<P>::T>::value, "links load in their own compute type");
   LinkIO<P>::load(L, mu, s, u);
-  if constexpr (!LinkIO<P>::full) reconstruct_row3(u);
+  reconstruct_row3(u);
 }
 
 // ------------------------------------------------------------------ geometry

@@ -1,0 +1,424 @@
+// The double-float Wilson kernel: K of dslash.cu (same modes, same meaning of its arguments)
+// with FP64-level accuracy on the FP32 pipes.
+//
+// Arithmetic: packed double-float (dfpair.cuh), lane 0 the site i of the first half of the
+// lattice in t, lane 1 the site i + V/2. Fields hold the pair's high words and low words as
+// one 16-byte chunk per real number, links likewise, so every load is a natural operand.
+//
+// Threads: two lanes of a warp share a pair of sites, lane `half` holding upper spin `half`.
+// The projection (1 -+ gamma_mu) leaves two half spinors h0, h1 (upper spins 0 and 1 plus a
+// power of i times a lower spin); the thread builds h_half, multiplies it by the link of the
+// hop (eight-slot link field: U_mu(x), or U_mu(x - mu)^dag, boundary sign folded in) and adds
+// the result to its upper spin and, times a power of i, to one lower spin: spin 3 - half for
+// mu <= 1, which the other lane owns (the sums change lanes once, after mu = 1), spin
+// 2 + half for mu >= 2. One rolled loop body serves every hop (unrolled over all eight it
+// leaves the instruction cache): a power of i only chooses which of the two chunks (re, im)
+// of the lower spin is loaded into which operand, and a sign, which rides on a multiply-add.
+//
+// What bounds it (ncu, 16^3 x 32, K): the FP32 pipes are busy 61% of the cycles (527 packed
+// operations per thread and hop), the rest is the latency of the loads that three warps per
+// scheduler do not cover. 168 registers (12 warps per SM) against 128 (16 warps, spilling and
+// scheduled with less overlap): 0.530 against 0.841 ms on 16^3 x 32 with 12 systems. Measured there
+// against the scalar kernel before it (one thread per site, 12 operations per product term):
+// K launch 0.678 -> 0.517 ms, on 24^3 x 48 2.61 ms (3.0 G site applications/s; 2.4 before), one
+// system on 16^3 x 32 0.070 -> 0.060 ms; a whole sign to 1e-10, 12 systems, 181 -> 146 ms. Error against
+// FP64 4.7e-15 of the norm (4.8e-15 before), with the hops shared among groups 3.4e-15 to 4.4e-15.
+#include "dfpair.cuh"
+#include "wilson.cuh"
+
+namespace ovl {
+
+namespace {
+
+constexpr int DP = 32;   // pairs of sites per block (64 sites: the partial sums keep the BX layout)
+
+// threads of a block (64 per group) and the resident blocks per SM its registers are capped for
+constexpr int df_threads(int G) { return 64 * G; }
+constexpr int df_resident(int G) { return G == 1 ? 6 : G == 2 ? 3 : G == 4 ? 2 : 1; }
+
+// partial sums each mode produces
+constexpr int df_nred(int mode) { return mode == MODE_OVL ? 4 : mode == MODE_K ? 2 : 1; }
+
+__device__ __forceinline__ void prefetch_l1(const void* p) { asm volatile("prefetch.global.L1 [%0];" ::"l"(p)); }
+
+// hop n seen from one thread
+struct Hop {
+  int nbr;        // index of the neighbour pair
+  bool swap;      // its lanes are exchanged (the hop leaves this half of the lattice in t)
+  int other;      // lower spin the projection pairs with spin `half`
+  int a, b;       // powers of i of the projection and of the lower-spin sum
+};
+__device__ __forceinline__ Hop hop_of(const Geom& g, int lth, const int x[4], int i, int half, int n) {
+  const int mu = n >> 1;
+  const bool fwd = (n & 1) == 0;
+  const int sS = fwd ? 2 : 0;   // (1 + S gamma_mu) with S = i^sS
+  const bool lo3 = mu <= 1;
+  const int a0 = sS + (mu == 0 || mu == 2 ? 1 : mu == 1 ? 2 : 0);
+  const int a1 = sS + (mu == 0 ? 1 : mu == 2 ? 3 : 0);
+  const int b0 = sS + (mu == 0 || mu == 2 ? 3 : 0);
+  const int b1 = sS + (mu == 0 ? 3 : mu == 1 ? 2 : mu == 2 ? 1 : 0);
+  Hop h;
+  h.other = lo3 ? 3 - half : 2 + half;
+  h.a = (half == 0 ? a0 : a1) & 3;
+  h.b = ((half == 0) == lo3 ? b1 : b0) & 3;
+  const int xm = mu == 0 ? x[0] : mu == 1 ? x[1] : mu == 2 ? x[2] : x[3];
+  const int lm = mu == 0 ? g.L[0] : mu == 1 ? g.L[1] : mu == 2 ? g.L[2] : lth;
+  const int st = mu == 0 ? 1 : mu == 1 ? g.L[0] : mu == 2 ? g.L[0] * g.L[1] : g.L[0] * g.L[1] * g.L[2];
+  const bool wrap = fwd ? xm == lm - 1 : xm == 0;
+  h.nbr = fwd ? (wrap ? i - (lm - 1) * st : i + st) : (wrap ? i + (lm - 1) * st : i - st);
+  h.swap = wrap && mu == 3;
+  return h;
+}
+
+// where the chunks of pair i of a field of nb blocks, and of the links of its hop n, begin
+__device__ __forceinline__ const ulonglong2* pair_at(const SpinorRef& in, size_t fblk, int i) {
+  return reinterpret_cast<const ulonglong2*>(in.data) + ((fblk + (i >> 5)) * 768 + (i & 31));
+}
+__device__ __forceinline__ const ulonglong2* link_at(const LinkRef& L, int i, int n) {
+  return reinterpret_cast<const ulonglong2*>(L.data) + ((size_t)((i >> 5) * 8 + n) * 576 + (i & 31));
+}
+// Prefetch of the next hop into L1, shared out over the lanes of a warp: eight pairs in a row
+// make a 128-byte line of every chunk, so of the sixteen lanes that hold them lane `m` fetches
+// chunks m and m + 16 at its own pair (one prefetch per lane and chunk asked for every line
+// sixteen times: 21 instructions per lane and hop instead of these 2 to 4).
+__device__ __forceinline__ void prefetch_spinor(const ulonglong2* b, int m) {
+  prefetch_l1(b + m * 32);
+  if (m < 8) prefetch_l1(b + (m + 16) * 32);
+}
+__device__ __forceinline__ void prefetch_link(const ulonglong2* u, int m) {
+  prefetch_l1(u + m * 32);
+  if (m < 2) prefetch_l1(u + (m + 16) * 32);
+}
+__device__ __forceinline__ void prefetch_l2_spinor(const ulonglong2* b, int m) {
+  asm volatile("prefetch.global.L2 [%0];" ::"l"(b + m * 32));
+  if (m < 8) asm volatile("prefetch.global.L2 [%0];" ::"l"(b + (m + 16) * 32));
+}
+// the operands of colour c of the projection: re, im of the upper spin and of the (i^a times)
+// lower spin of the neighbour
+struct Oper {
+  ulonglong2 p0, p1, q0, q1;
+};
+__device__ __forceinline__ Oper load_oper(const ulonglong2* b, int half, const Hop& h, int c) {
+  const ulonglong2* p = b + half * 192;
+  const ulonglong2* q0 = b + h.other * 192 + (h.a & 1) * 32;
+  const ulonglong2* q1 = b + h.other * 192 + 32 - (h.a & 1) * 32;
+  return {__ldg(p + 64 * c), __ldg(p + 64 * c + 32), __ldg(q0 + 64 * c), __ldg(q1 + 64 * c)};
+}
+__device__ __forceinline__ float sgn_re(int k) { return k == 1 || k == 2 ? -1.f : 1.f; }
+__device__ __forceinline__ float sgn_im(int k) { return k >= 2 ? -1.f : 1.f; }
+
+// up[c][r]: upper spin `half`; low[c][r]: the lower spin of the current half of the hops.
+// b, u: the neighbour's chunks and the link of this hop.
+template <bool TIGHT>
+__device__ __forceinline__ void hop_pair(const ulonglong2* b, const ulonglong2* u, int half, const Hop& h,
+                                         dd2 up[3][2], dd2 low[3][2]) {
+  const f2 ar = bc(sgn_re(h.a)), ai = bc(sgn_im(h.a));
+  dot2p wr[3], wi[3];
+#pragma unroll
+  for (int c = 0; c < 3; ++c) {
+    const Oper o = load_oper(b, half, h, c);
+    dd2 hr = dd2_lazy({o.p0.x, o.p0.y}, {o.q0.x, o.q0.y}, ar);
+    dd2 hi = dd2_lazy({o.p1.x, o.p1.y}, {o.q1.x, o.q1.y}, ai);
+    if (h.swap) {
+      hr = {swap2(hr.h), swap2(hr.l)};
+      hi = {swap2(hi.h), swap2(hi.l)};
+    }
+    const f2 nr = neg2(hr.h), ni = neg2(hi.h), nil = neg2(hi.l);
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+      const ulonglong2 ur = __ldg(u + (3 * a + c) * 64), ui = __ldg(u + (3 * a + c) * 64 + 32);
+      // w = U h: re = sum (Ur hr - Ui hi), im = sum (Ur hi + Ui hr)
+      if (c == 0) {
+        wr[a] = dot2p_first(ur.x, ur.y, hr.h, nr, hr.l);
+        wi[a] = dot2p_first(ur.x, ur.y, hi.h, ni, hi.l);
+      } else {
+        dot2p_add<TIGHT>(wr[a], ur.x, ur.y, hr.h, nr, hr.l);
+        dot2p_add<TIGHT>(wi[a], ur.x, ur.y, hi.h, ni, hi.l);
+      }
+      dot2p_add<TIGHT>(wr[a], ui.x, ui.y, ni, hi.h, nil);
+      dot2p_add<TIGHT>(wi[a], ui.x, ui.y, hr.h, nr, hr.l);
+    }
+  }
+  const bool oddb = (h.b & 1) != 0;
+  const f2 br = bc(sgn_re(h.b)), bi = bc(sgn_im(h.b));
+#pragma unroll
+  for (int a = 0; a < 3; ++a) {
+    const dd2 r = {wr[a].s, wr[a].c}, m = {wi[a].s, wi[a].c};
+    up[a][0] = dd2_lazy(up[a][0], r);
+    up[a][1] = dd2_lazy(up[a][1], m);
+    low[a][0] = dd2_lazy(low[a][0], oddb ? m : r, br);
+    low[a][1] = dd2_lazy(low[a][1], oddb ? r : m, bi);
+  }
+}
+
+__device__ __forceinline__ dd2 shfl_pair(dd2 v) {
+  return {__shfl_xor_sync(0xffffffffu, v.h, 1), __shfl_xor_sync(0xffffffffu, v.l, 1)};
+}
+
+// The epilogue of N complex components kc .. kc + N - 1 of the pair (the mode list of dslash.cu):
+// hop sums in, partial sums into d. Every load is issued before the first store (which may alias
+// them as far as the compiler can know).
+struct DfScal {
+  fac2 kap, s0, s1;   // -kappa; LZK: 1 / n_j; LZL: -a, -b; R: sigma0, -alpha; OVL: c1, c2
+};
+template <int MODE, int PIO, int N>
+__device__ __forceinline__ void df_epilogue(const DArgs& a, const DfScal& k, int rhs, int fin, int j, int kc, int i,
+                                            const dd2 (*sum)[2], dot2p d[4]) {
+  const int nb = df_blocks(a.g.V);
+  const bool red = a.partials != nullptr;
+  const bool two = MODE == MODE_LZL ? j > 0 : MODE == MODE_OVL ? a.coef != nullptr || a.c1 != 0.0 : true;
+  dd2 o[N][2], w[N][2], y[N][2];
+#pragma unroll
+  for (int c = 0; c < N; ++c)
+#pragma unroll
+    for (int r = 0; r < 2; ++r) {
+      o[c][r] = dfp_ldg(a.in, dfp_at(fin, kc + c, r, i, nb));
+      if constexpr (MODE == MODE_R) {
+        w[c][r] = dfp_ld(a.aux1, dfp_at(rhs, kc + c, r, i, nb));
+        y[c][r] = dfp_ld(a.aux2, dfp_at(rhs, kc + c, r, i, nb));
+      } else if constexpr (MODE == MODE_LZL) {
+        w[c][r] = dfp_ld(a.aux1, dfp_at(j * a.nrhs + rhs, kc + c, r, i, nb));
+        if (two) y[c][r] = dfp_ld(a.aux1, dfp_at((j - 1) * a.nrhs + rhs, kc + c, r, i, nb));
+      }
+    }
+  if constexpr (MODE == MODE_OVL) {
+#pragma unroll
+    for (int c = 0; c < N; ++c) {
+      if (two) dfp_load<PIO>(a.aux1, rhs, kc + c, i, w[c][0], w[c][1]);
+      if (red) dfp_load<PIO>(a.aux2, rhs, kc + c, i, y[c][0], y[c][1]);
+    }
+  }
+#pragma unroll
+  for (int c = 0; c < N; ++c) {
+#pragma unroll
+    for (int r = 0; r < 2; ++r) {
+      // in - kappa hop; gamma5 negates the lower spins
+      dd2 t = dd2_add(o[c][r], dd2_mul(k.kap, sum[c][r]));
+      if (MODE != MODE_OVL && kc >= 6) t = dd2_neg(t);
+      if constexpr (MODE == MODE_K) {
+        if (red) dot2p_add(d[1], o[c][r], o[c][r]);
+      } else if constexpr (MODE == MODE_R) {
+        t = dd2_add(y[c][r], dd2_mul(k.s1, dd2_add(t, dd2_mul(k.s0, w[c][r]))));
+      } else if constexpr (MODE == MODE_LZK) {
+        t = dd2_mul(k.s0, t);
+      } else if constexpr (MODE == MODE_LZL) {
+        t = dd2_add(t, dd2_mul(k.s0, w[c][r]));
+        if (two) t = dd2_add(t, dd2_mul(k.s1, y[c][r]));
+      } else {
+        t = dd2_mul(k.s1, t);
+        if (two) t = dd2_add(dd2_mul(k.s0, w[c][r]), t);
+        if (a.herm && kc >= 6) t = dd2_neg(t);
+      }
+      if (MODE != MODE_OVL && red) dot2p_add(d[0], t, t);
+      o[c][r] = t;
+    }
+    if constexpr (MODE == MODE_OVL) {
+      if (red) {
+        dot2p_add(d[0], y[c][0], o[c][0]);   // (w, out) = sum conj(w) out
+        dot2p_add(d[0], y[c][1], o[c][1]);
+        dot2p_add(d[1], y[c][0], o[c][1]);
+        dot2p_add(d[1], dd2_neg(y[c][1]), o[c][0]);
+        dot2p_add(d[2], o[c][0], o[c][0]);
+        dot2p_add(d[2], o[c][1], o[c][1]);
+        dot2p_add(d[3], y[c][0], y[c][0]);
+        dot2p_add(d[3], y[c][1], y[c][1]);
+      }
+    }
+  }
+  const SpinorRef& out = MODE == MODE_R ? a.aux2 : a.out;
+  const int fld = MODE == MODE_LZL ? (j + 1) * a.nrhs + rhs : rhs;
+#pragma unroll
+  for (int c = 0; c < N; ++c) dfp_store<MODE == MODE_OVL ? PIO : P64E>(out, fld, kc + c, i, o[c][0], o[c][1]);
+}
+
+// G groups of threads (threadIdx.z) share the eight hops of a pair, 8 / G each; their sums
+// meet in shared memory, where group z finishes the components z, z + G, .. of the spinor.
+template <int MODE, int PIO, int G>
+__global__ void __launch_bounds__(df_threads(G), df_resident(G)) df_wilson_kernel(const DArgs a) {
+  constexpr int NR = df_nred(MODE);
+  extern __shared__ ulonglong2 part[];   // G > 1: [z][component (6 x re, im)][thread x]
+  __shared__ double red[2 * G][NR];
+  const int half = threadIdx.x & 1;
+  const int grp = G > 1 ? threadIdx.z : 0;
+  const int sb = blockIdx.x / a.nrhs;   // the systems of one site block together: they share its links in L1 / L2
+  const int rhs = blockIdx.x - sb * a.nrhs;
+  const int Vh = a.g.V >> 1;
+  const int i = sb * DP + (threadIdx.x >> 1);
+  bool live = i < Vh;
+  if (live && a.ms != nullptr && (MODE == MODE_K || MODE == MODE_R)) live = !a.ms[rhs].done;
+  int fin = rhs, j = 0;   // field index of the hop input (the basis slot in MODE_LZK)
+  if constexpr (MODE == MODE_LZK || MODE == MODE_LZL) {
+    if (live) live = !a.lz[rhs].done;
+    if (live) j = a.lz[rhs].j;
+    if (MODE == MODE_LZK) fin = j * a.nrhs + rhs;
+  }
+  dd2 up[3][2], low[3][2];
+#pragma unroll
+  for (int c = 0; c < 3; ++c)
+#pragma unroll
+    for (int r = 0; r < 2; ++r) up[c][r] = low[c][r] = dd2_zero();
+  {
+    const int lth = a.g.L[3] >> 1;
+    const size_t fblk = (size_t)fin * df_blocks(a.g.V);
+    int x[4] = {0, 0, 0, 0};
+    if (live) site_coords(a.g, i, x);
+    const int n0 = grp * (8 / G), n1 = n0 + 8 / G;
+    const int m = (threadIdx.x >> 1 & 7) + 8 * half;
+    Hop h = hop_of(a.g, lth, x, i, half, n0);
+    const ulonglong2* b = pair_at(a.in, fblk, h.nbr);
+    const ulonglong2* u = link_at(a.links, i, n0);
+    if (live) {
+      prefetch_spinor(b, m);
+      prefetch_link(u, m);
+      if constexpr (MODE == MODE_LZL) {   // the basis vectors of the epilogue come from HBM
+        prefetch_l2_spinor(pair_at(a.aux1, (size_t)(j * a.nrhs + rhs) * df_blocks(a.g.V), i), m);
+        if (j > 0) prefetch_l2_spinor(pair_at(a.aux1, (size_t)((j - 1) * a.nrhs + rhs) * df_blocks(a.g.V), i), m);
+      }
+    }
+#pragma unroll 1
+    for (int n = n0; n < n1; ++n) {
+      if (live) {
+        const int nn = min(n + 1, n1 - 1);
+        const Hop nx = hop_of(a.g, lth, x, i, half, nn);
+        const ulonglong2 *bn = pair_at(a.in, fblk, n + 1 < n1 ? nx.nbr : i), *un = link_at(a.links, i, nn);
+        prefetch_spinor(bn, m);   // after the last hop the epilogue reads the pair itself
+        if (n + 1 < n1) prefetch_link(un, m);
+        hop_pair<(G >= 4)>(b, u, half, h, up, low);
+        h = nx;
+        b = bn;
+        u = un;
+      }
+      // the lower spins of mu <= 1 belong to the other lane: exchanged after the last of them
+      // (every lane of the warp takes part; the hops of a warp are the same)
+      if (n == min(n1 - 1, 3)) {
+#pragma unroll
+        for (int c = 0; c < 3; ++c)
+#pragma unroll
+          for (int r = 0; r < 2; ++r) {
+            low[c][r] = shfl_pair(dd2_norm(low[c][r]));
+            up[c][r] = dd2_norm(up[c][r]);
+          }
+      }
+    }
+  }
+  dot2p d[4];
+#pragma unroll
+  for (int k = 0; k < 4; ++k) d[k] = {0ull, 0ull};
+  DfScal k;
+  if (live) {
+    k.kap = fac2_bc(-a.kappa);
+    if constexpr (MODE == MODE_LZK) {
+      k.s0 = fac2_bc(a.lz[rhs].inv_n);
+    } else if constexpr (MODE == MODE_LZL) {
+      k.s0 = fac2_bc(-a.lz[rhs].a);
+      k.s1 = fac2_bc(-a.lz[rhs].b);
+    } else if constexpr (MODE == MODE_R) {
+      k.s0 = fac2_bc(a.sigma0);
+      k.s1 = fac2_bc(-a.ms[rhs].alpha);
+    } else if constexpr (MODE == MODE_OVL) {
+      k.s0 = fac2_bc(a.coef ? a.coef[2 * rhs] : a.c1);
+      k.s1 = fac2_bc(a.coef ? a.coef[2 * rhs + 1] : a.c2);
+    }
+  }
+  if constexpr (G == 1) {
+    if (live) {
+      df_epilogue<MODE, PIO, 3>(a, k, rhs, fin, j, 3 * half, i, up, d);
+      df_epilogue<MODE, PIO, 3>(a, k, rhs, fin, j, 6 + 3 * half, i, low, d);
+    }
+  } else {
+    ulonglong2* mine = part + grp * 12 * 64 + threadIdx.x;
+#pragma unroll
+    for (int c = 0; c < 3; ++c)
+#pragma unroll
+      for (int r = 0; r < 2; ++r) {
+        mine[(2 * c + r) * 64] = make_ulonglong2(up[c][r].h, up[c][r].l);
+        mine[(6 + 2 * c + r) * 64] = make_ulonglong2(low[c][r].h, low[c][r].l);
+      }
+    __syncthreads();
+    if (live) {
+      for (int q = grp; q < 6; q += G) {
+        const ulonglong2* s = part + 2 * q * 64 + threadIdx.x;
+        dd2 t[1][2];
+#pragma unroll
+        for (int r = 0; r < 2; ++r) {
+          t[0][r] = {s[r * 64].x, s[r * 64].y};
+#pragma unroll
+          for (int z = 1; z < G; ++z) {
+            const ulonglong2 w = s[(z * 12 + r) * 64];
+            t[0][r] = dd2_add(t[0][r], {w.x, w.y});
+          }
+        }
+        df_epilogue<MODE, PIO, 1>(a, k, rhs, fin, j, q < 3 ? 3 * half + q : 3 + 3 * half + q, i, t, d);
+      }
+    }
+  }
+  if (a.partials != nullptr) {
+    // warps in the order x, z: fixed, so that the sum is
+    const int warp = threadIdx.z * 2 + (threadIdx.x >> 5);
+#pragma unroll
+    for (int q = 0; q < NR; ++q) {
+      double v = dot2p_get(d[q]);
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
+      if ((threadIdx.x & 31) == 0) red[warp][q] = v;
+    }
+    __syncthreads();
+    if (threadIdx.x == 0 && threadIdx.z == 0) {
+      double* out = a.partials + ((size_t)rhs * a.nsb + sb) * NVRED;
+#pragma unroll
+      for (int q = 0; q < NR; ++q) {
+        double t = 0.0;
+        for (int z = 0; z < G; ++z) t += red[2 * z][q] + red[2 * z + 1][q];
+        out[q] = t;
+      }
+#pragma unroll
+      for (int q = NR; q < NVRED; ++q) out[q] = 0.0;
+    }
+  }
+  if constexpr (MODE == MODE_LZK || MODE == MODE_LZL) {
+    if (a.lzc.ctr != nullptr) lz_arrive<MODE>(a, rhs, a.nsb);
+  }
+}
+
+template <int MODE, int PIO, int G>
+void run_g(DArgs a, cudaStream_t st) {
+  const size_t smem = G == 1 ? 0 : sizeof(ulonglong2) * 64 * 12 * G;
+  if (smem > 40 * 1024)   // with the static arrays, past the 48 KB that need no opt-in
+    cudaFuncSetAttribute(df_wilson_kernel<MODE, PIO, G>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  df_wilson_kernel<MODE, PIO, G><<<dim3((unsigned)(a.nsb * a.nrhs)), dim3(64, 1, G), smem, st>>>(a);
+}
+
+template <int MODE, int PIO>
+void run_m(const DArgs& a, cudaStream_t st) {
+  switch (a.variant >= 0 ? a.variant : wilson_df_variant(a.g.V, a.nrhs)) {
+    case 0: run_g<MODE, PIO, 1>(a, st); break;
+    case 3: run_g<MODE, PIO, 2>(a, st); break;
+    case 2: run_g<MODE, PIO, 4>(a, st); break;
+    default: run_g<MODE, PIO, 8>(a, st); break;
+  }
+}
+
+}  // namespace
+
+// Two threads per pair and system, times 1, 2, 4 or 8 groups. One group is the cheapest form
+// (no exchange in shared memory) once its threads fill the SMs; below, the hops of a pair are
+// spread over more groups. K launches, us with 1 / 2 / 4 / 8 groups: 49152 threads (8^4, 12
+// systems) 24.6 / 24.7 / 30.8 / 32.9; 32768 (8^3 x 16, 4) 18.5 / 18.5 / 22.6 / 22.6; 20736 (12^4, 1)
+// 18.5 / 14.5 / 18.5 / 18.6; 16384 (8^4, 4) 14.4 / 12.4 / 12.4 / 12.6; 8192 (8^3 x 16, 1)
+// 14.4 / 10.3 / 8.3 / 8.3; 4096 (8^4, 1) 14.4 / 10.4 / 8.3 / 8.2.
+int wilson_df_variant(int V, int nrhs) {
+  const long long threads = (long long)V * nrhs;
+  return threads >= 40000 ? 0 : threads >= 18000 ? 3 : threads >= 9000 ? 2 : 1;
+}
+
+void run_wilson_df(int mode, int pio, DArgs a, cudaStream_t st) {
+  a.nsb = make_shape(a.g.V, a.nrhs).nsb;
+  if (mode == MODE_K) run_m<MODE_K, P64E>(a, st);
+  else if (mode == MODE_R) run_m<MODE_R, P64E>(a, st);
+  else if (mode == MODE_LZK) run_m<MODE_LZK, P64E>(a, st);
+  else if (mode == MODE_LZL) run_m<MODE_LZL, P64E>(a, st);
+  else if (pio == P64) run_m<MODE_OVL, P64>(a, st);
+  else run_m<MODE_OVL, P32>(a, st);
+}
+
+}  // namespace ovl

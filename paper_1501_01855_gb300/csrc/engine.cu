@@ -69,7 +69,7 @@ ovl_status get_field(ovl_ctx* c, const std::string& name, int prec, int n, Field
   f.prec = prec;
   f.V = c->V;
   f.n = n;
-  const size_t bytes = spinor_bytes(prec) * (size_t)c->V * n;
+  const size_t bytes = field_bytes(prec, c->V) * n;
   if (cudaMalloc(&f.data, bytes) != cudaSuccess) {
     cudaGetLastError();
     f.data = nullptr;
@@ -153,7 +153,7 @@ ovl_status ensure_lz(ovl_ctx* c, int nrhs, int cap) {
 }
 
 ovl_status lz_pool_field(ovl_ctx* c, int prec, int n, Field* out) {
-  const size_t data = (size_t)spinor_bytes(prec) * c->V * n;
+  const size_t data = field_bytes(prec, c->V) * n;
   const size_t norms = prec == P16 ? sizeof(float) * (size_t)c->V * n : 0;
   const size_t need = data + norms;
   if (need > c->lz_pool_bytes) {
@@ -217,6 +217,8 @@ LinkRef links_of(const ovl_ctx* c, int prec) {
   r.V = c->V;
   r.variant = c->wvar[prec];
   r.variant_multi = c->wvar_multi[prec];
+  // not forced: the double-float kernel chooses by the size of each launch
+  if (prec == P64E && (c->P.wilson_variant < 0 || c->P.wilson_variant > 3)) r.variant = r.variant_multi = -1;
   return r;
 }
 
@@ -460,7 +462,7 @@ ovl_status sign_op(ovl_ctx* c, int mode, const Field& v, int voff, Field& out, i
   for (int j = 0; j < n; ++j) emin = std::min(emin, eta[j] > 0 ? eta[j] : c->eps_sign);
   if (!c->exact_rational) emin = std::max(emin, c->delta);
   const int cap = lz_cap_for(c, mode, emin);
-  const double per_lz = (double)cap * c->V * (spinor_bytes(PP) + (PP == P16 ? 4.0 : 0.0));
+  const double per_lz = (double)cap * ((double)field_bytes(PP, c->V) + (PP == P16 ? 4.0 * c->V : 0.0));
   // the basis budget: params.basis_gb, and never more than 70% of what the device has free
   // (counting the pool this context already holds); the rest is left to the workspaces of
   // the solvers around the sign, and a workspace that still does not fit takes the pool back
@@ -491,7 +493,7 @@ ovl_status sign_op(ovl_ctx* c, int mode, const Field& v, int voff, Field& out, i
     }
     return OVL_OK;
   }
-  const double per = (double)c->npoles * c->V * spinor_bytes(PP);
+  const double per = (double)c->npoles * (double)field_bytes(PP, c->V);
   int nb = std::max(1, std::min(c->P.batch_max, (int)(kPoleBytes / per)));
   if (n <= nb) return sign_op_batch(c, mode, v, voff, out, ooff, n, eta, c1, c2, coef, herm, dot_w, woff, dots, stats);
   if (stats) {

@@ -25,10 +25,10 @@ struct Field {
   int V = 0;
   void* data = nullptr;
   float* norm = nullptr;
-  size_t chunk_bytes() const { return (size_t)n * V * spinor_site_bytes(prec); }
+  size_t chunk_bytes() const { return (size_t)n * field_bytes(prec, V); }
   SpinorRef ref(int off = 0) const {
     SpinorRef r;
-    const size_t per = (size_t)V * spinor_site_bytes(prec);
+    const size_t per = field_bytes(prec, V);
     r.data = data ? (void*)((char*)data + per * off) : nullptr;
     r.norm = norm ? norm + (size_t)V * off : nullptr;
     r.V = V;
@@ -96,6 +96,8 @@ struct Shape {
 Shape make_shape(int V, int nrhs);
 // the lattice is covered by whole tiles of Wilson-kernel variant 2
 bool wilson_tiles_fit(const Geom& g);
+// the variant the double-float Wilson kernel takes for a launch of nrhs systems
+int wilson_df_variant(int V, int nrhs);
 
 // ---------------------------------------------------------------- Wilson kernel
 // K in (Sec. 1) with optional per-(rhs, block) partials {||out||^2, ||in||^2}.

@@ -27,6 +27,7 @@
 // r_i = -||v|| (T_k + sigma_i)^-1_{k-1,0} W_k, parallel to the last vector, so the rest
 // of the sum is the same problem started from W_k with weights w_i ||v|| (-y_i,k-1): the
 // cycle's part of y is added and the next cycle starts there.
+#include "dfpair.cuh"
 #include "kernels.h"
 
 namespace ovl {
@@ -79,13 +80,45 @@ __global__ void __launch_bounds__(256) lz_init_kernel(SpinorRef v, SpinorRef W, 
   }
 }
 
+// Double-float: one thread per pair of sites and system.
+constexpr int DP = 32;   // pairs per block: the partial sums keep the 64-site blocks
+template <int PV>
+__global__ void __launch_bounds__(128) lz_init_df_kernel(SpinorRef v, SpinorRef W, SpinorRef y, int nrhs, int Vh,
+                                                         int nsb, int ngr, double* partials) {
+  const int sb = blockIdx.x / ngr;
+  const int rhs = (blockIdx.x - sb * ngr) * blockDim.y + threadIdx.y;
+  const int i = sb * DP + threadIdx.x;
+  dot2p d = {0ull, 0ull};
+  if (i < Vh && rhs < nrhs) {
+#pragma unroll 4
+    for (int k = 0; k < 12; ++k) {
+      dd2 re, im;
+      dfp_load<PV>(v, rhs, k, i, re, im);
+      dfp_store<P64E>(W, rhs, k, i, re, im);
+      dfp_store<P64E>(y, rhs, k, i, dd2_zero(), dd2_zero());
+      dot2p_add(d, re, re);
+      dot2p_add(d, im, im);
+    }
+  }
+  double s = dot2p_get(d);
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
+  if (threadIdx.x == 0 && rhs < nrhs) {
+    partials[((size_t)rhs * nsb + sb) * NVRED + 0] = s;
+    partials[((size_t)rhs * nsb + sb) * NVRED + 1] = 0.0;
+  }
+}
+
 void launch_lz_init(int pv, int pw, int py, SpinorRef v, SpinorRef W, SpinorRef y, int nrhs, int V,
                     double* partials, cudaStream_t st) {
   Shape sh = make_shape(V, nrhs);
 #define LZI(A, B, C) lz_init_kernel<A, B, C><<<sh.grid(), sh.block(), 0, st>>>(v, W, y, nrhs, V, sh.nsb, sh.ngr, partials)
   if (pv == P64 && pw == P64 && py == P64) LZI(P64, P64, P64);
-  else if (pv == P64 && pw == P64E && py == P64E) LZI(P64, P64E, P64E);
-  else if (pv == P32 && pw == P64E && py == P64E) LZI(P32, P64E, P64E);
+  else if (pw == P64E && py == P64E && (pv == P64 || pv == P32)) {
+    const dim3 block(DP, sh.by), grid(sh.grid());
+    if (pv == P64) lz_init_df_kernel<P64><<<grid, block, 0, st>>>(v, W, y, nrhs, V / 2, sh.nsb, sh.ngr, partials);
+    else lz_init_df_kernel<P32><<<grid, block, 0, st>>>(v, W, y, nrhs, V / 2, sh.nsb, sh.ngr, partials);
+  }
   else if (pv == P64 && pw == P32 && py == P32) LZI(P64, P32, P32);
   else if (pv == P32 && pw == P32 && py == P32) LZI(P32, P32, P32);
   else if (pv == P64 && pw == P16 && py == P32) LZI(P64, P16, P32);
@@ -228,42 +261,43 @@ void launch_lz_coef(LzRhs* lz, const double* ahist, const double* bhist, int cap
 }
 
 // ---------------------------------------------------------------- combine
-// y += sum_{l < k} coefW_l W_l. Double-float: chunk-major (one complex component of y at
-// a time, every stored vector's chunk read once), coefficients converted to double-float
-// once per block in shared memory.
-__global__ void __launch_bounds__(256) lz_combine_df_kernel(SpinorRef W, SpinorRef y, const double* coefW,
-                                                            const LzRhs* lz, int cap, int nrhs, int V, int ngr) {
-  extern __shared__ float2 cf[];   // [blockDim.y][cap]
-  const int sb = blockIdx.x / ngr;
-  const int rg = blockIdx.x - sb * ngr;
-  const int rhs = rg * blockDim.y + threadIdx.y;
-  const bool in_rhs = rhs < nrhs;
-  const int k = in_rhs ? lz[rhs].j : 0;
-  float2* c = cf + (size_t)threadIdx.y * cap;
-  if (in_rhs) {
-    for (int l = threadIdx.x; l < k; l += blockDim.x) {
-      const double v = coefW[(size_t)rhs * cap + l];
-      const float h = (float)v;
-      c[l] = make_float2(h, (float)(v - (double)h));
-    }
+// y += sum_{l < k} coefW_l W_l. Double-float: one thread per 16-byte chunk (one real number of
+// a pair of sites), every stored vector's chunk read once, eight loads in flight; coefficients
+// converted to double-float once per block in shared memory. Bound by HBM on large batches;
+// the chunk as a grid dimension keeps a small lattice from running 24 chunks in series.
+__global__ void __launch_bounds__(128) lz_combine_df_kernel(SpinorRef W, SpinorRef y, const double* coefW,
+                                                            const LzRhs* lz, int cap, int nrhs, int Vh, int nb) {
+  extern __shared__ f2 cf[];   // per stored vector: high word, its negative, low word (both lanes)
+  const int rhs = blockIdx.y;
+  const int k = lz[rhs].j;
+  for (int l = threadIdx.x; l < k; l += blockDim.x) {
+    const fac2 c = fac2_bc(coefW[(size_t)rhs * cap + l]);
+    cf[3 * l] = c.h;
+    cf[3 * l + 1] = c.n;
+    cf[3 * l + 2] = c.l;
   }
   __syncthreads();
-  const int s = sb * BX + threadIdx.x;
-  if (s >= V || !in_rhs || k == 0) return;
-  const size_t Vs = (size_t)V;
-  const float4* Wb = reinterpret_cast<const float4*>(W.data) + (size_t)rhs * 12 * Vs + s;
-  float4* yy = reinterpret_cast<float4*>(y.data) + (size_t)rhs * 12 * Vs + s;
-  const size_t slot = (size_t)nrhs * 12 * Vs;
-  for (int q = 0; q < 12; ++q) {
-    const float4 yw = yy[(size_t)q * Vs];
-    cpx<df> acc = cmk(df(yw.x, yw.y), df(yw.z, yw.w));
-    for (int l = 0; l < k; ++l) {
-      const float4 w = __ldg(Wb + (size_t)l * slot + (size_t)q * Vs);
-      const df cl(c[l].x, c[l].y);
-      acc = acc + cmk(cl * df(w.x, w.y), cl * df(w.z, w.w));
+  const int e = blockIdx.x * blockDim.x + threadIdx.x;   // chunk of the field
+  if (e / 768 * 32 + (e & 31) >= Vh || k == 0) return;
+  const size_t at = (size_t)rhs * nb * 768 + e;
+  const size_t slot = (size_t)nrhs * nb * 768;
+  dd2 acc = dfp_ld(y, at);
+  int l = 0;
+  for (; l + 8 <= k; l += 8) {
+    dd2 w[8];
+#pragma unroll
+    for (int u = 0; u < 8; ++u) w[u] = dfp_ldg(W, at + (size_t)(l + u) * slot);
+#pragma unroll
+    for (int u = 0; u < 8; ++u) {
+      const f2* c = cf + 3 * (l + u);
+      acc = dd2_add(acc, dd2_mul({c[0], c[1], c[2]}, w[u]));
     }
-    yy[(size_t)q * Vs] = make_float4(acc.r.hi, acc.r.lo, acc.i.hi, acc.i.lo);
   }
+  for (; l < k; ++l) {
+    const f2* c = cf + 3 * l;
+    acc = dd2_add(acc, dd2_mul({c[0], c[1], c[2]}, dfp_ldg(W, at + (size_t)l * slot)));
+  }
+  dfp_st(y, at, acc);
 }
 
 // Other precisions: whole spinors, accumulated in the compute type of y.
@@ -293,8 +327,8 @@ void launch_lz_combine(int pw, int py, SpinorRef W, SpinorRef y, const double* c
                        int nrhs, int V, cudaStream_t st) {
   Shape sh = make_shape(V, nrhs);
   if (pw == P64E && py == P64E) {
-    const size_t smem = sizeof(float2) * (size_t)sh.by * cap;
-    lz_combine_df_kernel<<<sh.grid(), sh.block(), smem, st>>>(W, y, coefW, lz, cap, nrhs, V, sh.ngr);
+    const size_t smem = 3 * sizeof(f2) * (size_t)cap;   // cap <= 1024: 24 KB
+    lz_combine_df_kernel<<<dim3(df_blocks(V) * 6, nrhs), 128, smem, st>>>(W, y, coefW, lz, cap, nrhs, V / 2, df_blocks(V));
     return;
   }
 #define LZC(A, B) lz_combine_kernel<A, B><<<sh.grid(), sh.block(), 0, st>>>(W, y, coefW, lz, cap, nrhs, V, sh.ngr)

@@ -17,6 +17,7 @@
 // running poles and those frozen by the stopped ones sum to eta ||v||; poles drop
 // from the largest shift down (they converge first). See ms_scalar2_kernel for how
 // the budget is shared.
+#include "dfpair.cuh"
 #include "kernels.h"
 
 namespace ovl {
@@ -52,6 +53,36 @@ __global__ void __launch_bounds__(256) ms_init_kernel(SpinorRef v, SpinorRef r, 
   }
 }
 
+// Double-float: one thread per pair of sites and system.
+constexpr int DP = 32;   // pairs per block: the partial sums keep the 64-site blocks
+template <int PV>
+__global__ void __launch_bounds__(128) ms_init_df_kernel(SpinorRef v, SpinorRef r, SpinorRef pb, SpinorRef y,
+                                                         int npoles, int nrhs, int Vh, int nsb, int ngr,
+                                                         double* partials) {
+  const int sb = blockIdx.x / ngr;
+  const int rhs = (blockIdx.x - sb * ngr) * blockDim.y + threadIdx.y;
+  const int s = sb * DP + threadIdx.x;
+  dot2p d = {0ull, 0ull};
+  if (s < Vh && rhs < nrhs) {
+    for (int k = 0; k < 12; ++k) {
+      dd2 re, im;
+      dfp_load<PV>(v, rhs, k, s, re, im);
+      dfp_store<P64E>(r, rhs, k, s, re, im);
+      dfp_store<P64E>(y, rhs, k, s, dd2_zero(), dd2_zero());
+      for (int i = 0; i < npoles; ++i) dfp_store<P64E>(pb, i * nrhs + rhs, k, s, re, im);
+      dot2p_add(d, re, re);
+      dot2p_add(d, im, im);
+    }
+  }
+  double t = dot2p_get(d);
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) t += __shfl_down_sync(0xffffffffu, t, o);
+  if (threadIdx.x == 0 && rhs < nrhs) {
+    partials[((size_t)rhs * nsb + sb) * NVRED + 0] = t;
+    partials[((size_t)rhs * nsb + sb) * NVRED + 1] = 0.0;
+  }
+}
+
 void launch_ms_init(int pv, int pr, int pp, SpinorRef v, SpinorRef r, SpinorRef pb, SpinorRef y, int npoles,
                     int nrhs, int V, double* partials, cudaStream_t st) {
   Shape sh = make_shape(V, nrhs);
@@ -62,8 +93,11 @@ void launch_ms_init(int pv, int pr, int pp, SpinorRef v, SpinorRef r, SpinorRef 
   else if (pv == P32 && pr == P32 && pp == P16) MS_INIT(P32, P32, P16);
   else if (pv == P64 && pr == P32 && pp == P16) MS_INIT(P64, P32, P16);
   else if (pv == P32 && pr == P64 && pp == P64) MS_INIT(P32, P64, P64);
-  else if (pv == P64 && pr == P64E && pp == P64E) MS_INIT(P64, P64E, P64E);
-  else if (pv == P32 && pr == P64E && pp == P64E) MS_INIT(P32, P64E, P64E);
+  else if (pr == P64E && pp == P64E && (pv == P64 || pv == P32)) {
+    const dim3 block(DP, sh.by), grid(sh.grid());
+    if (pv == P64) ms_init_df_kernel<P64><<<grid, block, 0, st>>>(v, r, pb, y, npoles, nrhs, V / 2, sh.nsb, sh.ngr, partials);
+    else ms_init_df_kernel<P32><<<grid, block, 0, st>>>(v, r, pb, y, npoles, nrhs, V / 2, sh.nsb, sh.ngr, partials);
+  }
   else note_bad_combo("ms_init");
 #undef MS_INIT
 }
@@ -275,67 +309,50 @@ __global__ void __launch_bounds__(256) ms_update_kernel(SpinorRef r, SpinorRef p
   store_spinor_as<PR, T>(y, rhs, s, yv);
 }
 
-// Double-float form of the same pass, chunk-major: for each 16-byte chunk (one complex
-// component) of r and y, every active pole's chunk is read, y accumulated and the pole
-// rewritten. Holding one component instead of whole spinors keeps the thread small
+// Double-float form of the same pass: one thread per 16-byte chunk (one real number of a pair
+// of sites) of r and y; every active pole's chunk is read, y accumulated and the pole
+// rewritten. Holding one number instead of whole spinors keeps the thread small
 // (the spinor-at-a-time form needs ~250 registers: 8 warps per SM, 78% of the copy
-// bandwidth), and the pole coefficients are converted to double-float once per block
-// into shared memory instead of per thread and pole.
-__global__ void __launch_bounds__(256) ms_update_df_kernel(SpinorRef r, SpinorRef pb, SpinorRef y, int nrhs, int V,
-                                                           int ngr, const MsRhs* ms) {
-  __shared__ float2 cf[4][NPMAX][3];   // (y, r, p) coefficients of the block's systems
-  const int sb = blockIdx.x / ngr;
-  const int rg = blockIdx.x - sb * ngr;
-  const int rhs = rg * blockDim.y + threadIdx.y;
-  const bool in_rhs = rhs < nrhs;
-  const int ny = in_rhs ? ms[rhs].nact_y : 0;
-  if (in_rhs) {
-    const MsRhs& m = ms[rhs];
-    for (int i = threadIdx.x; i < ny; i += blockDim.x) {
-      const double c3[3] = {m.coef_y[i], m.coef_r[i], m.coef_p[i]};
-#pragma unroll
-      for (int k = 0; k < 3; ++k) {
-        const float h = (float)c3[k];
-        cf[threadIdx.y][i][k] = make_float2(h, (float)(c3[k] - (double)h));
-      }
-    }
+// bandwidth), the chunk as a grid dimension keeps a small lattice from running 24 chunks in
+// series, and the pole coefficients are converted to double-float once per block into
+// shared memory instead of per thread and pole.
+__global__ void __launch_bounds__(128) ms_update_df_kernel(SpinorRef r, SpinorRef pb, SpinorRef y, int nrhs, int Vh, int nb,
+                                                           const MsRhs* ms) {
+  __shared__ f2 cf[NPMAX][9];   // (y, r, p) coefficients: high word, its negative, low word
+  const int rhs = blockIdx.y;
+  const MsRhs& m = ms[rhs];
+  const int ny = m.nact_y;
+  for (int e = threadIdx.x; e < 3 * ny; e += blockDim.x) {
+    const int i = e / 3, k = e - 3 * i;
+    const fac2 c = fac2_bc(k == 0 ? m.coef_y[i] : k == 1 ? m.coef_r[i] : m.coef_p[i]);
+    cf[i][3 * k] = c.h;
+    cf[i][3 * k + 1] = c.n;
+    cf[i][3 * k + 2] = c.l;
   }
   __syncthreads();
-  const int s = sb * BX + threadIdx.x;
-  if (s >= V || !in_rhs || ny == 0) return;
-  const int na = ms[rhs].active;
-  const size_t Vs = (size_t)V;
-  const float4* rr = reinterpret_cast<const float4*>(r.data) + (size_t)rhs * 12 * Vs + s;
-  float4* yy = reinterpret_cast<float4*>(y.data) + (size_t)rhs * 12 * Vs + s;
-  float4* pp = reinterpret_cast<float4*>(pb.data) + (size_t)rhs * 12 * Vs + s;
-  const size_t pole_stride = (size_t)nrhs * 12 * Vs;
-  const float2(*c)[3] = cf[threadIdx.y];
-  for (int k = 0; k < 12; ++k) {
-    const float4 rw = rr[(size_t)k * Vs];
-    const cpx<df> rc = cmk(df(rw.x, rw.y), df(rw.z, rw.w));
-    const float4 yw = yy[(size_t)k * Vs];
-    cpx<df> yc = cmk(df(yw.x, yw.y), df(yw.z, yw.w));
-    for (int i = 0; i < ny; ++i) {
-      float4* pi = pp + (size_t)i * pole_stride + (size_t)k * Vs;
-      const float4 pw = *pi;
-      cpx<df> pc = cmk(df(pw.x, pw.y), df(pw.z, pw.w));
-      const df cy(c[i][0].x, c[i][0].y);
-      yc = yc + cy * pc;
-      if (i < na) {
-        const df cr(c[i][1].x, c[i][1].y), cp(c[i][2].x, c[i][2].y);
-        pc = cr * rc + cp * pc;
-        *pi = make_float4(pc.r.hi, pc.r.lo, pc.i.hi, pc.i.lo);
-      }
-    }
-    yy[(size_t)k * Vs] = make_float4(yc.r.hi, yc.r.lo, yc.i.hi, yc.i.lo);
+  const int e = blockIdx.x * blockDim.x + threadIdx.x;   // chunk of the field
+  if (e / 768 * 32 + (e & 31) >= Vh || ny == 0) return;
+  const int na = m.active;
+  const size_t at = (size_t)rhs * nb * 768 + e;
+  const size_t pole_stride = (size_t)nrhs * nb * 768;
+  const dd2 rc = dfp_ld(r, at);
+  dd2 yc = dfp_ld(y, at);
+  for (int i = 0; i < ny; ++i) {
+    const f2* c = cf[i];
+    const dd2 pc = dfp_ld(pb, at + (size_t)i * pole_stride);
+    yc = dd2_add(yc, dd2_mul({c[0], c[1], c[2]}, pc));
+    if (i < na)
+      dfp_st(pb, at + (size_t)i * pole_stride,
+             dd2_add(dd2_mul({c[3], c[4], c[5]}, rc), dd2_mul({c[6], c[7], c[8]}, pc)));
   }
+  dfp_st(y, at, yc);
 }
 
 void launch_ms_update(int pr, int pp, SpinorRef r, SpinorRef pb, SpinorRef y, int npoles, int nrhs, int V,
                       const MsRhs* ms, cudaStream_t st) {
   Shape sh = make_shape(V, nrhs);
   if (pr == P64E && pp == P64E) {
-    ms_update_df_kernel<<<sh.grid(), sh.block(), 0, st>>>(r, pb, y, nrhs, V, sh.ngr, ms);
+    ms_update_df_kernel<<<dim3(df_blocks(V) * 6, nrhs), 128, 0, st>>>(r, pb, y, nrhs, V / 2, df_blocks(V), ms);
     return;
   }
   if (pr == P64 && pp == P64) ms_update_kernel<P64, P64><<<sh.grid(), sh.block(), 0, st>>>(r, pb, y, npoles, nrhs, V, sh.ngr, ms);

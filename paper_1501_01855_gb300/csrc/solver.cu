@@ -79,7 +79,7 @@ ovl_status axpby_batch(ovl_ctx* c, const std::vector<cd>& a, const Field& x, int
 
 ovl_status copy_convert(ovl_ctx* c, const Field& in, int ioff, Field& out, int ooff, int n) {
   if (in.prec == out.prec) {
-    const size_t per = (size_t)c->V * spinor_site_bytes(in.prec);
+    const size_t per = field_bytes(in.prec, c->V);
     OVL_CUDA(c, cudaMemcpyAsync((char*)out.data + per * ooff, (char*)in.data + per * ioff, per * n,
                                 cudaMemcpyDeviceToDevice, c->st));
     if (in.prec == P16)

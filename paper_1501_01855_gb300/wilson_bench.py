@@ -7,8 +7,8 @@ Unit links, a random input spinor, the kernel launched `--iters` times back to b
 the context stream and timed with CUDA events. Prints milliseconds per launch, the
 algorithmic bytes of one launch (each input spinor read once, each output written once,
 the links read once) and the rate they imply. `--variant` forces a kernel shape (0 one
-thread per site, 1 direction split, 2 4D tiles, 3 lane pairs for double-float); the
-default lets the create-time autotuner choose.
+thread per site, 1 direction split, 2 4D tiles; double-float: 0, 3, 2, 1 for 1, 2, 4, 8
+thread groups per pair of sites); the default lets the library choose.
 """
 import argparse
 
