@@ -86,6 +86,12 @@ __device__ __forceinline__ df operator*(df a, df b) {
 }
 __device__ __forceinline__ bool operator!=(df a, df b) { return a.hi != b.hi || a.lo != b.lo; }
 
+// x = hi + lo (x), both rounded to nearest
+__host__ __device__ __forceinline__ float2 split_df(double x) {
+  const float h = (float)x;
+  return make_float2(h, (float)(x - (double)h));
+}
+
 // ------------------------------------------------------------------ complex
 template <typename T>
 struct cpx {
@@ -279,11 +285,6 @@ __device__ __forceinline__ void store_spinor(const SpinorRef& f, int rhs, int s,
 template <int P, typename T>
 __device__ __forceinline__ void load_spinor_as(const SpinorRef& f, int rhs, int s, cpx<T> v[12]) {
   load_spinor_gen<P, T, false>(f, rhs, s, v);
-}
-// read-only path: only for fields that the kernel does not write (Wilson-kernel input)
-template <int P, typename T>
-__device__ __forceinline__ void load_spinor_as_ro(const SpinorRef& f, int rhs, int s, cpx<T> v[12]) {
-  load_spinor_gen<P, T, true>(f, rhs, s, v);
 }
 template <int P, typename T>
 __device__ __forceinline__ void store_spinor_as(const SpinorRef& f, int rhs, int s, const cpx<T> v[12]) {

@@ -106,6 +106,7 @@ struct fac2 {
 };
 __device__ __forceinline__ fac2 fac2_of(dd2 v) { return {v.h, neg2(v.h), v.l}; }
 __device__ __forceinline__ fac2 fac2_bc(double x) { return fac2_of(dd2_bc(x)); }
+__device__ __forceinline__ fac2 fac2_minus(float2 f) { return {bc(-f.x), bc(f.x), bc(-f.y)}; }   // -(f.x + f.y)
 __device__ __forceinline__ dd2 dd2_mul(fac2 a, dd2 b) {
   const f2 p = prod2(a.h, b.h);
   f2 e = fma2(a.h, b.h, prod2(a.n, b.h));   // the exact rounding error of p

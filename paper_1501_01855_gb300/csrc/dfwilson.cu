@@ -30,14 +30,10 @@ namespace ovl {
 
 namespace {
 
-constexpr int DP = 32;   // pairs of sites per block (64 sites: the partial sums keep the BX layout)
-
-// threads of a block (64 per group) and the resident blocks per SM its registers are capped for
-constexpr int df_threads(int G) { return 64 * G; }
-constexpr int df_resident(int G) { return G == 1 ? 6 : G == 2 ? 3 : G == 4 ? 2 : 1; }
-
-// partial sums each mode produces
-constexpr int df_nred(int mode) { return mode == MODE_OVL ? 4 : mode == MODE_K ? 2 : 1; }
+// P pairs of sites per block: 32 (64 sites: the partial sums keep the BX layout), or 8 for eight
+// groups on the smallest launches, which would otherwise leave most SMs without a block.
+// Resident blocks per SM that the registers are capped for:
+constexpr int df_resident(int G, int P) { return G == 1 ? 6 : G == 2 || P == 8 ? 3 : G == 4 ? 2 : 1; }
 
 __device__ __forceinline__ void prefetch_l1(const void* p) { asm volatile("prefetch.global.L1 [%0];" ::"l"(p)); }
 
@@ -102,7 +98,7 @@ __device__ __forceinline__ Oper load_oper(const ulonglong2* b, int half, const H
   const ulonglong2* p = b + half * 192;
   const ulonglong2* q0 = b + h.other * 192 + (h.a & 1) * 32;
   const ulonglong2* q1 = b + h.other * 192 + 32 - (h.a & 1) * 32;
-  return {__ldg(p + 64 * c), __ldg(p + 64 * c + 32), __ldg(q0 + 64 * c), __ldg(q1 + 64 * c)};
+  return {p[64 * c], p[64 * c + 32], q0[64 * c], q1[64 * c]};
 }
 __device__ __forceinline__ float sgn_re(int k) { return k == 1 || k == 2 ? -1.f : 1.f; }
 __device__ __forceinline__ float sgn_im(int k) { return k >= 2 ? -1.f : 1.f; }
@@ -172,7 +168,7 @@ __device__ __forceinline__ void df_epilogue(const DArgs& a, const DfScal& k, int
   for (int c = 0; c < N; ++c)
 #pragma unroll
     for (int r = 0; r < 2; ++r) {
-      o[c][r] = dfp_ldg(a.in, dfp_at(fin, kc + c, r, i, nb));
+      o[c][r] = dfp_ld(a.in, dfp_at(fin, kc + c, r, i, nb));
       if constexpr (MODE == MODE_R) {
         w[c][r] = dfp_ld(a.aux1, dfp_at(rhs, kc + c, r, i, nb));
         y[c][r] = dfp_ld(a.aux2, dfp_at(rhs, kc + c, r, i, nb));
@@ -233,23 +229,31 @@ __device__ __forceinline__ void df_epilogue(const DArgs& a, const DfScal& k, int
 
 // G groups of threads (threadIdx.z) share the eight hops of a pair, 8 / G each; their sums
 // meet in shared memory, where group z finishes the components z, z + G, .. of the spinor.
-template <int MODE, int PIO, int G>
-__global__ void __launch_bounds__(df_threads(G), df_resident(G)) df_wilson_kernel(const DArgs a) {
-  constexpr int NR = df_nred(MODE);
+template <int MODE, int PIO, int G, int P>
+__global__ void __launch_bounds__(2 * P * G, df_resident(G, P)) df_wilson_kernel(const DArgs a) {
+  constexpr int NR = nred(MODE);
   extern __shared__ ulonglong2 part[];   // G > 1: [z][component (6 x re, im)][thread x]
-  __shared__ double red[2 * G][NR];
+  constexpr int NW = 2 * P * G / 32;   // warps
+  __shared__ float2 red[NW][NR];
   const int half = threadIdx.x & 1;
   const int grp = G > 1 ? threadIdx.z : 0;
   const int sb = blockIdx.x / a.nrhs;   // the systems of one site block together: they share its links in L1 / L2
   const int rhs = blockIdx.x - sb * a.nrhs;
   const int Vh = a.g.V >> 1;
-  const int i = sb * DP + (threadIdx.x >> 1);
+  const int i = sb * P + (threadIdx.x >> 1);
   bool live = i < Vh;
+  const int m = (threadIdx.x >> 1 & 7) + 8 * half;   // this lane's share of the prefetches
+  const int n0 = grp * (8 / G), n1 = n0 + 8 / G;
+  if (live) prefetch_link(link_at(a.links, i, n0), m);
+  if constexpr (!kReadOnly<MODE>) {
+    pdl_wait();
+    pdl_release();
+  }
   if (live && a.ms != nullptr && (MODE == MODE_K || MODE == MODE_R)) live = !a.ms[rhs].done;
   int fin = rhs, j = 0;   // field index of the hop input (the basis slot in MODE_LZK)
   if constexpr (MODE == MODE_LZK || MODE == MODE_LZL) {
-    if (live) live = !a.lz[rhs].done;
-    if (live) j = a.lz[rhs].j;
+    if (a.lz[rhs].done) return;   // every thread of the block
+    j = a.lz[rhs].j;
     if (MODE == MODE_LZK) fin = j * a.nrhs + rhs;
   }
   dd2 up[3][2], low[3][2];
@@ -262,14 +266,11 @@ __global__ void __launch_bounds__(df_threads(G), df_resident(G)) df_wilson_kerne
     const size_t fblk = (size_t)fin * df_blocks(a.g.V);
     int x[4] = {0, 0, 0, 0};
     if (live) site_coords(a.g, i, x);
-    const int n0 = grp * (8 / G), n1 = n0 + 8 / G;
-    const int m = (threadIdx.x >> 1 & 7) + 8 * half;
     Hop h = hop_of(a.g, lth, x, i, half, n0);
     const ulonglong2* b = pair_at(a.in, fblk, h.nbr);
     const ulonglong2* u = link_at(a.links, i, n0);
     if (live) {
       prefetch_spinor(b, m);
-      prefetch_link(u, m);
       if constexpr (MODE == MODE_LZL) {   // the basis vectors of the epilogue come from HBM
         prefetch_l2_spinor(pair_at(a.aux1, (size_t)(j * a.nrhs + rhs) * df_blocks(a.g.V), i), m);
         if (j > 0) prefetch_l2_spinor(pair_at(a.aux1, (size_t)((j - 1) * a.nrhs + rhs) * df_blocks(a.g.V), i), m);
@@ -289,7 +290,8 @@ __global__ void __launch_bounds__(df_threads(G), df_resident(G)) df_wilson_kerne
         u = un;
       }
       // the lower spins of mu <= 1 belong to the other lane: exchanged after the last of them
-      // (every lane of the warp takes part; the hops of a warp are the same)
+      // (every lane of the warp takes part: the hops of a warp are the same, or with P = 8 the
+      // two hops of one direction)
       if (n == min(n1 - 1, 3)) {
 #pragma unroll
         for (int c = 0; c < 3; ++c)
@@ -306,12 +308,13 @@ __global__ void __launch_bounds__(df_threads(G), df_resident(G)) df_wilson_kerne
   for (int k = 0; k < 4; ++k) d[k] = {0ull, 0ull};
   DfScal k;
   if (live) {
-    k.kap = fac2_bc(-a.kappa);
+    k.kap = fac2_minus(make_float2(a.kap_h, a.kap_l));
     if constexpr (MODE == MODE_LZK) {
-      k.s0 = fac2_bc(a.lz[rhs].inv_n);
+      const float2 f = a.lz[rhs].fn;
+      k.s0 = {bc(f.x), bc(-f.x), bc(f.y)};
     } else if constexpr (MODE == MODE_LZL) {
-      k.s0 = fac2_bc(-a.lz[rhs].a);
-      k.s1 = fac2_bc(-a.lz[rhs].b);
+      k.s0 = fac2_minus(a.lz[rhs].fa);
+      k.s1 = fac2_minus(a.lz[rhs].fb);
     } else if constexpr (MODE == MODE_R) {
       k.s0 = fac2_bc(a.sigma0);
       k.s1 = fac2_bc(-a.ms[rhs].alpha);
@@ -326,25 +329,26 @@ __global__ void __launch_bounds__(df_threads(G), df_resident(G)) df_wilson_kerne
       df_epilogue<MODE, PIO, 3>(a, k, rhs, fin, j, 6 + 3 * half, i, low, d);
     }
   } else {
-    ulonglong2* mine = part + grp * 12 * 64 + threadIdx.x;
+    constexpr int X = 2 * P;
+    ulonglong2* mine = part + grp * 12 * X + threadIdx.x;
 #pragma unroll
     for (int c = 0; c < 3; ++c)
 #pragma unroll
       for (int r = 0; r < 2; ++r) {
-        mine[(2 * c + r) * 64] = make_ulonglong2(up[c][r].h, up[c][r].l);
-        mine[(6 + 2 * c + r) * 64] = make_ulonglong2(low[c][r].h, low[c][r].l);
+        mine[(2 * c + r) * X] = make_ulonglong2(up[c][r].h, up[c][r].l);
+        mine[(6 + 2 * c + r) * X] = make_ulonglong2(low[c][r].h, low[c][r].l);
       }
     __syncthreads();
     if (live) {
       for (int q = grp; q < 6; q += G) {
-        const ulonglong2* s = part + 2 * q * 64 + threadIdx.x;
+        const ulonglong2* s = part + 2 * q * X + threadIdx.x;
         dd2 t[1][2];
 #pragma unroll
         for (int r = 0; r < 2; ++r) {
-          t[0][r] = {s[r * 64].x, s[r * 64].y};
+          t[0][r] = {s[r * X].x, s[r * X].y};
 #pragma unroll
           for (int z = 1; z < G; ++z) {
-            const ulonglong2 w = s[(z * 12 + r) * 64];
+            const ulonglong2 w = s[(z * 12 + r) * X];
             t[0][r] = dd2_add(t[0][r], {w.x, w.y});
           }
         }
@@ -353,39 +357,40 @@ __global__ void __launch_bounds__(df_threads(G), df_resident(G)) df_wilson_kerne
     }
   }
   if (a.partials != nullptr) {
-    // warps in the order x, z: fixed, so that the sum is
-    const int warp = threadIdx.z * 2 + (threadIdx.x >> 5);
+    // lanes in double-float, a fixed tree; then FP64 over the warps in the order z, x
+    const int lin = threadIdx.z * 2 * P + threadIdx.x;
 #pragma unroll
     for (int q = 0; q < NR; ++q) {
-      double v = dot2p_get(d[q]);
+      float s0, s1, c0, c1;
+      upk(d[q].s, s0, s1);
+      upk(d[q].c, c0, c1);
+      df v = df(s0, c0) + df(s1, c1);
 #pragma unroll
-      for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
-      if ((threadIdx.x & 31) == 0) red[warp][q] = v;
+      for (int o = 16; o > 0; o >>= 1)
+        v = v + df(__shfl_down_sync(0xffffffffu, v.hi, o), __shfl_down_sync(0xffffffffu, v.lo, o));
+      if ((lin & 31) == 0) red[lin >> 5][q] = make_float2(v.hi, v.lo);
     }
     __syncthreads();
     if (threadIdx.x == 0 && threadIdx.z == 0) {
-      double* out = a.partials + ((size_t)rhs * a.nsb + sb) * NVRED;
+      double tot[NVRED] = {0.0, 0.0, 0.0, 0.0};
 #pragma unroll
-      for (int q = 0; q < NR; ++q) {
-        double t = 0.0;
-        for (int z = 0; z < G; ++z) t += red[2 * z][q] + red[2 * z + 1][q];
-        out[q] = t;
-      }
-#pragma unroll
-      for (int q = NR; q < NVRED; ++q) out[q] = 0.0;
+      for (int q = 0; q < NR; ++q)
+        for (int w = 0; w < NW; ++w) tot[q] += (double)red[w][q].x + (double)red[w][q].y;
+      store_partials<MODE>(a, rhs, sb, tot);
     }
   }
   if constexpr (MODE == MODE_LZK || MODE == MODE_LZL) {
-    if (a.lzc.ctr != nullptr) lz_arrive<MODE>(a, rhs, a.nsb);
+    if (threadIdx.z * 2 * P + threadIdx.x < 32) lz_arrive<MODE>(a, rhs, a.nsb);
   }
 }
 
-template <int MODE, int PIO, int G>
+template <int MODE, int PIO, int G, int P = 32>
 void run_g(DArgs a, cudaStream_t st) {
-  const size_t smem = G == 1 ? 0 : sizeof(ulonglong2) * 64 * 12 * G;
+  a.nsb = ((a.g.V >> 1) + P - 1) / P;
+  const size_t smem = G == 1 ? 0 : sizeof(ulonglong2) * 2 * P * 12 * G;
   if (smem > 40 * 1024)   // with the static arrays, past the 48 KB that need no opt-in
-    cudaFuncSetAttribute(df_wilson_kernel<MODE, PIO, G>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  df_wilson_kernel<MODE, PIO, G><<<dim3((unsigned)(a.nsb * a.nrhs)), dim3(64, 1, G), smem, st>>>(a);
+    cudaFuncSetAttribute(df_wilson_kernel<MODE, PIO, G, P>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  launch_step(df_wilson_kernel<MODE, PIO, G, P>, dim3((unsigned)(a.nsb * a.nrhs)), dim3(2 * P, 1, G), smem, st, a);
 }
 
 template <int MODE, int PIO>
@@ -394,7 +399,15 @@ void run_m(const DArgs& a, cudaStream_t st) {
     case 0: run_g<MODE, PIO, 1>(a, st); break;
     case 3: run_g<MODE, PIO, 2>(a, st); break;
     case 2: run_g<MODE, PIO, 4>(a, st); break;
-    default: run_g<MODE, PIO, 8>(a, st); break;
+    default:
+      // small blocks where the caller does not read partial sums per 64 sites
+      if constexpr (MODE == MODE_LZK || MODE == MODE_LZL || MODE == MODE_K) {
+        if ((long long)a.g.V * a.nrhs <= 4864 && (MODE != MODE_K || a.partials == nullptr)) {
+          run_g<MODE, PIO, 8, 8>(a, st);
+          break;
+        }
+      }
+      run_g<MODE, PIO, 8>(a, st);
   }
 }
 
@@ -412,7 +425,6 @@ int wilson_df_variant(int V, int nrhs) {
 }
 
 void run_wilson_df(int mode, int pio, DArgs a, cudaStream_t st) {
-  a.nsb = make_shape(a.g.V, a.nrhs).nsb;
   if (mode == MODE_K) run_m<MODE_K, P64E>(a, st);
   else if (mode == MODE_R) run_m<MODE_R, P64E>(a, st);
   else if (mode == MODE_LZK) run_m<MODE_LZK, P64E>(a, st);

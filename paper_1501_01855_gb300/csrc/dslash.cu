@@ -128,7 +128,7 @@ __device__ __forceinline__ void acc_norm(Acc<T>& a, const cpx<T>& z) {
   a.add(z.i, z.i);
 }
 
-template <int MU, int PIN, int PL, typename T>
+template <int MU, int PIN, int PL, bool RO, typename T>
 __device__ __forceinline__ void hop_dir(const Geom& g, const LinkRef& L, const SpinorRef& in, int rhs, int s,
                                         const int x[4], int stride, cpx<T> acc[12]) {
   cpx<T> psi[12], h[6], w[6], u[9];
@@ -136,7 +136,7 @@ __device__ __forceinline__ void hop_dir(const Geom& g, const LinkRef& L, const S
   {
     const bool wrap = x[MU] == g.L[MU] - 1;
     const int sf = wrap ? s - (g.L[MU] - 1) * stride : s + stride;
-    load_spinor_as_ro<PIN, T>(in, rhs, sf, psi);
+    load_spinor_gen<PIN, T, RO>(in, rhs, sf, psi);
     project<MU, -1>(psi, h);
     if (MU == 3 && g.bc_t && wrap) {
 #pragma unroll
@@ -150,7 +150,7 @@ __device__ __forceinline__ void hop_dir(const Geom& g, const LinkRef& L, const S
   {
     const bool wrap = x[MU] == 0;
     const int sb = wrap ? s + (g.L[MU] - 1) * stride : s - stride;
-    load_spinor_as_ro<PIN, T>(in, rhs, sb, psi);
+    load_spinor_gen<PIN, T, RO>(in, rhs, sb, psi);
     project<MU, +1>(psi, h);
     if (MU == 3 && g.bc_t && wrap) {
 #pragma unroll
@@ -162,16 +162,16 @@ __device__ __forceinline__ void hop_dir(const Geom& g, const LinkRef& L, const S
   }
 }
 
-template <int PIN, int PL, typename T>
+template <int PIN, int PL, bool RO, typename T>
 __device__ __forceinline__ void hop(const Geom& g, const LinkRef& L, const SpinorRef& in, int rhs, int s,
                                     const int x[4], cpx<T> acc[12]) {
 #pragma unroll
   for (int k = 0; k < 12; ++k) acc[k] = cmk(T(0), T(0));
   const int sy = g.L[0], sz = g.L[0] * g.L[1], st = sz * g.L[2];
-  hop_dir<0, PIN, PL, T>(g, L, in, rhs, s, x, 1, acc);
-  hop_dir<1, PIN, PL, T>(g, L, in, rhs, s, x, sy, acc);
-  hop_dir<2, PIN, PL, T>(g, L, in, rhs, s, x, sz, acc);
-  hop_dir<3, PIN, PL, T>(g, L, in, rhs, s, x, st, acc);
+  hop_dir<0, PIN, PL, RO, T>(g, L, in, rhs, s, x, 1, acc);
+  hop_dir<1, PIN, PL, RO, T>(g, L, in, rhs, s, x, sy, acc);
+  hop_dir<2, PIN, PL, RO, T>(g, L, in, rhs, s, x, sz, acc);
+  hop_dir<3, PIN, PL, RO, T>(g, L, in, rhs, s, x, st, acc);
 }
 
 // Epilogue shared by both kernel variants: acc holds the hop sum of site s; v gets this
@@ -180,12 +180,16 @@ template <int MODE, int PIN, int POUT, int PA1, int PA2, typename T>
 __device__ __forceinline__ void wilson_epilogue(const DArgs& a, int rhs, int fin, int s, cpx<T> acc[12],
                                                 typename RedT<T>::type v[NVRED]) {
   cpx<T> c[12];
-  load_spinor_as_ro<PIN, T>(a.in, fin, s, c);
-  const T kap = (T)a.kappa;
+  load_spinor_gen<PIN, T, kReadOnly<MODE>>(a.in, fin, s, c);
+  T kap;   // the compute type's copies of the coefficients (conversions from FP64 are slow)
+  if constexpr (std::is_same<T, float>::value) kap = a.kap_h;
+  else kap = a.kappa;
   const bool red = a.partials != nullptr;
   if constexpr (MODE == MODE_LZK) {
     // t = (1 / n_j) gamma5 (W_j - kappa hop W_j)
-    const T sc = (T)a.lz[rhs].inv_n;
+    T sc;
+    if constexpr (std::is_same<T, float>::value) sc = a.lz[rhs].fn.x;
+    else sc = a.lz[rhs].inv_n;
 #pragma unroll
     for (int k = 0; k < 12; ++k) {
       cpx<T> o = c[k] - kap * acc[k];
@@ -203,7 +207,14 @@ __device__ __forceinline__ void wilson_epilogue(const DArgs& a, int rhs, int fin
     // W_{j+1} = gamma5 (t - kappa hop t) - a W_j - b W_{j-1}
     const LzRhs& L = a.lz[rhs];
     const int j = L.j;
-    const T ca = (T)L.a, cb = (T)L.b;
+    T ca, cb;
+    if constexpr (std::is_same<T, float>::value) {
+      ca = L.fa.x;
+      cb = L.fb.x;
+    } else {
+      ca = L.a;
+      cb = L.b;
+    }
     cpx<T> w[12];
     load_spinor_as<PA1, T>(a.aux1, j * a.nrhs + rhs, s, w);
 #pragma unroll
@@ -344,34 +355,41 @@ __global__ void __launch_bounds__(256) __maxnreg__((MaxReg<PL, PIN>::v)) wilson_
     live = (s < a.g.V) && (rhs < a.nrhs);
     if (live) site_coords(a.g, s, x);
   }
+  if constexpr (!kReadOnly<MODE>) {
+    pdl_wait();
+    pdl_release();
+  }
   if (live && a.ms != nullptr && (MODE == MODE_K || MODE == MODE_R)) live = !a.ms[rhs].done;
   int fin = rhs;   // field index of the hop input (the basis slot in MODE_LZK)
+  bool act = false;
   if constexpr (MODE == MODE_LZK || MODE == MODE_LZL) {
-    if (live) live = !a.lz[rhs].done;
+    act = rhs < a.nrhs && !a.lz[rhs].done;
+    // a block whose systems are all done leaves at once: launches past the end of a sign cost
+    // little more than their dispatch
+    if (blockDim.y == 1 ? !act : !__syncthreads_or(act)) return;
+    live = live && act;
     if (MODE == MODE_LZK && live) fin = a.lz[rhs].j * a.nrhs + rhs;
   }
   using R = typename RedT<T>::type;
   R v[NVRED] = {R(0), R(0), R(0), R(0)};
   if (live) {
     cpx<T> acc[12];
-    hop<PIN, PL, T>(a.g, a.links, a.in, fin, s, x, acc);
+    hop<PIN, PL, kReadOnly<MODE>, T>(a.g, a.links, a.in, fin, s, x, acc);
     wilson_epilogue<MODE, PIN, POUT, PA1, PA2, T>(a, rhs, fin, s, acc, v);
   }
   if (a.partials != nullptr) {
     double tot[NVRED];
-    block_reduce_partials<R>(v, red, tot);
+    block_reduce_partials<R, nred(MODE)>(v, red, tot);
     if (threadIdx.x == 0 && rhs < a.nrhs) {
-#pragma unroll
-      for (int j = 0; j < NVRED; ++j) a.partials[((size_t)rhs * a.nsb + sb) * NVRED + j] = tot[j];
+      store_partials<MODE>(a, rhs, sb, tot);
       if constexpr (TILED) {
-        for (int q = 1; q < TX * TY * TZ * TT / BX; ++q)
-#pragma unroll
-          for (int j = 0; j < NVRED; ++j) a.partials[((size_t)rhs * a.nsb + sb + q) * NVRED + j] = 0.0;
+        const double zero[NVRED] = {0.0, 0.0, 0.0, 0.0};
+        for (int q = 1; q < TX * TY * TZ * TT / BX; ++q) store_partials<MODE>(a, rhs, sb + q, zero);
       }
     }
   }
   if constexpr (MODE == MODE_LZK || MODE == MODE_LZL) {
-    if (a.lzc.ctr != nullptr) lz_arrive<MODE>(a, rhs, TILED ? (int)gridDim.x : a.nsb);
+    if (threadIdx.x < 32 && act) lz_arrive<MODE>(a, rhs, TILED ? (int)gridDim.x : a.nsb);
   }
 }
 
@@ -397,11 +415,15 @@ __global__ void __launch_bounds__(4 * BX) __maxnreg__((MaxReg<PL, PIN>::v)) wils
   const int sl = grp * 32 + lane;
   const int s = sb * BX + sl;
   bool live = s < a.g.V;
+  if constexpr (!kReadOnly<MODE>) {
+    pdl_wait();
+    pdl_release();
+  }
   if (live && a.ms != nullptr && (MODE == MODE_K || MODE == MODE_R)) live = !a.ms[rhs].done;
   int fin = rhs;
   if constexpr (MODE == MODE_LZK || MODE == MODE_LZL) {
-    if (live) live = !a.lz[rhs].done;
-    if (MODE == MODE_LZK && live) fin = a.lz[rhs].j * a.nrhs + rhs;
+    if (a.lz[rhs].done) return;   // every thread of the block
+    if (MODE == MODE_LZK) fin = a.lz[rhs].j * a.nrhs + rhs;
   }
   cpx<T> acc[12];
 #pragma unroll
@@ -410,10 +432,10 @@ __global__ void __launch_bounds__(4 * BX) __maxnreg__((MaxReg<PL, PIN>::v)) wils
     int x[4];
     site_coords(a.g, s, x);
     const int sy = a.g.L[0], sz = sy * a.g.L[1], st = sz * a.g.L[2];
-    if (dir == 0) hop_dir<0, PIN, PL, T>(a.g, a.links, a.in, fin, s, x, 1, acc);
-    else if (dir == 1) hop_dir<1, PIN, PL, T>(a.g, a.links, a.in, fin, s, x, sy, acc);
-    else if (dir == 2) hop_dir<2, PIN, PL, T>(a.g, a.links, a.in, fin, s, x, sz, acc);
-    else hop_dir<3, PIN, PL, T>(a.g, a.links, a.in, fin, s, x, st, acc);
+    if (dir == 0) hop_dir<0, PIN, PL, kReadOnly<MODE>, T>(a.g, a.links, a.in, fin, s, x, 1, acc);
+    else if (dir == 1) hop_dir<1, PIN, PL, kReadOnly<MODE>, T>(a.g, a.links, a.in, fin, s, x, sy, acc);
+    else if (dir == 2) hop_dir<2, PIN, PL, kReadOnly<MODE>, T>(a.g, a.links, a.in, fin, s, x, sz, acc);
+    else hop_dir<3, PIN, PL, kReadOnly<MODE>, T>(a.g, a.links, a.in, fin, s, x, st, acc);
   }
   if (dir != 0) {
 #pragma unroll
@@ -429,14 +451,13 @@ __global__ void __launch_bounds__(4 * BX) __maxnreg__((MaxReg<PL, PIN>::v)) wils
   }
   if (a.partials != nullptr) {
     double tot[NVRED];
-    block_reduce_partials<R>(v, red, tot);
+    block_reduce_partials<R, nred(MODE)>(v, red, tot);
     if (threadIdx.x == 0) {
-#pragma unroll
-      for (int j = 0; j < NVRED; ++j) a.partials[((size_t)rhs * a.nsb + sb) * NVRED + j] = tot[j];
+      store_partials<MODE>(a, rhs, sb, tot);
     }
   }
   if constexpr (MODE == MODE_LZK || MODE == MODE_LZL) {
-    if (a.lzc.ctr != nullptr) lz_arrive<MODE>(a, rhs, a.nsb);
+    if (threadIdx.x < 32) lz_arrive<MODE>(a, rhs, a.nsb);
   }
 }
 
@@ -455,12 +476,12 @@ static void run(DArgs a, cudaStream_t st) {
   a.ngr = sh.ngr;
   if (a.variant == 1) {
     // one system per block; partials keep the (system, BX-site block) layout of variant 0
-    wilson_split_kernel<MODE, PIN, PL, POUT, PA1, PA2><<<dim3((unsigned)(sh.nsb * a.nrhs)), dim3(4 * BX), 0, st>>>(a);
+    launch_step(wilson_split_kernel<MODE, PIN, PL, POUT, PA1, PA2>, dim3((unsigned)(sh.nsb * a.nrhs)), dim3(4 * BX), 0, st, a);
   } else if (a.variant == 2 && wilson_tiles_fit(a.g)) {
     const unsigned ntiles = (unsigned)(a.g.V / (TX * TY * TZ * TT));
-    wilson_kernel<MODE, PIN, PL, POUT, PA1, PA2, true><<<dim3(ntiles, (unsigned)a.nrhs), dim3(TX * TY * TZ * TT), 0, st>>>(a);
+    launch_step(wilson_kernel<MODE, PIN, PL, POUT, PA1, PA2, true>, dim3(ntiles, (unsigned)a.nrhs), dim3(TX * TY * TZ * TT), 0, st, a);
   } else {
-    wilson_kernel<MODE, PIN, PL, POUT, PA1, PA2, false><<<sh.grid(), sh.block(), 0, st>>>(a);
+    launch_step(wilson_kernel<MODE, PIN, PL, POUT, PA1, PA2, false>, sh.grid(), sh.block(), 0, st, a);
   }
 }
 
@@ -468,6 +489,9 @@ static DArgs base_args(const Geom& g, double kappa, LinkRef links, int nrhs) {
   DArgs a;
   a.g = g;
   a.kappa = kappa;
+  const float2 kf = split_df(kappa);
+  a.kap_h = kf.x;
+  a.kap_l = kf.y;
   a.links = links;
   a.in = a.out = a.aux1 = a.aux2 = SpinorRef{nullptr, nullptr, g.V};
   a.nrhs = nrhs;
@@ -480,7 +504,7 @@ static DArgs base_args(const Geom& g, double kappa, LinkRef links, int nrhs) {
   a.herm = 0;
   a.variant = nrhs >= 4 ? links.variant_multi : links.variant;
   a.lz = nullptr;
-  a.lzc = LzCtl{nullptr, nullptr, nullptr, nullptr, 0, nullptr};
+  a.lzc = LzCtl{nullptr, nullptr, nullptr, nullptr, 0, nullptr, 0};
   return a;
 }
 

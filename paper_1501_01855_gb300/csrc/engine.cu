@@ -630,7 +630,7 @@ static ovl_status sign_op_batch_lz(ovl_ctx* c, int mode, const Field& v, int vof
   double* ahist = c->lz_hist;
   double* bhist = c->lz_hist + (size_t)c->lz_n * c->lz_cap;
   const int hcap = c->lz_cap;   // row length of the histories and coefficient buffers
-  const LzCtl ctl{c->lz, c->lz_ctr, ahist, bhist, hcap, c->dpoles};
+  const LzCtl ctl{c->lz, c->lz_ctr, ahist, bhist, hcap, c->dpoles, 0};
   ProfPair pp;
 
   const Field* vin;
@@ -656,10 +656,12 @@ static ovl_status sign_op_batch_lz(ovl_ctx* c, int mode, const Field& v, int vof
         (unsigned long long)(uintptr_t)c->partials, (unsigned long long)(uintptr_t)c->lz,
         (unsigned long long)(uintptr_t)c->lz_hist, (unsigned long long)(uintptr_t)L.data,
         (unsigned long long)L.variant};
+    LzCtl gctl = ctl;
+    gctl.pdl = 1;
     OVL_TRY(ms_graph(c, key, &gexec, [&](cudaStream_t cs) {
       for (int k = 0; k < kGraphIters; ++k) {
-        launch_wilson_lzK(PB, PL, PB, c->g, c->kappa, L, W->ref(), t->ref(), n, c->partials, ctl, cs);
-        launch_wilson_lzL(PB, PL, PB, c->g, c->kappa, L, t->ref(), W->ref(), n, c->partials, ctl, cs);
+        launch_wilson_lzK(PB, PL, PB, c->g, c->kappa, L, W->ref(), t->ref(), n, c->partials, gctl, cs);
+        launch_wilson_lzL(PB, PL, PB, c->g, c->kappa, L, t->ref(), W->ref(), n, c->partials, gctl, cs);
       }
     }));
   }

@@ -72,7 +72,8 @@ struct LzRhs {
   int even;            // 1: stop when every pole is within thr / N_Z (relaxed signs of relCG)
   long long w_reads;   // basis vector passes of the L mode (bytes accounting)
   double w[NPMAX];     // pole weights of this cycle (omega_i in the first)
-  double d[NPMAX];     // LDL^T pivots of T_j + sigma_i
+  float2 fn, fa, fb;   // inv_n, a, b as hi + lo of two floats (.x is the float nearest to each)
+  double rd[NPMAX];    // reciprocals of the LDL^T pivots of T_j + sigma_i
   double rho[NPMAX];   // residual norms of the shifted Galerkin solutions
 };
 
@@ -132,6 +133,7 @@ struct LzCtl {
   double* bhist;       // beta_j
   int hcap;
   const Poles* poles;
+  int pdl = 0;         // launch each step as a programmatic dependent of the one before (graphs)
 };
 void launch_wilson_lzK(int pw, int plink, int pt, const Geom& g, double kappa, LinkRef links, SpinorRef W,
                        SpinorRef t, int nrhs, double* partials, const LzCtl& ctl, cudaStream_t st);

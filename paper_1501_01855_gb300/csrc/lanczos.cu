@@ -12,7 +12,7 @@
 // pass over the stored vectors.
 //
 // Per step j (lz[rhs].j = j, unnormalised vectors W_l with v_l = W_l / n_l), two Wilson
-// launches whose last block per system also runs the scalar step (dslash.cu, lz_finish):
+// launches whose last block per system also runs the scalar step (wilson.cuh, lz_step):
 //   MODE_LZK   t = K v_j;  alpha_j = ||t||^2,  a = alpha_j / n_j,  b = beta_{j-1} / n_{j-1}
 //   MODE_LZL   W_{j+1} = K t - a W_j - b W_{j-1};  beta_j = ||W_{j+1}|| = n_{j+1}, for every
 //              pole the LDL^T pivot d_j = alpha_j + sigma_i - beta_{j-1}^2 / d_{j-1} and the
@@ -174,7 +174,7 @@ __global__ void lz_start_kernel(LzRhs* lz, const double* partials, int nsb, cons
   const double n0 = sqrt(nn);
   for (int i = threadIdx.x; i < P->n; i += blockDim.x) {
     if (first) L.w[i] = P->omega[i];
-    L.d[i] = 0.0;
+    L.rd[i] = 0.0;
     L.rho[i] = n0;
   }
   if (threadIdx.x == 0) {
@@ -191,6 +191,8 @@ __global__ void lz_start_kernel(LzRhs* lz, const double* partials, int nsb, cons
     L.vnorm = n0;
     L.inv_n = n0 > 0.0 ? 1.0 / n0 : 0.0;
     L.inv_nprev = 0.0;
+    L.fn = split_df(L.inv_n);
+    L.fa = L.fb = make_float2(0.f, 0.f);
     L.a = L.b = L.alpha = L.beta_prev = 0.0;
     L.err = 0.0;
     L.j = 0;

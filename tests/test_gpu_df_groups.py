@@ -23,3 +23,20 @@ def test_df_wilson_groups(dims, variant, apt):
     c.wilson_apply(psi, out, 3)
     for j in range(3):
         assert rel(out[j], wilson.apply_K(U, psi[j], M0, bool(apt))) <= 2e-13
+
+
+@pytest.mark.parametrize("dims", [(2, 2, 2, 2), (6, 2, 4, 6), (4, 14, 2, 4), (10, 6, 14, 12)])
+@pytest.mark.parametrize("n", [1, 3])
+@pytest.mark.parametrize("prec,eta,bound", [(3, 1e-10, 2e-10), (1, 1e-5, 2e-5)])
+def test_sign_step_on_few_and_ragged_blocks(dims, n, prec, eta, bound):
+    """The Lanczos step sums one partial per block of a launch: one to dozens of blocks, odd and
+    even counts, small double-float blocks. Both signs are within their stopping bounds of the
+    same rational, so they differ by at most the sum of the two."""
+    U = synth.gauge_links(dims, 0.3, 63)
+    c = ctx(dims, U, n_poles=20, a=0.1, b=2.7)
+    v = synth.gaussian_source(dims, 64, nvec=n)
+    ref, out = np.zeros_like(v), np.zeros_like(v)
+    c.sign_apply(v, ref, eta=min(eta, 1e-10), prec=0)
+    c.sign_apply(v, out, eta=eta, prec=prec)
+    for j in range(n):
+        assert rel(out[j], ref[j]) <= bound
