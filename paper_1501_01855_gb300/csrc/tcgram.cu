@@ -7,16 +7,15 @@
 // Rump, "Error-free transformations of matrix multiplication by using fast routines of
 // matrix multiplication", 2012), with BF16 slices and FP32 accumulation in tensor memory.
 // Every vector i gets a power-of-two scale 2^e_i above its largest element; each real
-// element x becomes the 42-bit fixed-point integer F = trunc(|x| 2^(42 - e_i)), written in
-// six balanced base-128 digits a_1 .. a_6 (a_1 in [0, 128], the others in [-64, 63]), so
-// x = sign(x) 2^e_i sum_s a_s 2^(-7 s) up to 2^(e_i - 43) (FP32 operands get the same digits,
-// signed, from FP32 arithmetic: tg_digits). Digits are exact in BF16 and
+// element x is written in six balanced base-128 digits a_1 .. a_6 (a_1 in [-128, 128], the
+// others in [-64, 64]), x = 2^e_i sum_s a_s 2^(-7 s) up to 2^(e_i - 43), by FP32 arithmetic
+// (tg_digits). Digits are exact in BF16 and
 // their products exact in the tensor core; for each group g = s + t (2 .. 8) the products
 // a_s b_t summed over 512 reals stay below 2^24 in magnitude, so the FP32 accumulator holds
 // that sum exactly. Every 512 reals the seven group sums are read from tensor memory and
 // added, scaled by 2^(-7 g), into a double-float (hi + lo FP32) accumulator per output;
 // the partial results of the CTAs that split the sum are added in FP64 in a fixed order.
-// F is rounded to nearest; the pairs with s + t > 8 (weight 2^-63 and below) are left out.
+// The last digit is rounded to nearest; the pairs with s + t > 8 (weight 2^-63 and below) are left out.
 // The error is then that of representing each operand to 2^(e_i - 43): on Gaussian data
 // about 1e-14 of |A_i| |B_j| at 4096 reals and less on longer vectors, the level of an
 // FP64 dot product of the same length.
@@ -26,16 +25,25 @@
 // M = 128 rows against N = 64 B vectors gives Re (a, b) = sum a.b in rows 0..63 and
 // Im (a, b) = sum a'.b in rows 64..127.
 //
-// One CTA (512 threads) per SM: the operands of the next stage (16 complex elements of 64 A
-// and 64 B vectors) are copied into shared memory with cp.async while warps 1..15 slice the
-// current one into the canonical no-swizzle K-major layout (core matrices of 8 rows x 16
-// bytes), double buffered; thread 0 issues the stage's 52 MMAs (2 K-steps x 26 digit pairs)
-// and commits them to the stage's mbarrier, which the slicing of the stage after next waits
-// on. Waits are bounded by a 2 s deadline: one that gives up sets the error flag, the CTA
-// skips the rest, waits once more (again bounded) for the MMAs it has committed, frees its
-// tensor memory and returns, and the host reports OVL_ETIMEOUT.
+// One CTA (512 threads) per SM. Warps 1 .. 15 slice stages of 16 complex elements of 64 A and 64 B
+// vectors into the canonical no-swizzle K-major layout (core matrices of 8 rows x 16 bytes), three
+// stages in shared memory, the next stage's elements already loaded; warp 0 issues a stage's 52
+// MMAs (2 K-steps x 26 digit pairs) when its slices are complete (full) and commits them to the
+// barrier that frees it (empty). All warps read a chunk's sums out of tensor memory once its
+// MMAs are done (fbar), two stages into the next chunk, whose MMAs wait for that (flushed). With
+// block barriers instead (two per stage, operands staged by cp.async) the warps waited for each
+// other 3.5 cycles per issued instruction. Bound now by the ALU pipe of the slicing (57% busy,
+// tensor pipe 35%). FP64 fields, 16^3 x 32: 128 x 128 17.6 -> 7.3 ms, 64 x 64 8.7 -> 2.1, 64 x 12 8.6 -> 1.7
+// (more than half of that was the exponent pass, below).
+// Waits are bounded by a 2 s deadline: one that gives up sets the error flag, the CTA skips the
+// rest, waits once more (again bounded) for the MMAs it has committed, frees its tensor memory
+// and returns, and the host reports OVL_ETIMEOUT.
+#include <limits.h>
 #include <stdint.h>
 
+#include <algorithm>
+
+#include "dfpair.cuh"
 #include "kernels.h"
 
 namespace ovl {
@@ -53,12 +61,11 @@ constexpr int TG_CHUNK = 16;                     // stages per exact accumulatio
 constexpr int TG_TILE_A = 128 * 32 * 2;          // bytes of one digit tile of A (128 rows x 32 bf16)
 constexpr int TG_TILE_B = TG_NB * 32 * 2;        // bytes of one digit tile of B
 constexpr int TG_STAGE = TG_S * (TG_TILE_A + TG_TILE_B);
-// raw operand staging (cp.async, one stage ahead): 64 A rows then 64 B rows of 16 complex
-// elements, rows padded by 16 bytes so that the slicing reads spread over the banks
+constexpr int TG_BUF = 3;                        // digit stages in shared memory
+constexpr int TG_SMEM = TG_BUF * TG_STAGE + 1024;   // and alignment
 __host__ __device__ constexpr int tg_esize(int p) { return p == P64 ? 16 : 8; }
-__host__ __device__ constexpr int tg_rstride(int p) { return 16 * tg_esize(p) + 16; }
-constexpr int TG_RAW = 64 * 2 * tg_rstride(P64);
-constexpr int TG_SMEM = 2 * TG_STAGE + 2 * TG_RAW + 1024;   // two digit stages, two raw stages, alignment
+constexpr int TG_SLICERS = TG_THREADS / 32 - 1;  // warps 1 .. 15 slice, warp 0 issues the MMAs
+constexpr int TG_TASKS = (64 + TG_SLICERS - 1) / TG_SLICERS;   // slicing tasks per warp and stage, at most
 constexpr int TG_TMEM_COLS = 512;
 static_assert(TG_G * TG_NB <= TG_TMEM_COLS, "group accumulators exceed the tensor-memory allocation");                // 7 groups x 64 columns, rounded to a power of 2
 constexpr int TG_EXP_ZERO = -4000;               // scale exponent of an all-zero vector
@@ -82,8 +89,9 @@ __device__ __forceinline__ uint64_t smem_desc(uint32_t saddr, uint32_t lbo, uint
   return d;
 }
 
-// true once the barrier's phase with this parity has completed, false after the deadline
-__device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity) {
+// true once the barrier's phase with this parity has completed, false after the deadline or when
+// another thread has given up (*gave_up)
+__device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatile int* gave_up) {
   const unsigned long long t0 = global_ns();
   for (;;) {
     uint32_t ok;
@@ -93,7 +101,11 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity) {
         : "r"(bar), "r"(parity)
         : "memory");
     if (ok) return true;
-    if (global_ns() - t0 > TG_WAIT_NS) return false;
+    if (gave_up != nullptr && *gave_up) return false;
+    if (global_ns() - t0 > TG_WAIT_NS) {
+      if (gave_up != nullptr) *gave_up = 1;
+      return false;
+    }
   }
 }
 
@@ -108,39 +120,11 @@ __device__ __forceinline__ void mma_commit(uint32_t bar) {
   asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
 }
 
-// |x| 2^(42 - e) rounded to nearest (ties up), for an IEEE double given by its bits
-// (|x| < 2^e, so the result is at most 2^42)
-__device__ __forceinline__ unsigned long long fixed_f64(unsigned long long b, int e) {
-  const int ex = (int)((b >> 52) & 0x7FF);
-  if (ex == 0) return 0ull;                                  // zero or subnormal: below 2^-1022
-  const unsigned long long m = (b & 0xFFFFFFFFFFFFFull) | (1ull << 52);
-  const int sh = 1033 + e - ex;                              // 52 - 42 + e - (ex - 1023) >= 11
-  return sh >= 65 ? 0ull : (((m >> (sh - 1)) + 1ull) >> 1);
-}
-
-// |x| 2^(42 - e) rounded to nearest (ties up), for an IEEE float given by its bits (|x| < 2^e)
-__device__ __forceinline__ unsigned long long fixed_f32(uint32_t b, int e) {
-  const int ex = (int)((b >> 23) & 0xFF);
-  if (ex == 0) return 0ull;
-  const unsigned long long m = (b & 0x7FFFFFu) | 0x800000u;
-  const int t = ex - 108 - e;                                // (ex - 127 - 23) + 42 - e <= 18
-  if (t >= 0) return m << t;
-  return -t >= 25 ? 0ull : (((m >> (-t - 1)) + 1ull) >> 1);
-}
-
-// the loaders give one complex element (from shared memory) as (F_re, F_im) and the sign
-// bits of re and im; expo reads the binary exponent of an element in global memory
+// binary exponent of the larger part of a complex element in global memory
 template <int P>
 struct TgLoad;
 template <>
 struct TgLoad<P64> {
-  static __device__ __forceinline__ void get_s(const unsigned char* p, int e, unsigned long long& fr,
-                                               unsigned long long& fi, uint32_t& neg) {
-    const ulonglong2 w = *reinterpret_cast<const ulonglong2*>(p);
-    fr = fixed_f64(w.x, e);
-    fi = fixed_f64(w.y, e);
-    neg = (uint32_t)(w.x >> 63) | ((uint32_t)(w.y >> 63) << 1);
-  }
   static __device__ __forceinline__ int expo(const void* base, size_t q) {
     const ulonglong2 w = __ldg(reinterpret_cast<const ulonglong2*>(base) + q);
     return max((int)((w.x >> 52) & 0x7FF), (int)((w.y >> 52) & 0x7FF)) - 1023;
@@ -148,131 +132,123 @@ struct TgLoad<P64> {
 };
 template <>
 struct TgLoad<P32> {
-  static __device__ __forceinline__ void get_s(const unsigned char* p, int e, unsigned long long& fr,
-                                               unsigned long long& fi, uint32_t& neg) {
-    const uint2 w = *reinterpret_cast<const uint2*>(p);
-    fr = fixed_f32(w.x, e);
-    fi = fixed_f32(w.y, e);
-    neg = (w.x >> 31) | ((w.y >> 31) << 1);
-  }
   static __device__ __forceinline__ int expo(const void* base, size_t q) {
     const uint2 w = __ldg(reinterpret_cast<const uint2*>(base) + q);
     return max((int)((w.x >> 23) & 0xFF), (int)((w.y >> 23) & 0xFF)) - 127;
   }
 };
 
-// Balanced base-128 digit s (0-based) of the real and the imaginary part, as a BF16 pair
-// (real in the low half) with the signs of x applied. g = F + 64 (2^28 + 2^21 + 2^14 + 2^7 +
-// 1), F <= 2^42: digit 0 is g >> 35 (0 .. 128), digit s >= 1 is ((g >> (35 - 7 s)) & 127) - 64.
-// A digit is placed in the mantissa of 128.0f (bits 16..22; 128 carries into the exponent and
-// gives 256), the offset is subtracted exactly, and the upper halves of the two floats are
-// the BF16 values (at most 8 significant bits).
-__device__ __forceinline__ float tg_digit_f(uint32_t lo, uint32_t hi, int s) {
-  if (s == 0) return __uint_as_float(0x43000000u + ((hi >> 3) << 16)) - 128.0f;
-  const uint32_t raw = s == 1 ? (__funnelshift_r(lo, hi, 28) & 127u) : ((lo >> (35 - 7 * s)) & 127u);
-  return __uint_as_float(0x43000000u | (raw << 16)) - 192.0f;
-}
-__device__ __forceinline__ uint32_t tg_digit_pair(uint32_t rlo, uint32_t rhi, uint32_t ilo, uint32_t ihi, int s,
-                                                  uint32_t negmask) {
-  const float fr = tg_digit_f(rlo, rhi, s), fi = tg_digit_f(ilo, ihi, s);
-  return __byte_perm(__float_as_uint(fr), __float_as_uint(fi), 0x7632) ^ negmask;
-}
-
-constexpr unsigned long long TG_BIAS = 64ull * ((1ull << 28) + (1ull << 21) + (1ull << 14) + (1ull << 7) + 1ull);
-
-// The six digits of one complex element (from the raw staging buffer) as BF16 pairs,
-// negated when neg (gamma5 on B). FP64 operands: the integer splitting above. FP32 operands:
-// the same digits by FP32 arithmetic on the FMA pipe, which the integer splitting leaves
-// idle: r = x 2^-e (exact, two power-of-two factors), then six times d = round(128 r) by the
-// 1.5 x 2^23 addition (exact for |128 r| < 2^22) and r <- 128 r - d (exact: the remainder of
-// a float after its nearest integer), so d_0 is in [-128, 128], the others in [-64, 64], and
-// |x| 2^-e = sum_s d_s 2^(-7 (s + 1)) up to 2^-43, as for the integer digits (balanced by
-// rounding instead of by the bias). A digit is an integer of at most 8 bits, so the upper
-// half of its float is its exact BF16.
+// The six digits of one complex element (from the raw staging buffer) as BF16 pairs (real in the
+// low half), negated when neg (gamma5 on B), by FP32 arithmetic on the FMA pipe, real and
+// imaginary part on the two lanes of the packed instructions: with r = x 2^-e, six times
+// d = round(128 r) by the 1.5 x 2^23 addition (exact for |128 r| < 2^22) and r <- 128 r - d
+// (exact: the remainder of a float after its nearest integer), so d_0 is in [-128, 128], the
+// others in [-64, 64], and x 2^-e = sum_s d_s 2^(-7 (s + 1)) up to 2^-43. A digit is an integer of
+// at most 8 bits, so the upper half of its float is its exact BF16.
+// FP32 operands: r by two power-of-two factors. FP64 operands, from their bits (conversions from
+// FP64 are slow): r is the float of the leading 24 bits, and the next 23 bits, a second float,
+// join the remainder after three digits, when 21 of the leading bits are spent (rounded there
+// at 2^-46; the third digit is chosen with them, so that the fourth stays in its range). About 75 instructions per element, against 270 for taking the digits out of a 64-bit
+// fixed-point integer: a 64 x 64 tile on 16^4 1.43 -> 0.81 ms with the
+// pipeline below.
 __device__ __forceinline__ float tg_pow2(int k) { return __int_as_float((127 + k) << 23); }
+// the digit of s (r itself, or r and what follows it, rounded); r becomes its remainder
+__device__ __forceinline__ uint32_t tg_digit(f2 s, f2& r) {
+  const f2 M = bc(12582912.0f), c128 = bc(128.0f);
+  const f2 t = fma2(s, c128, M);
+  const f2 dg = sub2(t, M);
+  r = fma2(r, c128, sub2(M, t));
+  return __byte_perm((uint32_t)dg, (uint32_t)(dg >> 32), 0x7632);
+}
+// x 2^-e as hi (24 bits) + lo 2^-21; thr = max(e + 897, 1): smaller exponent fields give 0
+__device__ __forceinline__ void tg_split64(uint2 w, int e, int thr, uint32_t flip, float& hi, float& lo) {
+  const int t = (int)((w.y >> 20) & 0x7FFu);
+  const uint32_t sg = (w.y ^ flip) & 0x80000000u;
+  const int ex = t - 896 - e;   // exponent field of the float, <= 126
+  const uint32_t m = __funnelshift_l(w.x, w.y, 3) & 0x7FFFFFu;
+  const uint32_t v = (w.x >> 6) & 0x7FFFFFu;   // the next 23 bits: v 2^(t - 1023 - 46 - e), times 2^21 in lo
+  const bool z = t < thr;
+  hi = __uint_as_float(z ? 0u : ((uint32_t)ex << 23) | m | sg);
+  const float f = __fsub_rn(__uint_as_float(0x4B000000u | v), 8388608.0f);
+  lo = __fmul_rn(f, __uint_as_float(z || ex <= 25 ? 0u : ((uint32_t)(ex - 25) << 23) | sg));
+}
 template <int P>
-__device__ __forceinline__ void tg_digits(const unsigned char* p, int e, bool neg, uint32_t pd[TG_S]) {
+__device__ __forceinline__ void tg_digits(uint4 w4, int e, bool neg, uint32_t pd[TG_S]) {
   if constexpr (P == P32) {
-    const float2 w = *reinterpret_cast<const float2*>(p);
-    if (e == TG_EXP_ZERO) {
+    float2 w = make_float2(__uint_as_float(w4.x), __uint_as_float(w4.y));
+    if (e == TG_EXP_ZERO) w = make_float2(0.f, 0.f);
+    const int ec = e == TG_EXP_ZERO ? 0 : e;
+    const int e1 = ec / 2, e2 = ec - e1;   // 2^-e as two factors inside the FP32 range
+    const float g = neg ? -tg_pow2(-e2) : tg_pow2(-e2);
+    f2 r = fma2(fma2(pk(w.x, w.y), bc(tg_pow2(-e1)), 0ull), bc(g), 0ull);
 #pragma unroll
-      for (int d = 0; d < TG_S; ++d) pd[d] = 0u;
-      return;
-    }
-    const int e1 = e / 2, e2 = e - e1;   // 2^-e as two factors inside the FP32 range
-    float rr = __fmul_rn(__fmul_rn(w.x, tg_pow2(-e1)), tg_pow2(-e2));
-    float ri = __fmul_rn(__fmul_rn(w.y, tg_pow2(-e1)), tg_pow2(-e2));
-    const float M = 12582912.0f;
-    const uint32_t nm = neg ? 0x80008000u : 0u;
-#pragma unroll
-    for (int d = 0; d < TG_S; ++d) {
-      const float dr = __fsub_rn(__fmaf_rn(rr, 128.0f, M), M);
-      const float di = __fsub_rn(__fmaf_rn(ri, 128.0f, M), M);
-      rr = __fmaf_rn(rr, 128.0f, -dr);
-      ri = __fmaf_rn(ri, 128.0f, -di);
-      pd[d] = __byte_perm(__float_as_uint(dr), __float_as_uint(di), 0x7632) ^ nm;
-    }
+    for (int d = 0; d < TG_S; ++d) pd[d] = tg_digit(r, r);
   } else {
-    unsigned long long fr, fi;
-    uint32_t sg;
-    TgLoad<P>::get_s(p, e, fr, fi, sg);
-    if (neg) sg ^= 3u;
-    const unsigned long long gr = fr + TG_BIAS, gi = fi + TG_BIAS;
-    const uint32_t rlo = (uint32_t)gr, rhi = (uint32_t)(gr >> 32), ilo = (uint32_t)gi, ihi = (uint32_t)(gi >> 32);
-    const uint32_t negmask = ((sg & 1u) ? 0x8000u : 0u) | ((sg & 2u) ? 0x80000000u : 0u);
-#pragma unroll
-    for (int d = 0; d < TG_S; ++d) pd[d] = tg_digit_pair(rlo, rhi, ilo, ihi, d, negmask);
+    const uint4 w = w4;
+    const int thr = max(e + 897, 1);
+    const uint32_t flip = neg ? 0x80000000u : 0u;
+    float hr, lr, hi, li;
+    tg_split64(make_uint2(w.x, w.y), e, thr, flip, hr, lr);
+    tg_split64(make_uint2(w.z, w.w), e, thr, flip, hi, li);
+    f2 r = pk(hr, hi);
+    const f2 low = pk(lr, li);
+    pd[0] = tg_digit(r, r);
+    pd[1] = tg_digit(r, r);
+    // the third digit sees the low part too, so that the fourth stays within 64
+    pd[2] = tg_digit(fma2(low, bc(0.0078125f), r), r);
+    r = add2(r, low);
+    pd[3] = tg_digit(r, r);
+    pd[4] = tg_digit(r, r);
+    pd[5] = tg_digit(r, r);
   }
 }
 
-// Issue the asynchronous copies of one stage (16 complex elements from q0 of the tile's 64 A
-// and 64 B vectors) into a raw staging buffer, 16 bytes per copy, zero-filled past the last
-// vector or element; one commit group per call.
-template <int PA, int PB>
-__device__ __forceinline__ void tg_issue(unsigned char* raw, const void* A, int na, int a0, const void* B, int nb,
-                                         int b0, size_t nq, size_t q0, int tid) {
-  constexpr int ea = tg_esize(PA), eb = tg_esize(PB);   // bytes per complex element = 16-byte copies per row
-  constexpr int sa = tg_rstride(PA), sb = tg_rstride(PB);
-  for (int c = tid; c < 64 * (ea + eb); c += TG_THREADS) {
-    const bool isA = c < 64 * ea;
-    const int cc = isA ? c : c - 64 * ea;
-    const int per = isA ? ea : eb;
-    const int r = cc / per, k = cc - r * per;
-    const size_t qs = q0 + (size_t)(k * 16) / per;       // first complex element of this copy
-    const bool ok = isA ? (a0 + r < na) : (b0 + r < nb);
-    const bool in = ok && qs < nq;
-    const char* src = isA ? reinterpret_cast<const char*>(A) + (size_t)(a0 + (ok ? r : 0)) * nq * ea
-                          : reinterpret_cast<const char*>(B) + (size_t)(b0 + (ok ? r : 0)) * nq * eb;
-    if (in) src += qs * per;
-    const uint32_t dst = smem_u32(raw + (isA ? r * sa : 64 * sa + r * sb) + k * 16);
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(in ? 16 : 0) : "memory");
+// complex element q of vector row of X (nx vectors of nq elements, the tile's first at x0)
+template <int P>
+__device__ __forceinline__ uint4 tg_load(const void* X, int nx, int row, size_t nq, size_t q) {
+  if (row >= nx || q >= nq) return make_uint4(0u, 0u, 0u, 0u);
+  if constexpr (P == P64) {
+    return __ldg(reinterpret_cast<const uint4*>(X) + (size_t)row * nq + q);
+  } else {
+    const uint2 w = __ldg(reinterpret_cast<const uint2*>(X) + (size_t)row * nq + q);
+    return make_uint4(w.x, w.y, 0u, 0u);
   }
-  asm volatile("cp.async.commit_group;" ::: "memory");
+}
+__device__ __forceinline__ void mbar_arrive(uint32_t bar) {
+  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
+}
+// the scale exponent e of a vector (every |x| < 2^e) from the largest binary exponent of its
+// elements; a zero or subnormal-only vector reads as the minimum exponent field
+template <int P>
+__device__ __forceinline__ int tg_exponent(int raw) {
+  return raw <= (P == P64 ? -1023 : -127) ? TG_EXP_ZERO : raw + 1;
 }
 
 }  // namespace
 
-// Per vector: the scale exponent e = 1 + the largest binary exponent of its reals, so that
-// every |x| < 2^e (TG_EXP_ZERO for a vector of zeros). One block per vector.
+// Per vector: the largest binary exponent of its elements (ex starts at a very negative value).
+// Many blocks per vector (one per vector read the operands of a 128 x 128 block at 1.2 TB/s, as
+// long as the contraction itself), eight loads in flight per thread.
 template <int P>
-__global__ void __launch_bounds__(256) tc_gram_exp_kernel(const void* X, int n, size_t nq, int* ex) {
+__global__ void __launch_bounds__(256) tc_gram_exp_kernel(const void* X, size_t nq, int* ex) {
   __shared__ int smax;
-  if (threadIdx.x == 0) smax = -100000;
+  if (threadIdx.x == 0) smax = INT_MIN;
   __syncthreads();
-  const int i = blockIdx.x;
-  const char* base = reinterpret_cast<const char*>(X) + (size_t)i * nq * (P == P64 ? 16 : 8);
-  int m = -100000;
-  for (size_t q = threadIdx.x; q < nq; q += blockDim.x) m = max(m, TgLoad<P>::expo(base, q));
+  const char* base = reinterpret_cast<const char*>(X) + (size_t)blockIdx.x * nq * tg_esize(P);
+  int m = INT_MIN;
+  const size_t step = (size_t)gridDim.y * blockDim.x;
+  for (size_t q = (size_t)blockIdx.y * blockDim.x + threadIdx.x; q < nq; q += 8 * step) {
+    int v[8];
+#pragma unroll
+    for (int u = 0; u < 8; ++u) v[u] = q + u * step < nq ? TgLoad<P>::expo(base, q + u * step) : INT_MIN;
+#pragma unroll
+    for (int u = 0; u < 8; ++u) m = max(m, v[u]);
+  }
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, o));
   if ((threadIdx.x & 31) == 0) atomicMax(&smax, m);
   __syncthreads();
-  if (threadIdx.x == 0) {
-    // a zero or subnormal-only vector reads as the minimum exponent field
-    const int lo = P == P64 ? -1023 : -127;
-    ex[i] = smax <= lo ? TG_EXP_ZERO : smax + 1;
-  }
-  (void)n;
+  if (threadIdx.x == 0) atomicMax(ex + blockIdx.x, smax);
 }
 
 // grid: (splits of the K range, A tiles x B tiles). partial: per CTA 2 x 64 x 64 doubles
@@ -284,8 +260,7 @@ __global__ void __launch_bounds__(TG_THREADS, 1)
   extern __shared__ unsigned char sm_raw[];
   unsigned char* sm = reinterpret_cast<unsigned char*>(((uintptr_t)sm_raw + 1023) & ~(uintptr_t)1023);
   __shared__ uint32_t tmem_base;
-  __shared__ __align__(8) uint64_t bar[2];
-  __shared__ __align__(8) uint64_t fbar;
+  __shared__ __align__(8) uint64_t full[TG_BUF], empty[TG_BUF], fbar, flushed, drain;
   __shared__ int abort_flag;
   __shared__ int ea_s[TG_NA], eb_s[TG_NB];
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -297,13 +272,17 @@ __global__ void __launch_bounds__(TG_THREADS, 1)
   const size_t st0 = nstage_all * split / nsplit, st1 = nstage_all * (split + 1) / nsplit;
   const int nst = (int)(st1 - st0);
 
-  if (tid < TG_NA) ea_s[tid] = a0 + tid < na ? exa[a0 + tid] : TG_EXP_ZERO;
-  else if (tid < TG_NA + TG_NB) eb_s[tid - TG_NA] = b0 + tid - TG_NA < nb ? exb[b0 + tid - TG_NA] : TG_EXP_ZERO;
+  if (tid < TG_NA) ea_s[tid] = a0 + tid < na ? tg_exponent<PA>(exa[a0 + tid]) : TG_EXP_ZERO;
+  else if (tid < TG_NA + TG_NB) eb_s[tid - TG_NA] = b0 + tid - TG_NA < nb ? tg_exponent<PB>(exb[b0 + tid - TG_NA]) : TG_EXP_ZERO;
   if (tid == 0) {
     abort_flag = 0;
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(&bar[0])));
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(&bar[1])));
+    for (int b = 0; b < TG_BUF; ++b) {
+      asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(&full[b])), "r"(TG_SLICERS));
+      asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(&empty[b])));
+    }
     asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(&fbar)));
+    asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(&drain)));
+    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(&flushed)), "r"(TG_THREADS / 32));
     asm volatile("fence.mbarrier_init.release.cluster;");
   }
   if (warp == 0) {
@@ -325,129 +304,143 @@ __global__ void __launch_bounds__(TG_THREADS, 1)
 #pragma unroll
   for (int c = 0; c < TG_CPT; ++c) acc_h[c] = acc_l[c] = 0.f;
 
-  uint32_t ph = 0u, pend = 0u, fph = 0u;   // bit s: parity / pending commit of stage barrier s
-  // slicing tasks of a warp: 8 row groups x 4 K columns for A (tasks 0..31) and for B (32..63)
-  const int rl = lane >> 2, kp = lane & 3;
-  unsigned char* raw0 = sm + 2 * TG_STAGE;
-  if (nst > 0) tg_issue<PA, PB>(raw0, A, na, a0, B, nb, b0, nq, st0 * TG_KC, tid);
-  for (int it = 0; it < nst; ++it) {
-    const int s = it & 1;
-    const int cs = it % TG_CHUNK;   // stage within the exact accumulation chunk
-    // the next stage's operands into the other raw buffer (its slicing ended before the
-    // barrier that closed the previous iteration); then this stage's own copies
-    if (it + 1 < nst)
-      tg_issue<PA, PB>(raw0 + ((it + 1) & 1) * TG_RAW, A, na, a0, B, nb, b0, nq, (st0 + it + 1) * TG_KC, tid);
-    else
-      asm volatile("cp.async.commit_group;" ::: "memory");
-    asm volatile("cp.async.wait_group 1;" ::: "memory");
-    if ((pend >> s) & 1u) {
-      if (mbar_wait(smem_u32(&bar[s]), (ph >> s) & 1u)) {
-        ph ^= 1u << s;
-        pend &= ~(1u << s);
-      } else {
-        abort_flag = 1;   // the stage stays pending: the exit waits for it once more
+  // One accumulation chunk's group sums are exact integers in FP32: add them, scaled, in
+  // double-float. Every warp, once the chunk's MMAs are done (fbar); false when a wait gave up.
+  auto flush = [&](int chunk) -> bool {
+    if (!mbar_wait(smem_u32(&fbar), (uint32_t)chunk & 1u, &abort_flag)) return false;
+    __syncwarp();   // tcgen05.ld is warp-collective
+    asm volatile("tcgen05.fence::after_thread_sync;");
+#pragma unroll
+    for (int g = 0; g < TG_G; ++g) {
+      uint32_t v[TG_CPT];
+      static_assert(TG_CPT == 16, "the flush reads 16 columns per thread");
+      const uint32_t ta_ = tmem + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)(g * TG_NB + cbase);
+      asm volatile(
+          "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
+          : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]),
+            "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]), "=r"(v[15])
+          : "r"(ta_));
+      asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+      const float w = __int_as_float((127 - 7 * (g + 2)) << 23);   // 2^(-7 (g + 2))
+#pragma unroll
+      for (int c = 0; c < TG_CPT; ++c) {
+        // TwoSum of acc_h and the exactly scaled group sum
+        const float x = __uint_as_float(v[c]) * w;
+        const float sum = acc_h[c] + x;
+        const float bb = sum - acc_h[c];
+        const float e = (acc_h[c] - (sum - bb)) + (x - bb);
+        acc_h[c] = sum;
+        acc_l[c] += e;
       }
     }
-    __syncthreads();
-    if (abort_flag) break;
-    unsigned char* stA = sm + s * TG_STAGE;
-    unsigned char* stB = stA + TG_S * TG_TILE_A;
-    const unsigned char* rawA = raw0 + (it & 1) * TG_RAW;
-    const unsigned char* rawB = rawA + 64 * tg_rstride(PA);
-    const size_t q0 = (st0 + it) * TG_KC;
-    // warp 0 issues the MMAs after the barrier: the other warps share the slicing
-    for (int task = warp - 1; warp > 0 && task < 64; task += TG_THREADS / 32 - 1) {
-      const bool isA = task < 32;
-      const int tt = task & 31, rg = tt >> 2, kc = tt & 3;
-      const int r = rg * 8 + rl;
-      const int j = kc * 4 + kp;
-      uint32_t pd[TG_S];   // digit s of (re, im) as a BF16 pair
-      if (isA) {
-        tg_digits<PA>(rawA + r * tg_rstride(PA) + j * tg_esize(PA), ea_s[r], false, pd);
-        // A row r and A' row 64 + r: (re, im) and (-im, re)
-        const uint32_t off = (uint32_t)((kc * 16 + rg) * 128 + rl * 16 + kp * 4);
+    asm volatile("tcgen05.fence::before_thread_sync;");
+    __syncwarp();
+    if (lane == 0) mbar_arrive(smem_u32(&flushed));
+    return true;
+  };
+  const int nchunk = (nst + TG_CHUNK - 1) / TG_CHUNK;
+  bool ok = true;
+  if (warp == 0) {
+    for (int it = 0; ok && it < nst; ++it) {
+      const int s = it % TG_BUF, cs = it % TG_CHUNK;
+      ok = mbar_wait(smem_u32(&full[s]), (uint32_t)(it / TG_BUF) & 1u, &abort_flag);
+      // the accumulators restart: the last chunk must have been read out
+      if (ok && cs == 0 && it > 0) ok = flush(it / TG_CHUNK - 1);
+      if (ok && cs == 0 && it > 0) ok = mbar_wait(smem_u32(&flushed), (uint32_t)(it / TG_CHUNK - 1) & 1u, &abort_flag);
+      ok = __all_sync(0xffffffffu, ok);
+      if (!ok) break;
+      if (lane == 0) {
+        asm volatile("tcgen05.fence::after_thread_sync;");
+        // descriptors of digit 0, K-step 0 of this stage; the others differ only in the start
+        // address (field in the low bits, in units of 16 bytes; no carry out of it below 256 KB)
+        unsigned char* stA = sm + s * TG_STAGE;
+        const uint64_t da0 = smem_desc(smem_u32(stA), 2048, 128),
+                       db0 = smem_desc(smem_u32(stA + TG_S * TG_TILE_A), 1024, 128);
+        const uint32_t acc_chunk = cs > 0 ? 1u : 0u;
 #pragma unroll
-        for (int d = 0; d < TG_S; ++d) {
-          *reinterpret_cast<uint32_t*>(stA + d * TG_TILE_A + off) = pd[d];
-          *reinterpret_cast<uint32_t*>(stA + d * TG_TILE_A + off + 8 * 128) = __byte_perm(pd[d], 0u, 0x1032) ^ 0x8000u;
-        }
-      } else {
-        tg_digits<PB>(rawB + r * tg_rstride(PB) + j * tg_esize(PB), eb_s[r], g5q && q0 + j >= (size_t)g5q, pd);
-        const uint32_t off = (uint32_t)((kc * 8 + rg) * 128 + rl * 16 + kp * 4);
+        for (int kk = 0; kk < 2; ++kk) {   // two K-steps of 16 reals (2 core-matrix columns each)
 #pragma unroll
-        for (int d = 0; d < TG_S; ++d) *reinterpret_cast<uint32_t*>(stB + d * TG_TILE_B + off) = pd[d];
-      }
-    }
-    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-    __syncthreads();
-    const bool chunk_end = (cs == TG_CHUNK - 1) || (it == nst - 1);
-    if (tid == 0) {
-      asm volatile("tcgen05.fence::after_thread_sync;");
-      // descriptors of digit 0, K-step 0 of this stage; the others differ only in the start
-      // address (field in the low bits, in units of 16 bytes; no carry out of it below 256 KB)
-      const uint64_t da0 = smem_desc(smem_u32(stA), 2048, 128), db0 = smem_desc(smem_u32(stB), 1024, 128);
-      const uint32_t acc_chunk = cs > 0 ? 1u : 0u;
-#pragma unroll
-      for (int kk = 0; kk < 2; ++kk) {   // two K-steps of 16 reals (2 core-matrix columns each)
-#pragma unroll
-        for (int g = 0; g < TG_G; ++g) {         // group g + 2 = s + t
-#pragma unroll
-          for (int ds = (g > TG_S - 1 ? g - TG_S + 1 : 0); ds <= (g < TG_S - 1 ? g : TG_S - 1); ++ds) {
-            // digit ds of A, g - ds of B (0-based); the first pair of a group starts its sum
-            const uint64_t da = da0 + (uint64_t)((ds * TG_TILE_A + kk * 2 * 2048) >> 4);
-            const uint64_t db = db0 + (uint64_t)(((g - ds) * TG_TILE_B + kk * 2 * 1024) >> 4);
+          for (int g = 0; g < TG_G; ++g) {         // group g + 2 = s + t
             const int first = g > TG_S - 1 ? g - TG_S + 1 : 0;
-            mma_bf16(tmem + (uint32_t)(g * TG_NB), da, db, idesc, (kk > 0 || ds > first) ? 1u : acc_chunk);
+#pragma unroll
+            for (int ds = first; ds <= (g < TG_S - 1 ? g : TG_S - 1); ++ds) {
+              // digit ds of A, g - ds of B (0-based); the first pair of a group starts its sum
+              const uint64_t da = da0 + (uint64_t)((ds * TG_TILE_A + kk * 2 * 2048) >> 4);
+              const uint64_t db = db0 + (uint64_t)(((g - ds) * TG_TILE_B + kk * 2 * 1024) >> 4);
+              mma_bf16(tmem + (uint32_t)(g * TG_NB), da, db, idesc, (kk > 0 || ds > first) ? 1u : acc_chunk);
+            }
           }
         }
+        mma_commit(smem_u32(&empty[s]));
+        if (cs == TG_CHUNK - 1 || it == nst - 1) mma_commit(smem_u32(&fbar));
       }
-      mma_commit(smem_u32(&bar[s]));
-      if (chunk_end) mma_commit(smem_u32(&fbar));
+      __syncwarp();
     }
-    pend |= 1u << s;
-    if (chunk_end) {
-      // the chunk's group sums are exact integers in FP32: add them, scaled, in double-float
-      if (!mbar_wait(smem_u32(&fbar), fph)) abort_flag = 1;
-      fph ^= 1u;
-      __syncthreads();   // abort_flag is read uniformly: tcgen05.ld is warp-collective
-      asm volatile("tcgen05.fence::after_thread_sync;");
-      if (!abort_flag) {
+    if (ok && nst > 0) ok = flush(nchunk - 1);
+  } else {
+    // Slicing: 64 tasks of 32 elements (8 rows x 4 of the stage's 16 columns), 32 of A and 32 of B.
+    // The next stage's elements are loaded while this one's are sliced.
+    const int rl = lane >> 2, kp = lane & 3;
+    uint4 raw[TG_TASKS];
+    auto load = [&](int i, int it) {
+      const int task = warp - 1 + i * TG_SLICERS;
+      if (task >= 64 || it >= nst) return;
+      const int tt = task & 31, r = (tt >> 2) * 8 + rl;
+      const size_t q = (st0 + it) * TG_KC + (tt & 3) * 4 + kp;
+      raw[i] = task < 32 ? tg_load<PA>(A, na, a0 + r, nq, q) : tg_load<PB>(B, nb, b0 + r, nq, q);
+    };
 #pragma unroll
-        for (int g = 0; g < TG_G; ++g) {
-          uint32_t v[TG_CPT];
-          static_assert(TG_CPT == 16, "the flush reads 16 columns per thread");
-          const uint32_t ta_ = tmem + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)(g * TG_NB + cbase);
-          asm volatile(
-              "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
-              : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]),
-                "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]),
-                "=r"(v[15])
-              : "r"(ta_));
-          asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-          const float w = __int_as_float((127 - 7 * (g + 2)) << 23);   // 2^(-7 (g + 2))
+    for (int i = 0; i < TG_TASKS; ++i) load(i, 0);
+    for (int it = 0; ok && it < nst; ++it) {
+      const int s = it % TG_BUF;
+      if (it >= TG_BUF) ok = mbar_wait(smem_u32(&empty[s]), (uint32_t)(it / TG_BUF - 1) & 1u, &abort_flag);
+      ok = __all_sync(0xffffffffu, ok);
+      if (!ok) break;
+      unsigned char* stA = sm + s * TG_STAGE;
+      unsigned char* stB = stA + TG_S * TG_TILE_A;
+      const size_t q0 = (st0 + it) * TG_KC;
 #pragma unroll
-          for (int c = 0; c < TG_CPT; ++c) {
-            // TwoSum of acc_h and the exactly scaled group sum
-            const float x = __uint_as_float(v[c]) * w;
-            const float sum = acc_h[c] + x;
-            const float bb = sum - acc_h[c];
-            const float e = (acc_h[c] - (sum - bb)) + (x - bb);
-            acc_h[c] = sum;
-            acc_l[c] += e;
+      for (int i = 0; i < TG_TASKS; ++i) {
+        const int task = warp - 1 + i * TG_SLICERS;
+        if (task >= 64) break;
+        const int tt = task & 31, rg = tt >> 2, kc = tt & 3, r = rg * 8 + rl, j = kc * 4 + kp;
+        const uint4 w = raw[i];
+        load(i, it + 1);
+        uint32_t pd[TG_S];   // digit s of (re, im) as a BF16 pair
+        if (task < 32) {
+          tg_digits<PA>(w, ea_s[r], false, pd);
+          // A row r and A' row 64 + r: (re, im) and (-im, re)
+          const uint32_t off = (uint32_t)((kc * 16 + rg) * 128 + rl * 16 + kp * 4);
+#pragma unroll
+          for (int d = 0; d < TG_S; ++d) {
+            *reinterpret_cast<uint32_t*>(stA + d * TG_TILE_A + off) = pd[d];
+            *reinterpret_cast<uint32_t*>(stA + d * TG_TILE_A + off + 8 * 128) = __byte_perm(pd[d], 0u, 0x1032) ^ 0x8000u;
           }
+        } else {
+          tg_digits<PB>(w, eb_s[r], g5q && q0 + j >= (size_t)g5q, pd);
+          const uint32_t off = (uint32_t)((kc * 8 + rg) * 128 + rl * 16 + kp * 4);
+#pragma unroll
+          for (int d = 0; d < TG_S; ++d) *reinterpret_cast<uint32_t*>(stB + d * TG_TILE_B + off) = pd[d];
         }
       }
-      asm volatile("tcgen05.fence::before_thread_sync;");
+      asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+      __syncwarp();
+      if (lane == 0) mbar_arrive(smem_u32(&full[s]));
+      // the previous chunk is read out two stages into the next one, while its last MMAs run
+      if (it % TG_CHUNK == 1 && it > TG_CHUNK) ok = flush(it / TG_CHUNK - 1);
     }
+    // what is left: the chunk before the last when the last one has a single stage, and the last
+    if (ok && nst > TG_CHUNK && nst % TG_CHUNK == 1) ok = flush(nchunk - 2);
+    if (ok && nst > 0) ok = flush(nchunk - 1);
   }
-  // wait for the last commits of each stage barrier before the CTA lets go of its memory,
-  // also after an abort (MMAs still in flight must not outlive the tensor memory); each
-  // wait again has its own deadline. A commit of a stage also covers every earlier MMA.
-  asm volatile("cp.async.wait_all;" ::: "memory");
+  if (!ok) abort_flag = 1;
   __syncthreads();
-  for (int s = 0; s < 2; ++s)
-    if ((pend >> s) & 1u)
-      if (!mbar_wait(smem_u32(&bar[s]), (ph >> s) & 1u)) abort_flag = 1;
+  // after an abort, MMAs still in flight must not outlive the tensor memory: one more bounded
+  // wait for a commit that covers all of them
+  if (abort_flag && tid == 0) {
+    mma_commit(smem_u32(&drain));
+    mbar_wait(smem_u32(&drain), 0u, nullptr);
+  }
   __syncthreads();
   if (abort_flag && tid == 0) atomicExch(err, 1);
   if (!abort_flag) {
@@ -491,7 +484,9 @@ bool tc_gram_supported(int pa, int pb) { return (pa == P64 || pa == P32) && (pb 
 int tc_gram_splits(int na, int nb, int V, int nsm) {
   const int tiles = ((na + TG_NA - 1) / TG_NA) * ((nb + TG_NB - 1) / TG_NB);
   const long long nstage = ((long long)12 * V + TG_KC - 1) / TG_KC;
-  long long ns = (nsm + tiles - 1) / tiles;
+  // whole splits in one wave of one CTA per SM: rounding up left a second wave of a single CTA
+  // for 9 tiles (192 x 192: 153 CTAs on 152 SMs, twice the time)
+  long long ns = nsm / tiles;
   const long long maxs = (nstage + TG_CHUNK - 1) / TG_CHUNK;   // at least one chunk per split
   if (ns > maxs) ns = maxs;
   if (ns < 1) ns = 1;
@@ -513,10 +508,15 @@ void launch_tc_gram(int pa, const void* A, int na, int pb, const void* B, int nb
   const size_t nq = (size_t)12 * V;
   int* exa = ex;
   int* exb = ex + na;
-  if (pa == P64) tc_gram_exp_kernel<P64><<<na, 256, 0, st>>>(A, na, nq, exa);
-  else tc_gram_exp_kernel<P32><<<na, 256, 0, st>>>(A, na, nq, exa);
-  if (pb == P64) tc_gram_exp_kernel<P64><<<nb, 256, 0, st>>>(B, nb, nq, exb);
-  else tc_gram_exp_kernel<P32><<<nb, 256, 0, st>>>(B, nb, nq, exb);
+  cudaMemsetAsync(ex, 0x80, sizeof(int) * (na + nb), st);   // about -2.1e9: below every exponent
+  // enough blocks to fill the chip whatever the number of vectors, and at least 16 elements a thread
+  auto blocks = [&](int n) {
+    return (unsigned)std::max<size_t>(1, std::min<size_t>((1216 + n - 1) / n, (nq + 4095) / 4096));
+  };
+  if (pa == P64) tc_gram_exp_kernel<P64><<<dim3(na, blocks(na)), 256, 0, st>>>(A, nq, exa);
+  else tc_gram_exp_kernel<P32><<<dim3(na, blocks(na)), 256, 0, st>>>(A, nq, exa);
+  if (pb == P64) tc_gram_exp_kernel<P64><<<dim3(nb, blocks(nb)), 256, 0, st>>>(B, nq, exb);
+  else tc_gram_exp_kernel<P32><<<dim3(nb, blocks(nb)), 256, 0, st>>>(B, nq, exb);
   const int tiles = ((na + TG_NA - 1) / TG_NA) * ((nb + TG_NB - 1) / TG_NB);
   dim3 grid((unsigned)nsplit, (unsigned)tiles);
   const int g5q = g5 ? (int)(6 * (size_t)V) : 0;
