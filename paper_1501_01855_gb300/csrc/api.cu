@@ -269,6 +269,8 @@ extern "C" void overlap_destroy(ovl_ctx* c) {
   if (c->lz_Y) cudaFree(c->lz_Y);
   if (c->lz_coefW) cudaFree(c->lz_coefW);
   if (c->lz_ctr) cudaFree(c->lz_ctr);
+  if (c->lzp_bar) cudaFree(c->lzp_bar);
+  if (c->lzp_part) cudaFree(c->lzp_part);
   if (c->dpoles) cudaFree(c->dpoles);
   if (c->dwork) cudaFree(c->dwork);
   if (c->hpin) cudaFreeHost(c->hpin);

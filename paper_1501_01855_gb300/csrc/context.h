@@ -84,6 +84,9 @@ struct ovl_ctx {
   double* lz_coefW = nullptr;    // coefficients of the stored vectors, lz_n * lz_cap doubles
   unsigned int* lz_ctr = nullptr;  // arrival counters of the fused scalar steps, lz_n
   int lz_cap = 0;
+  unsigned int* lzp_bar = nullptr;  // barrier and flags of the one-launch Lanczos iteration
+  double* lzp_part = nullptr;       // its blocks' partial sums
+  int nsm = 0;                      // SMs of the device
   void* lz_pool = nullptr;       // stored Lanczos bases of every sign precision (one at a time)
   size_t lz_pool_bytes = 0;
   bool lz_pool_busy = false;     // a sign application holds a view of the pool

@@ -411,7 +411,143 @@ void run_m(const DArgs& a, cudaStream_t st) {
   }
 }
 
+// ---- the whole Lanczos iteration in one launch (lzp_run) --------------------------------
+// A tile is P pairs of one system in G groups, as in df_wilson_kernel.
+template <int G, int P>
+struct LzpBodyDf {
+  static constexpr int X = 2 * P, T = X * G;   // threads of a group, of a tile
+  const LzPersist& p;
+  const DArgs& a;
+  ulonglong2* part;   // of this tile: [group][component (6 x re, im)][thread x]
+  int rhs, i, half, grp, x;
+  bool in_tile;
+  __device__ __forceinline__ LzpBodyDf(const LzPersist& q, ulonglong2* sm) : p(q), a(q.a) {
+    const int slot = threadIdx.x / T, lin = threadIdx.x % T, tile = blockIdx.x * p.tb + slot;
+    part = sm + slot * (G * 12 * X);
+    x = lin % X;
+    half = x & 1;
+    grp = lin / X;
+    rhs = tile % a.nrhs;
+    i = tile / a.nrhs * P + (x >> 1);
+    in_tile = tile < p.ntile && i < (a.g.V >> 1);
+  }
+  template <int MODE>
+  __device__ __forceinline__ void hop(int j, const LzpShared& sh) {
+    const bool live = in_tile && !sh.c[rhs].done;
+    dd2 up[3][2], low[3][2];
+#pragma unroll
+    for (int c = 0; c < 3; ++c)
+#pragma unroll
+      for (int r = 0; r < 2; ++r) up[c][r] = low[c][r] = dd2_zero();
+    const SpinorRef& in = MODE == MODE_LZK ? p.W : p.t;
+    const int nb = df_blocks(a.g.V), lth = a.g.L[3] >> 1, m = (x >> 1 & 7) + 8 * half;
+    const size_t fblk = (size_t)(MODE == MODE_LZK ? j * a.nrhs + rhs : rhs) * nb;
+    int xc[4] = {0, 0, 0, 0};
+    if (live) {
+      site_coords(a.g, i, xc);
+      if constexpr (MODE == MODE_LZL) {
+        // what the epilogue reads besides: on its way from HBM or L2 while the hops are summed
+        if (grp == 0) prefetch_l2_spinor(pair_at(p.W, (size_t)(j * a.nrhs + rhs) * nb, i), m);
+        if (grp == 1 && j > 0) prefetch_l2_spinor(pair_at(p.W, (size_t)((j - 1) * a.nrhs + rhs) * nb, i), m);
+      }
+    }
+    const int n0 = grp * (8 / G), n1 = n0 + 8 / G;
+    Hop h = hop_of(a.g, lth, xc, i, half, n0);
+#pragma unroll 1
+    for (int n = n0; n < n1; ++n) {
+      if (live) {
+        const int nn = min(n + 1, n1 - 1);
+        const Hop nx = hop_of(a.g, lth, xc, i, half, nn);
+        if (n + 1 < n1) {
+          prefetch_spinor(pair_at(in, fblk, nx.nbr), m);
+          prefetch_link(link_at(a.links, i, nn), m);
+        }
+        hop_pair<(G >= 4)>(pair_at(in, fblk, h.nbr), link_at(a.links, i, n), half, h, up, low);
+        h = nx;
+      }
+      if (n == min(n1 - 1, 3)) {   // as in df_wilson_kernel: the same for a warp, or for G = 8 its two hops
+#pragma unroll
+        for (int c = 0; c < 3; ++c)
+#pragma unroll
+          for (int r = 0; r < 2; ++r) {
+            low[c][r] = shfl_pair(dd2_norm(low[c][r]));
+            up[c][r] = dd2_norm(up[c][r]);
+          }
+      }
+    }
+    ulonglong2* mine = part + grp * 12 * X + x;
+#pragma unroll
+    for (int c = 0; c < 3; ++c)
+#pragma unroll
+      for (int r = 0; r < 2; ++r) {
+        mine[(2 * c + r) * X] = make_ulonglong2(up[c][r].h, up[c][r].l);
+        mine[(6 + 2 * c + r) * X] = make_ulonglong2(low[c][r].h, low[c][r].l);
+      }
+  }
+  template <int MODE>
+  __device__ __forceinline__ void finish(int j, LzpShared& sh) {
+    const LzCoef& L = sh.c[rhs];
+    dot2p d[4];
+    d[0] = {0ull, 0ull};
+    if (in_tile && !L.done) {
+      DfScal k;
+      k.kap = fac2_minus(make_float2(a.kap_h, a.kap_l));
+      if constexpr (MODE == MODE_LZK) {
+        k.s0 = {bc(L.fn.x), bc(-L.fn.x), bc(L.fn.y)};
+      } else {
+        k.s0 = fac2_minus(L.fa);
+        k.s1 = fac2_minus(L.fb);
+      }
+      for (int q = grp; q < 6; q += G) {
+        const ulonglong2* s = part + 2 * q * X + x;
+        dd2 t[1][2];
+#pragma unroll
+        for (int r = 0; r < 2; ++r) {
+          t[0][r] = {s[r * X].x, s[r * X].y};
+#pragma unroll
+          for (int z = 1; z < G; ++z) {
+            const ulonglong2 w = s[(z * 12 + r) * X];
+            t[0][r] = dd2_add(t[0][r], {w.x, w.y});
+          }
+        }
+        df_epilogue<MODE, P64E, 1>(MODE == MODE_LZK ? p.a : p.l, k, rhs, MODE == MODE_LZK ? j * a.nrhs + rhs : rhs, j,
+                                   q < 3 ? 3 * half + q : 3 + 3 * half + q, i, t, d);
+      }
+    }
+    float s0, s1, c0, c1;
+    upk(d[0].s, s0, s1);
+    upk(d[0].c, c0, c1);
+    df v = df(s0, c0) + df(s1, c1);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1)
+      v = v + df(__shfl_down_sync(0xffffffffu, v.hi, o), __shfl_down_sync(0xffffffffu, v.lo, o));
+    if (lane_id() == 0) sh.acc[threadIdx.x >> 5][rhs] = (double)v;
+  }
+};
+template <int G, int P, int TB>
+__global__ void __launch_bounds__(2 * P * G * TB + 32, 1) lz_persistent_df_kernel(const LzPersist p) {
+  extern __shared__ ulonglong2 part[];
+  __shared__ LzpShared sh;
+  LzpBodyDf<G, P> body(p, part);
+  lzp_run(p, body, sh);
+}
+template <int G, int P, int TB>
+bool lzp_df(LzPersist& p, int nsm, cudaStream_t st) {
+  p.ntile = ((p.a.g.V >> 1) + P - 1) / P * p.a.nrhs;
+  p.tb = (p.ntile + nsm - 1) / nsm;
+  return p.tb <= TB && lzp_launch(lz_persistent_df_kernel<G, P, TB>, p, 2 * P * G / 32,
+                                  sizeof(ulonglong2) * G * 12 * 2 * P, nsm, st);
+}
+
 }  // namespace
+
+// Eight groups on 8 pairs while the SMs hold every tile at 96 registers or more (9728 sites x
+// systems on 152 SMs; 80 registers spill: 8^3 x 16 2.2 instead of 2.1 ms), two groups on 16 pairs up
+// to 34048.
+bool launch_lz_persistent_df(LzPersist& p, int nsm, cudaStream_t st) {
+  return lzp_df<8, 8, 3>(p, nsm, st) || lzp_df<8, 8, 4>(p, nsm, st) || lzp_df<2, 16, 5>(p, nsm, st) ||
+         lzp_df<2, 16, 7>(p, nsm, st);
+}
 
 // Two threads per pair and system, times 1, 2, 4 or 8 groups. One group is the cheapest form
 // (no exchange in shared memory) once its threads fill the SMs; below, the hops of a pair are

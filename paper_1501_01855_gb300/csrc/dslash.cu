@@ -176,8 +176,8 @@ __device__ __forceinline__ void hop(const Geom& g, const LinkRef& L, const Spino
 
 // Epilogue shared by both kernel variants: acc holds the hop sum of site s; v gets this
 // thread's contributions to the NVRED partial sums (see the mode list at the top).
-template <int MODE, int PIN, int POUT, int PA1, int PA2, typename T>
-__device__ __forceinline__ void wilson_epilogue(const DArgs& a, int rhs, int fin, int s, cpx<T> acc[12],
+template <int MODE, int PIN, int POUT, int PA1, int PA2, typename T, typename LT>
+__device__ __forceinline__ void wilson_epilogue(const DArgs& a, const LT* L, int rhs, int fin, int s, cpx<T> acc[12],
                                                 typename RedT<T>::type v[NVRED]) {
   cpx<T> c[12];
   load_spinor_gen<PIN, T, kReadOnly<MODE>>(a.in, fin, s, c);
@@ -188,8 +188,8 @@ __device__ __forceinline__ void wilson_epilogue(const DArgs& a, int rhs, int fin
   if constexpr (MODE == MODE_LZK) {
     // t = (1 / n_j) gamma5 (W_j - kappa hop W_j)
     T sc;
-    if constexpr (std::is_same<T, float>::value) sc = a.lz[rhs].fn.x;
-    else sc = a.lz[rhs].inv_n;
+    if constexpr (std::is_same<T, float>::value) sc = L->fn.x;
+    else sc = L->inv_n;
 #pragma unroll
     for (int k = 0; k < 12; ++k) {
       cpx<T> o = c[k] - kap * acc[k];
@@ -205,15 +205,14 @@ __device__ __forceinline__ void wilson_epilogue(const DArgs& a, int rhs, int fin
     }
   } else if constexpr (MODE == MODE_LZL) {
     // W_{j+1} = gamma5 (t - kappa hop t) - a W_j - b W_{j-1}
-    const LzRhs& L = a.lz[rhs];
-    const int j = L.j;
+    const int j = L->j;
     T ca, cb;
     if constexpr (std::is_same<T, float>::value) {
-      ca = L.fa.x;
-      cb = L.fb.x;
+      ca = L->fa.x;
+      cb = L->fb.x;
     } else {
-      ca = L.a;
-      cb = L.b;
+      ca = L->a;
+      cb = L->b;
     }
     cpx<T> w[12];
     load_spinor_as<PA1, T>(a.aux1, j * a.nrhs + rhs, s, w);
@@ -375,7 +374,7 @@ __global__ void __launch_bounds__(256) __maxnreg__((MaxReg<PL, PIN>::v)) wilson_
   if (live) {
     cpx<T> acc[12];
     hop<PIN, PL, kReadOnly<MODE>, T>(a.g, a.links, a.in, fin, s, x, acc);
-    wilson_epilogue<MODE, PIN, POUT, PA1, PA2, T>(a, rhs, fin, s, acc, v);
+    wilson_epilogue<MODE, PIN, POUT, PA1, PA2, T>(a, a.lz + rhs, rhs, fin, s, acc, v);
   }
   if (a.partials != nullptr) {
     double tot[NVRED];
@@ -447,7 +446,7 @@ __global__ void __launch_bounds__(4 * BX) __maxnreg__((MaxReg<PL, PIN>::v)) wils
   if (dir == 0 && live) {
 #pragma unroll
     for (int k = 0; k < 12; ++k) acc[k] = acc[k] + part[0][sl][k] + part[1][sl][k] + part[2][sl][k];
-    wilson_epilogue<MODE, PIN, POUT, PA1, PA2, T>(a, rhs, fin, s, acc, v);
+    wilson_epilogue<MODE, PIN, POUT, PA1, PA2, T>(a, a.lz + rhs, rhs, fin, s, acc, v);
   }
   if (a.partials != nullptr) {
     double tot[NVRED];
@@ -459,6 +458,80 @@ __global__ void __launch_bounds__(4 * BX) __maxnreg__((MaxReg<PL, PIN>::v)) wils
   if constexpr (MODE == MODE_LZK || MODE == MODE_LZL) {
     if (threadIdx.x < 32) lz_arrive<MODE>(a, rhs, a.nsb);
   }
+}
+
+// ---- FP32, the whole Lanczos iteration in one launch (lzp_run) ---------------------------
+// A tile is 32 sites of one system: one warp (NS = 1), or four warps, one per direction, whose
+// sums meet in shared memory (NS = 4, when that still gives every tile its warps at once).
+template <int NS>
+struct LzpBody32 {
+  const LzPersist& p;
+  const DArgs& a;
+  cpx<float>* part;   // NS > 1: [warp][component][lane]
+  cpx<float> acc[12];
+  int rhs, s;
+  bool in_tile, live;
+  __device__ __forceinline__ LzpBody32(const LzPersist& q, cpx<float>* sm) : p(q), a(q.a), part(sm) {
+    const int tile = blockIdx.x * p.tb + (threadIdx.x >> 5) / NS;
+    rhs = tile % a.nrhs;
+    s = tile / a.nrhs * 32 + lane_id();
+    in_tile = tile < p.ntile && s < a.g.V;
+  }
+  template <int MODE>
+  __device__ __forceinline__ void sum(int j, const LzpShared& sh) {
+    live = in_tile && !sh.c[rhs].done;
+#pragma unroll
+    for (int k = 0; k < 12; ++k) acc[k] = cmk(0.f, 0.f);
+    if (!live) return;
+    const SpinorRef& in = MODE == MODE_LZK ? p.W : p.t;
+    const int fin = MODE == MODE_LZK ? j * a.nrhs + rhs : rhs;
+    int x[4];
+    site_coords(a.g, s, x);
+    const int sy = a.g.L[0], sz = sy * a.g.L[1], st = sz * a.g.L[2];
+    const int dir = NS == 1 ? -1 : (threadIdx.x >> 5) % NS;
+    if (NS == 1 || dir == 0) hop_dir<0, P32, P32, false, float>(a.g, a.links, in, fin, s, x, 1, acc);
+    if (NS == 1 || dir == 1) hop_dir<1, P32, P32, false, float>(a.g, a.links, in, fin, s, x, sy, acc);
+    if (NS == 1 || dir == 2) hop_dir<2, P32, P32, false, float>(a.g, a.links, in, fin, s, x, sz, acc);
+    if (NS == 1 || dir == 3) hop_dir<3, P32, P32, false, float>(a.g, a.links, in, fin, s, x, st, acc);
+  }
+  template <int MODE>
+  __device__ __forceinline__ void hop(int j, const LzpShared& sh) {
+    sum<MODE>(j, sh);
+    if constexpr (NS > 1) {
+      const int w = threadIdx.x >> 5;
+      if (w % NS != 0) {
+#pragma unroll
+        for (int k = 0; k < 12; ++k) part[(w * 12 + k) * 32 + lane_id()] = acc[k];
+      }
+    }
+  }
+  template <int MODE>
+  __device__ __forceinline__ void finish(int j, LzpShared& sh) {
+    const int w = threadIdx.x >> 5, lane = lane_id();
+    if (NS > 1 && w % NS != 0) return;
+    if constexpr (NS > 1) {
+#pragma unroll
+      for (int k = 0; k < 12; ++k) {
+        const cpx<float>* q = part + ((w + 1) * 12 + k) * 32 + lane;
+        acc[k] = acc[k] + q[0] + q[12 * 32] + q[24 * 32];
+      }
+    }
+    float v[NVRED] = {0.f, 0.f, 0.f, 0.f};
+    // this phase's flags: a system found done since the hop keeps its vectors
+    if (live && !sh.c[rhs].done)
+      wilson_epilogue<MODE, P32, P32, P32, P32, float>(MODE == MODE_LZK ? p.a : p.l, &sh.c[rhs], rhs,
+                                                       MODE == MODE_LZK ? j * a.nrhs + rhs : rhs, s, acc, v);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v[0] += __shfl_down_sync(0xffffffffu, v[0], o);
+    if (lane == 0) sh.acc[w][rhs] = (double)v[0];
+  }
+};
+template <int NS, int WARPS>
+__global__ void __launch_bounds__(32 * WARPS, 1) lz_persistent_f32_kernel(const LzPersist p) {
+  extern __shared__ cpx<float> parts32[];
+  __shared__ LzpShared sh;
+  LzpBody32<NS> body(p, parts32);
+  lzp_run(p, body, sh);
 }
 
 Shape make_shape(int V, int nrhs) {
@@ -506,6 +579,34 @@ static DArgs base_args(const Geom& g, double kappa, LinkRef links, int nrhs) {
   a.lz = nullptr;
   a.lzc = LzCtl{nullptr, nullptr, nullptr, nullptr, 0, nullptr, 0};
   return a;
+}
+
+bool launch_lz_persistent(int prec, const Geom& g, double kappa, LinkRef links, SpinorRef W, SpinorRef t, int nrhs,
+                          const LzCtl& ctl, double* part, unsigned int* bar, int nsm, cudaStream_t st) {
+  if (nrhs > LZP_SYS) return false;
+  LzPersist p;
+  p.a = base_args(g, kappa, links, nrhs);
+  p.a.lz = ctl.lz;
+  p.a.lzc = ctl;
+  p.a.partials = part;   // the epilogues form their partial sums
+  p.a.in = W;
+  p.a.out = t;
+  p.l = p.a;
+  p.l.in = t;
+  p.l.out = p.l.aux1 = W;
+  p.W = W;
+  p.t = t;
+  p.part = part;
+  p.bar = bar;
+  if (prec == P64E) return launch_lz_persistent_df(p, nsm, st);
+  if (prec != P32) return false;
+  // FP32: every tile has its warps at once, up to 27 per SM (72 registers; up to 19: 102)
+  p.ntile = (g.V + 31) / 32 * nrhs;
+  p.tb = (p.ntile + nsm - 1) / nsm;
+  if (4 * p.tb <= 19) return lzp_launch(lz_persistent_f32_kernel<4, 20>, p, 4, 4 * 12 * 32 * sizeof(cpx<float>), nsm, st);
+  if (p.tb <= 19) return lzp_launch(lz_persistent_f32_kernel<1, 20>, p, 1, 0, nsm, st);
+  if (p.tb <= LZP_WARPS - 1) return lzp_launch(lz_persistent_f32_kernel<1, LZP_WARPS>, p, 1, 0, nsm, st);
+  return false;
 }
 
 #define OVL_BAD_COMBO() note_bad_combo(__func__)

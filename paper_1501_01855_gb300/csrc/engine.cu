@@ -147,6 +147,11 @@ ovl_status ensure_lz(ovl_ctx* c, int nrhs, int cap) {
   // sized for the largest pole count (kernel deflation can change the count later)
   OVL_CUDA(c, cudaMalloc((void**)&c->lz_Y, sizeof(double) * (size_t)n * NPMAX * 2 * k));
   OVL_CUDA(c, cudaMalloc((void**)&c->lz_coefW, sizeof(double) * (size_t)n * k));
+  if (!c->lzp_bar) {
+    OVL_CUDA(c, cudaMalloc((void**)&c->lzp_bar, sizeof(unsigned int) * LZP_WORDS));
+    OVL_CUDA(c, cudaMalloc((void**)&c->lzp_part, sizeof(double) * 2 * LZP_SYS * LZP_BLOCKS));
+    OVL_CUDA(c, cudaDeviceGetAttribute(&c->nsm, cudaDevAttrMultiProcessorCount, c->device));
+  }
   c->lz_n = n;
   c->lz_cap = k;
   return OVL_OK;
@@ -645,8 +650,13 @@ static ovl_status sign_op_batch_lz(ovl_ctx* c, int mode, const Field& v, int vof
   prof_end(c, &pp, 0.0);
   OVL_TRY(check_launch(c, __func__));
 
+  // A small sign runs each cycle as one cooperative launch; a larger one, one with a forced launch
+  // shape, or one on a device that cannot hold its blocks, as cached graphs of kGraphIters steps.
+  bool persist = !c->prof.on && c->P.use_graphs && c->P.wilson_variant < 0 && n <= LZP_SYS;
+  unsigned int* hlzp = reinterpret_cast<unsigned int*>(c->hpin + 12288 + 4096);
   cudaGraphExec_t gexec = nullptr;
-  if (!c->prof.on && c->P.use_graphs) {
+  auto get_graph = [&]() -> ovl_status {
+    if (gexec || c->prof.on || !c->P.use_graphs) return OVL_OK;
     const std::vector<unsigned long long> key = {
         1000ull + (unsigned long long)PB, (unsigned long long)PL, (unsigned long long)n, (unsigned long long)hcap,
         (unsigned long long)(uintptr_t)W->data, (unsigned long long)(uintptr_t)t->data,
@@ -664,7 +674,8 @@ static ovl_status sign_op_batch_lz(ovl_ctx* c, int mode, const Field& v, int vof
         launch_wilson_lzL(PB, PL, PB, c->g, c->kappa, L, t->ref(), W->ref(), n, c->partials, gctl, cs);
       }
     }));
-  }
+    return OVL_OK;
+  };
   int* hflags = reinterpret_cast<int*>(c->hpin + 8192);
   int total = 0;
   long long live = 0, wreads = 0;
@@ -673,7 +684,18 @@ static ovl_status sign_op_batch_lz(ovl_ctx* c, int mode, const Field& v, int vof
   std::vector<int> it(n, 0), stt(n, 0);
   for (int cycle = 0;; ++cycle) {
     int chunk = 8;
-    while (true) {
+    if (persist) {
+      OVL_CUDA(c, cudaMemsetAsync(c->lzp_bar, 0, sizeof(unsigned int) * LZP_WORDS, c->st));
+      persist = launch_lz_persistent(PL, c->g, c->kappa, L, W->ref(), t->ref(), n, ctl, c->lzp_part, c->lzp_bar,
+                                     c->nsm, c->st);
+    }
+    if (persist) {
+      OVL_TRY(check_launch(c, __func__));
+      OVL_CUDA(c, cudaMemcpyAsync(hlzp, c->lzp_bar + 1, sizeof(unsigned int), cudaMemcpyDeviceToHost, c->st));
+    } else {
+      OVL_TRY(get_graph());
+    }
+    while (!persist) {
       if (gexec) {
         for (int k = 0; k < chunk; k += kGraphIters) OVL_CUDA(c, cudaGraphLaunch(gexec, c->st));
       } else {
@@ -705,6 +727,8 @@ static ovl_status sign_op_batch_lz(ovl_ctx* c, int mode, const Field& v, int vof
     OVL_CUDA(c, cudaMemcpy2DAsync(hflags, sizeof(int), &c->lz[0].j, sizeof(LzRhs), sizeof(int), n,
                                   cudaMemcpyDeviceToHost, c->st));
     OVL_CUDA(c, cudaStreamSynchronize(c->st));
+    if (persist && *hlzp)
+      return set_err(c, OVL_ETIMEOUT, "Lanczos iteration of the sign: a bounded wait between its blocks gave up");
     long long kk = 0;
     for (int j = 0; j < n; ++j) kk += hflags[j];
     const double cb = (double)kk * sbytes + (double)n * 2.0 * rbytes;

@@ -135,6 +135,16 @@ struct LzCtl {
   const Poles* poles;
   int pdl = 0;         // launch each step as a programmatic dependent of the one before (graphs)
 };
+// A whole cycle of the iteration in one cooperative launch, for launches too small to hide the
+// tail and the dispatch of two launches per step (see lzp_run in wilson.cuh). part: 2 nrhs
+// LZP_BLOCKS doubles; bar: LZP_WORDS zeroed words, word 1 of which is set when a bounded wait gave
+// up. False (nothing launched): this precision or size has no such form, or the device cannot hold
+// its blocks at once.
+constexpr int LZP_SYS = 4;         // systems
+constexpr int LZP_BLOCKS = 512;
+constexpr int LZP_WORDS = 2 + 2 * LZP_SYS;
+bool launch_lz_persistent(int prec, const Geom& g, double kappa, LinkRef links, SpinorRef W, SpinorRef t, int nrhs,
+                          const LzCtl& ctl, double* part, unsigned int* bar, int nsm, cudaStream_t st);
 void launch_wilson_lzK(int pw, int plink, int pt, const Geom& g, double kappa, LinkRef links, SpinorRef W,
                        SpinorRef t, int nrhs, double* partials, const LzCtl& ctl, cudaStream_t st);
 void launch_wilson_lzL(int pt, int plink, int pw, const Geom& g, double kappa, LinkRef links, SpinorRef t,
