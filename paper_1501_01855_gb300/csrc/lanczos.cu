@@ -329,7 +329,49 @@ __global__ void __launch_bounds__(128) lz_combine_df_kernel(SpinorRef W, SpinorR
   dfp_st(y, at, acc);
 }
 
-// Other precisions: whole spinors, accumulated in the compute type of y.
+// FP32 and FP64: the same, one thread per 16-byte chunk, which is contiguous over the whole field
+// (the spinor-at-a-time form below loaded one stored vector after the other: on a small lattice a
+// chain of one load latency per vector). FP32 sign on 10 x 6 x 14 x 12 588 -> 572 us, solve on
+// 16^3 x 32 287 -> 284 ms.
+__device__ __forceinline__ void axpy_word(float4& y, float c, const float4& w) {
+  y.x += c * w.x;
+  y.y += c * w.y;
+  y.z += c * w.z;
+  y.w += c * w.w;
+}
+__device__ __forceinline__ void axpy_word(double2& y, double c, const double2& w) {
+  y.x += c * w.x;
+  y.y += c * w.y;
+}
+template <typename W4, typename T>
+__global__ void __launch_bounds__(128) lz_combine_words_kernel(const W4* W, W4* y, const double* coefW, const LzRhs* lz,
+                                                               int cap, int nrhs, int words) {
+  extern __shared__ double cfd[];
+  T* cf = reinterpret_cast<T*>(cfd);
+  const int rhs = blockIdx.y;
+  const int k = lz[rhs].j;
+  if (k == 0) return;
+  for (int l = threadIdx.x; l < k; l += blockDim.x) cf[l] = (T)coefW[(size_t)rhs * cap + l];
+  __syncthreads();
+  const int e = blockIdx.x * blockDim.x + threadIdx.x;
+  if (e >= words) return;
+  const size_t slot = (size_t)nrhs * words;
+  const W4* p = W + (size_t)rhs * words + e;
+  W4* q = y + (size_t)rhs * words + e;
+  W4 acc = *q;
+  int l = 0;
+  for (; l + 8 <= k; l += 8) {
+    W4 w[8];
+#pragma unroll
+    for (int u = 0; u < 8; ++u) w[u] = __ldcs(p + (size_t)(l + u) * slot);
+#pragma unroll
+    for (int u = 0; u < 8; ++u) axpy_word(acc, cf[l + u], w[u]);
+  }
+  for (; l < k; ++l) axpy_word(acc, cf[l], __ldcs(p + (size_t)l * slot));
+  *q = acc;
+}
+
+// FP16 storage (a scale per site): whole spinors, accumulated in the compute type of y.
 template <int PW, int PY>
 __global__ void __launch_bounds__(256) lz_combine_kernel(SpinorRef W, SpinorRef y, const double* coefW,
                                                          const LzRhs* lz, int cap, int nrhs, int V, int ngr) {
@@ -360,12 +402,18 @@ void launch_lz_combine(int pw, int py, SpinorRef W, SpinorRef y, const double* c
     lz_combine_df_kernel<<<dim3(df_blocks(V) * 6, nrhs), 128, smem, st>>>(W, y, coefW, lz, cap, nrhs, V / 2, df_blocks(V));
     return;
   }
-#define LZC(A, B) lz_combine_kernel<A, B><<<sh.grid(), sh.block(), 0, st>>>(W, y, coefW, lz, cap, nrhs, V, sh.ngr)
-  if (pw == P64 && py == P64) LZC(P64, P64);
-  else if (pw == P32 && py == P32) LZC(P32, P32);
-  else if (pw == P16 && py == P32) LZC(P16, P32);
-  else note_bad_combo("lz_combine");
-#undef LZC
+  const size_t smem = sizeof(double) * (size_t)cap;
+  if (pw == P64 && py == P64) {
+    lz_combine_words_kernel<double2, double><<<dim3((12 * V + 127) / 128, nrhs), 128, smem, st>>>(
+        static_cast<const double2*>(W.data), static_cast<double2*>(y.data), coefW, lz, cap, nrhs, 12 * V);
+  } else if (pw == P32 && py == P32) {
+    lz_combine_words_kernel<float4, float><<<dim3((6 * V + 127) / 128, nrhs), 128, smem, st>>>(
+        static_cast<const float4*>(W.data), static_cast<float4*>(y.data), coefW, lz, cap, nrhs, 6 * V);
+  } else if (pw == P16 && py == P32) {
+    lz_combine_kernel<P16, P32><<<sh.grid(), sh.block(), 0, st>>>(W, y, coefW, lz, cap, nrhs, V, sh.ngr);
+  } else {
+    note_bad_combo("lz_combine");
+  }
 }
 
 }  // namespace ovl
