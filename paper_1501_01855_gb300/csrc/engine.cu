@@ -677,6 +677,8 @@ static ovl_status sign_op_batch_lz(ovl_ctx* c, int mode, const Field& v, int vof
     return OVL_OK;
   };
   int* hflags = reinterpret_cast<int*>(c->hpin + 8192);
+  LzState* hs = reinterpret_cast<LzState*>(c->hpin + 8192 + 512);   // n <= 256 systems, after their flags
+  static_assert(sizeof(LzState) * 256 <= sizeof(double) * (4096 - 512), "the states fit the staging area");
   int total = 0;
   long long live = 0, wreads = 0;
   int itmax = 0;
@@ -723,28 +725,23 @@ static ovl_status sign_op_batch_lz(ovl_ctx* c, int mode, const Field& v, int vof
     prof_begin(c, 5, &pp);
     launch_lz_coef(c->lz, ahist, bhist, hcap, c->dpoles, c->lz_Y, c->lz_coefW, n, c->st);
     prof_end(c, &pp, 0.0);
-    // steps of this cycle per system (the basis vectors the combine reads)
-    OVL_CUDA(c, cudaMemcpy2DAsync(hflags, sizeof(int), &c->lz[0].j, sizeof(LzRhs), sizeof(int), n,
-                                  cudaMemcpyDeviceToHost, c->st));
+    prof_begin(c, 3, &pp);
+    launch_lz_combine(PB, PR, W->ref(), y->ref(), c->lz_coefW, c->lz, hcap, n, V, c->st);
+    prof_end(c, &pp, 0.0);
+    OVL_TRY(check_launch(c, __func__));
+    OVL_CUDA(c, cudaMemcpy2DAsync(hs, sizeof(LzState), c->lz, sizeof(LzRhs), sizeof(LzState), n, cudaMemcpyDeviceToHost,
+                                  c->st));
     OVL_CUDA(c, cudaStreamSynchronize(c->st));
     if (persist && *hlzp)
       return set_err(c, OVL_ETIMEOUT, "Lanczos iteration of the sign: a bounded wait between its blocks gave up");
-    long long kk = 0;
-    for (int j = 0; j < n; ++j) kk += hflags[j];
-    const double cb = (double)kk * sbytes + (double)n * 2.0 * rbytes;
-    comb_bytes += cb;
-    prof_begin(c, 3, &pp);
-    launch_lz_combine(PB, PR, W->ref(), y->ref(), c->lz_coefW, c->lz, hcap, n, V, c->st);
-    prof_end(c, &pp, cb);
-    OVL_TRY(check_launch(c, __func__));
-    // cycles that filled up continue from their last basis vector
-    OVL_CUDA(c, cudaMemcpy2DAsync(hflags, sizeof(int), &c->lz[0].status, sizeof(LzRhs), sizeof(int), n,
-                                  cudaMemcpyDeviceToHost, c->st));
-    OVL_CUDA(c, cudaMemcpy2DAsync(hflags + 4096, sizeof(int), &c->lz[0].finished, sizeof(LzRhs), sizeof(int), n,
-                                  cudaMemcpyDeviceToHost, c->st));
-    OVL_CUDA(c, cudaStreamSynchronize(c->st));
     bool more = false;
-    for (int j = 0; j < n; ++j) more = more || (hflags[j] == 3 && !hflags[4096 + j]);
+    double cb = (double)n * 2.0 * rbytes;   // y, and the basis vectors of this cycle per system
+    for (int j = 0; j < n; ++j) {
+      cb += (double)hs[j].j * sbytes;
+      more = more || (hs[j].status == 3 && !hs[j].finished);   // a cycle that filled up goes on from its last vector
+    }
+    comb_bytes += cb;
+    if (c->prof.on) c->prof.bytes[3] += cb;
     if (!more) break;
     prof_begin(c, 4, &pp);
     launch_lz_restart(PB, W->ref(), c->lz, n, V, c->partials, c->st);
@@ -762,19 +759,11 @@ static ovl_status sign_op_batch_lz(ovl_ctx* c, int mode, const Field& v, int vof
   prof_end(c, &pp, (double)n * V * (spinor_bytes(PR) + 2.0 * spinor_bytes(out.prec)) + lbytes);
   OVL_TRY(check_launch(c, __func__));
   if (dot_w) OVL_TRY(reduce_to_host_nv(c, sh.nsb, n, dots, 4));
-  long long* hll = reinterpret_cast<long long*>(c->hpin + 12288);
-  OVL_CUDA(c, cudaMemcpy2DAsync(hflags, sizeof(int), &c->lz[0].total, sizeof(LzRhs), sizeof(int), n,
-                                cudaMemcpyDeviceToHost, c->st));
-  OVL_CUDA(c, cudaMemcpy2DAsync(hflags + 4096, sizeof(int), &c->lz[0].status, sizeof(LzRhs), sizeof(int), n,
-                                cudaMemcpyDeviceToHost, c->st));
-  OVL_CUDA(c, cudaMemcpy2DAsync(hll, sizeof(long long), &c->lz[0].w_reads, sizeof(LzRhs), sizeof(long long), n,
-                                cudaMemcpyDeviceToHost, c->st));
-  OVL_CUDA(c, cudaStreamSynchronize(c->st));
   for (int j = 0; j < n; ++j) {
-    it[j] = hflags[j];
-    stt[j] = hflags[4096 + j];
+    it[j] = hs[j].total;
+    stt[j] = hs[j].status;
     live += it[j];
-    wreads += hll[j];
+    wreads += hs[j].w_reads;
     itmax = std::max(itmax, it[j]);
   }
   c->wcalls[PL] += 2 * live + n;

@@ -53,15 +53,7 @@ struct MsRhs {
 // tridiagonal solve and one combination of the stored vectors, with no per-pole vector
 // traffic. One cycle holds at most `cap` basis vectors; a cycle that fills up restarts
 // from the last vector, to which every pole's residual is parallel.
-struct LzRhs {
-  double vnorm;        // n_0 = ||W_0|| of this cycle
-  double inv_n;        // 1 / n_j: K-mode scale of the current basis vector
-  double inv_nprev;    // 1 / n_{j-1}
-  double a, b;         // L-mode coefficients alpha_j / n_j and beta_{j-1} / n_{j-1}
-  double alpha;        // alpha_j = (v_j, K^2 v_j)
-  double beta_prev;    // beta_{j-1}
-  double thr;          // error budget eta ||v|| of the caller's vector
-  double err;          // current error bound sum_i |w_i| g_i rho_i
+struct LzState {       // what the host reads after a cycle
   int j;               // basis vectors completed in this cycle (next K-mode input W_j)
   int done;            // 1: this cycle has stopped
   int status;          // 0 converged, 1 iteration limit, 2 breakdown, 3 cycle full (restart)
@@ -71,6 +63,16 @@ struct LzRhs {
   int cycles;
   int even;            // 1: stop when every pole is within thr / N_Z (relaxed signs of relCG)
   long long w_reads;   // basis vector passes of the L mode (bytes accounting)
+};
+struct LzRhs : LzState {
+  double vnorm;        // n_0 = ||W_0|| of this cycle
+  double inv_n;        // 1 / n_j: K-mode scale of the current basis vector
+  double inv_nprev;    // 1 / n_{j-1}
+  double a, b;         // L-mode coefficients alpha_j / n_j and beta_{j-1} / n_{j-1}
+  double alpha;        // alpha_j = (v_j, K^2 v_j)
+  double beta_prev;    // beta_{j-1}
+  double thr;          // error budget eta ||v|| of the caller's vector
+  double err;          // current error bound sum_i |w_i| g_i rho_i
   double w[NPMAX];     // pole weights of this cycle (omega_i in the first)
   float2 fn, fa, fb;   // inv_n, a, b as hi + lo of two floats (.x is the float nearest to each)
   double rd[NPMAX];    // reciprocals of the LDL^T pivots of T_j + sigma_i
