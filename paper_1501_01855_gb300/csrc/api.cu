@@ -566,8 +566,16 @@ extern "C" ovl_status ovl_wilson_apply(ovl_ctx* c, const void* in, void* out, in
   if (prec < P64 || prec > P64E) return set_err(c, OVL_EINVAL, "prec must be OVL_PREC_F64, F32, F16 or F64E");
   Field *fi, *fo;
   OVL_TRY(get_field(c, "api_wi", prec, n, &fi));
-  OVL_TRY(get_field(c, "api_wo", prec, n, &fo));
   OVL_TRY(import_spinors(c, in, dtype, on_device, n, *fi, 0));
+  // FP32 into a caller's single-precision buffer: one launch (every input has been read by then)
+  if (prec == P32 && dtype == OVL_C64 && on_device && !c->prof.on &&
+      launch_wilson_K_canon32(c->g, c->kappa, links_of(c, P32), fi->ref(), (float*)out, n, c->st)) {
+    OVL_TRY(check_launch(c, __func__));
+    c->wcalls[P32] += n;
+    OVL_CUDA(c, cudaStreamSynchronize(c->st));
+    return OVL_OK;
+  }
+  OVL_TRY(get_field(c, "api_wo", prec, n, &fo));
   OVL_TRY(wilson_apply_field(c, prec, *fi, 0, *fo, 0, n));
   OVL_TRY(export_spinors(c, out, dtype, on_device, n, *fo, 0));
   OVL_CUDA(c, cudaStreamSynchronize(c->st));

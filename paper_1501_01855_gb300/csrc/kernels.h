@@ -108,6 +108,10 @@ int wilson_df_variant(int V, int nrhs);
 void launch_wilson_K(int pin, int plink, int pout, const Geom& g, double kappa, LinkRef links,
                      SpinorRef in, SpinorRef out, int nrhs, double* partials, const MsRhs* ms,
                      cudaStream_t st);
+// K in FP32 into the caller's canonical single-precision spinors; false (nothing launched) where
+// the launch shape or the alignment of the buffer asks for K and the unpacking apart.
+bool launch_wilson_K_canon32(const Geom& g, double kappa, LinkRef links, SpinorRef in, float* canon, int nrhs,
+                             cudaStream_t st);
 // Multi-shift CG second half: Ap = K in + sigma0 p;  r -= alpha Ap; partials {||r||^2}.
 void launch_wilson_mscg_r(int pt, int plink, int pr, int pp, const Geom& g, double kappa, LinkRef links,
                           SpinorRef t, SpinorRef p0, SpinorRef r, int nrhs, double sigma0,
