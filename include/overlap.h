@@ -145,9 +145,10 @@ ovl_status ovl_params_default(ovl_params* p);
  *   ctx       receives the new context (caller frees it with overlap_destroy).
  *   dims[4]   {Lx, Ly, Lz, Lt}, each even and >= 2.
  *   links     host, canonical layout, complex128, 4*9*V entries; copied (the caller
- *             keeps ownership) into the library's device layouts: 12-real FP64 / FP32 /
- *             FP16 copies (row 3 of every SU(3) link rebuilt as conj(row1 x row2) in
- *             registers) and an 18-real double-float copy with one slot per hop.
+ *             keeps ownership) into the library's device layouts: 12-real FP32 / FP16
+ *             copies (row 3 of every SU(3) link rebuilt as conj(row1 x row2) in
+ *             registers), an FP64 copy that stores that row 3 as well, and an 18-real
+ *             double-float copy with one slot per hop.
  *   m0        Wilson mass, kappa = 1/(8 - 2 m0) (Sec. 1).
  *   mu        default overlap mass parameter of D(mu) (Sec. 1).
  *   n_poles   Zolotarev order N_Z (Sec. 3), 1..64.

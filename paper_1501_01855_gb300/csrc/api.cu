@@ -68,12 +68,12 @@ extern "C" ovl_status ovl_trim(ovl_ctx* c) {
 static void convert_links(const double* links, const int L[4], int bc_t, std::vector<double>& l64,
                           std::vector<float>& l32, std::vector<__half>& l16, std::vector<float>& l64e) {
   const int V = L[0] * L[1] * L[2] * L[3];
-  // canonical [site][mu][row][col] complex -> [mu][chunk][V] keeping rows 0, 1.
+  // canonical [site][mu][row][col] complex -> [mu][chunk][V], FP32 and FP16 keeping rows 0, 1.
   // The double-float copy holds, for each site x, the matrix of each of the eight hops
   // in slot n = 2 mu + b: b = 0 U_mu(x), b = 1 U_mu(x - mu)^dag, all 9 entries, in the
   // pair layout ([i / 32][n][2 e + r][i % 32] of (hi, hi', lo, lo') for the sites i, i + V/2), with
   // the antiperiodic-t sign of the hops that cross the boundary folded in.
-  l64.assign((size_t)4 * 6 * V * 2, 0.0);
+  l64.assign((size_t)4 * 9 * V * 2, 0.0);
   l32.assign((size_t)4 * 3 * V * 4, 0.f);
   l16.assign((size_t)4 * 3 * V * 4, __float2half(0.f));
   l64e.assign((size_t)df_blocks(V) * 8 * 18 * 32 * 4, 0.f);
@@ -107,13 +107,19 @@ static void convert_links(const double* links, const int L[4], int bc_t, std::ve
       }
       for (int e = 0; e < 6; ++e) {
         const double re = u[2 * e], im = u[2 * e + 1];
-        l64[(((size_t)mu * 6 + e) * V + s) * 2 + 0] = re;
-        l64[(((size_t)mu * 6 + e) * V + s) * 2 + 1] = im;
+        l64[(((size_t)mu * 9 + e) * V + s) * 2 + 0] = re;
+        l64[(((size_t)mu * 9 + e) * V + s) * 2 + 1] = im;
         const int ch = e / 2, w = e % 2;
         l32[(((size_t)mu * 3 + ch) * V + s) * 4 + 2 * w + 0] = (float)re;
         l32[(((size_t)mu * 3 + ch) * V + s) * 4 + 2 * w + 1] = (float)im;
         l16[(((size_t)mu * 3 + ch) * V + s) * 4 + 2 * w + 0] = __float2half_rn((float)re);
         l16[(((size_t)mu * 3 + ch) * V + s) * 4 + 2 * w + 1] = __float2half_rn((float)im);
+      }
+      for (int e = 6; e < 9; ++e) {   // row 3 = conj(row 1 x row 2), as the kernels rebuild it
+        const double *a = u + 2 * ((e - 5) % 3), *b = u + 2 * ((e - 4) % 3);
+        double* d = &l64[(((size_t)mu * 9 + e) * V + s) * 2];
+        d[0] = a[0] * b[6] - a[1] * b[7] - (b[0] * a[6] - b[1] * a[7]);
+        d[1] = -(a[0] * b[7] + a[1] * b[6] - (b[0] * a[7] + b[1] * a[6]));
       }
     }
   }

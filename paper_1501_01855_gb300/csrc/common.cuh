@@ -18,9 +18,11 @@
 //         float scale per site (components stored as value / max|component|)
 // A batch of n spinors is n such fields back to back.
 //
-// Links keep only rows 1 and 2 of each SU(3) matrix (12 reals); row 3 is
+// F32 and F16 links keep only rows 1 and 2 of each SU(3) matrix (12 reals); row 3 is
 // rebuilt in registers as conj(row1 x row2). Layout [mu][chunk][V]:
-//   F64: 6 chunks double2, F32: 3 chunks float4, F16: 3 chunks of 4 halves.
+//   F32: 3 chunks float4, F16: 3 chunks of 4 halves, F64: 9 chunks double2 (every entry, row 3
+// from the same formula: the FP64 kernel is bound by its arithmetic, not by bytes, and
+// rebuilding the row was a sixth of it).
 // F64E links: eight slots per site, one per hop (slot n = 2 mu + b holds U_mu(x) for b = 0 and
 // U_mu(x - mu)^dag for b = 1, with the antiperiodic sign folded in), all 9 entries, in pairs
 // of sites like the spinors: [i / 32][n][2 e + r][i % 32] float4. The double-float kernel is bound by
@@ -106,6 +108,15 @@ template <typename T> __host__ __device__ __forceinline__ cpx<T> operator*(cpx<T
   return {a.r * b.r - a.i * b.i, a.r * b.i + a.i * b.r};
 }
 template <typename T> __host__ __device__ __forceinline__ cpx<T> operator*(T s, cpx<T> a) { return {s * a.r, s * a.i}; }
+// t += a b, t += conj(a) b: four multiply-adds
+template <typename T> __device__ __forceinline__ void cmac(cpx<T>& t, cpx<T> a, cpx<T> b) {
+  t.r = fma(-a.i, b.i, fma(a.r, b.r, t.r));
+  t.i = fma(a.i, b.r, fma(a.r, b.i, t.i));
+}
+template <typename T> __device__ __forceinline__ void cmacc(cpx<T>& t, cpx<T> a, cpx<T> b) {
+  t.r = fma(a.i, b.i, fma(a.r, b.r, t.r));
+  t.i = fma(-a.i, b.r, fma(a.r, b.i, t.i));
+}
 // conj(a) * b
 template <typename T> __host__ __device__ __forceinline__ cpx<T> cmulc(cpx<T> a, cpx<T> b) {
   return {a.r * b.r + a.i * b.i, a.r * b.i - a.i * b.r};
@@ -308,21 +319,26 @@ struct LinkRef {
   int variant_multi; // the variant chosen for launches of 4 or more systems
 };
 
+// row 3 = conj(row 1 x row 2)
 template <typename T>
 __device__ __forceinline__ void reconstruct_row3(cpx<T> u[9]) {
-  // row3 = conj(row1 x row2)
-  u[6] = conj(u[1] * u[5] - u[2] * u[4]);
-  u[7] = conj(u[2] * u[3] - u[0] * u[5]);
-  u[8] = conj(u[0] * u[4] - u[1] * u[3]);
+  auto minor = [](cpx<T> a, cpx<T> b, cpx<T> c, cpx<T> d) {   // conj(a b - c d)
+    cpx<T> t = a * b;
+    cmac(t, -c, d);
+    return conj(t);
+  };
+  u[6] = minor(u[1], u[5], u[2], u[4]);
+  u[7] = minor(u[2], u[3], u[0], u[5]);
+  u[8] = minor(u[0], u[4], u[1], u[3]);
 }
 
 template <int P> struct LinkIO;
 template <>
 struct LinkIO<P64> {
   static __device__ __forceinline__ void load(const LinkRef& L, int mu, int s, cpx<double> u[9]) {
-    const double2* p = reinterpret_cast<const double2*>(L.data) + (size_t)mu * 6 * L.V + s;
+    const double2* p = reinterpret_cast<const double2*>(L.data) + (size_t)mu * 9 * L.V + s;
 #pragma unroll
-    for (int c = 0; c < 6; ++c) {
+    for (int c = 0; c < 9; ++c) {
       double2 w = __ldg(p + (size_t)c * L.V);
       u[c] = cmk(w.x, w.y);
     }
@@ -360,7 +376,7 @@ template <int P, typename T>
 __device__ __forceinline__ void load_link(const LinkRef& L, int mu, int s, cpx<T> u[9]) {
   static_assert(std::is_same<T, typename Real<P>::T>::value, "links load in their own compute type");
   LinkIO<P>::load(L, mu, s, u);
-  reconstruct_row3(u);
+  if constexpr (P != P64) reconstruct_row3(u);
 }
 
 // ------------------------------------------------------------------ geometry

@@ -62,7 +62,7 @@ struct ovl_ctx {
   ovl_params P;
   cudaStream_t st = nullptr;
   int device = 0;
-  void* link[4] = {nullptr, nullptr, nullptr, nullptr};  // P64, P32, P16, P64E 12-real layouts
+  void* link[4] = {nullptr, nullptr, nullptr, nullptr};  // P64, P32, P16, P64E layouts
   int wvar[4] = {0, 0, 0, 0};                            // Wilson-kernel variant per precision
   float wtime[4][4] = {{0}};                             // autotuner timings (ms per launch)
   int wvar_multi[4] = {0, 0, 0, 0};                      // the same for launches of >= 4 systems

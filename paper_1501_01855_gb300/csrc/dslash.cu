@@ -6,7 +6,7 @@
 // One thread per (site, system). (1 -+ gamma_mu) has rank 2, so each neighbour is
 // projected to a half spinor (2 spins x 3 colours), multiplied by the link and
 // expanded again; the spin algebra below is the DeGrand-Rossi chiral basis,
-// gamma5 = diag(1, 1, -1, -1). FP64 / FP32 / FP16 links are 12-real (row 3 rebuilt in
+// gamma5 = diag(1, 1, -1, -1). FP32 and FP16 links are 12-real (row 3 rebuilt in
 // registers) and the eight neighbours are unrolled; the double-float kernel is in
 // dfwilson.cu. Threads of one block that share a site but belong to different
 // systems read the same links, so the link bytes of a multi-system launch come from L1
@@ -96,21 +96,66 @@ __device__ __forceinline__ void accumulate(cpx<T> acc[12], const cpx<T> w[6]) {
   }
 }
 
+// Both hops of a direction: upper spins + (wf + wb), lower spins + the S = +1 expansion of
+// wb - wf; p = wf + wb comes out of the backward product's chain of multiply-adds, wb - wf = p - 2 wf.
+// FIRST: nothing accumulated yet.
+template <int MU, bool FIRST, typename T>
+__device__ __forceinline__ void accumulate_pair(cpx<T> acc[12], const cpx<T> p[6], const cpx<T> wf[6]) {
+  cpx<T> low[6];
+#pragma unroll
+  for (int c = 0; c < 3; ++c) {
+    const cpx<T> m0 = {fma(T(-2), wf[c].r, p[c].r), fma(T(-2), wf[c].i, p[c].i)};
+    const cpx<T> m1 = {fma(T(-2), wf[3 + c].r, p[3 + c].r), fma(T(-2), wf[3 + c].i, p[3 + c].i)};
+    low[c] = MU == 0 ? timesMinusI(m1) : MU == 1 ? m1 : MU == 2 ? timesMinusI(m0) : m0;
+    low[3 + c] = MU == 0 ? timesMinusI(m0) : MU == 1 ? -m0 : MU == 2 ? timesI(m1) : m1;
+  }
+#pragma unroll
+  for (int k = 0; k < 6; ++k) {
+    acc[k] = FIRST ? p[k] : acc[k] + p[k];
+    acc[6 + k] = FIRST ? low[k] : acc[6 + k] + low[k];
+  }
+}
+
+// Sums of products as one chain of multiply-adds: written as a sum of complex products every
+// product ended in an addition of its own (8 instead of 6 operations per real number). FP32 signs
+// 21.3 -> 20.2 ms (16^3 x 32, 12 systems), 2.08 -> 1.89 ms (one).
 template <typename T>
 __device__ __forceinline__ void su3_mul(const cpx<T> u[9], const cpx<T> h[6], cpx<T> w[6]) {
 #pragma unroll
   for (int sp = 0; sp < 2; ++sp)
 #pragma unroll
-    for (int a = 0; a < 3; ++a)
-      w[3 * sp + a] = u[3 * a] * h[3 * sp] + u[3 * a + 1] * h[3 * sp + 1] + u[3 * a + 2] * h[3 * sp + 2];
+    for (int a = 0; a < 3; ++a) {
+      cpx<T> t = u[3 * a] * h[3 * sp];
+      cmac(t, u[3 * a + 1], h[3 * sp + 1]);
+      cmac(t, u[3 * a + 2], h[3 * sp + 2]);
+      w[3 * sp + a] = t;
+    }
 }
 template <typename T>
 __device__ __forceinline__ void su3_dag_mul(const cpx<T> u[9], const cpx<T> h[6], cpx<T> w[6]) {
 #pragma unroll
   for (int sp = 0; sp < 2; ++sp)
 #pragma unroll
-    for (int a = 0; a < 3; ++a)
-      w[3 * sp + a] = cmulc(u[a], h[3 * sp]) + cmulc(u[3 + a], h[3 * sp + 1]) + cmulc(u[6 + a], h[3 * sp + 2]);
+    for (int a = 0; a < 3; ++a) {
+      cpx<T> t = cmulc(u[a], h[3 * sp]);
+      cmacc(t, u[3 + a], h[3 * sp + 1]);
+      cmacc(t, u[6 + a], h[3 * sp + 2]);
+      w[3 * sp + a] = t;
+    }
+}
+
+// p = wf + U^dag h
+template <typename T>
+__device__ __forceinline__ void su3_dag_mul_add(const cpx<T> u[9], const cpx<T> h[6], const cpx<T> wf[6], cpx<T> p[6]) {
+#pragma unroll
+  for (int sp = 0; sp < 2; ++sp)
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+      cpx<T> t = wf[3 * sp + a];
+#pragma unroll
+      for (int b = 0; b < 3; ++b) cmacc(t, u[3 * b + a], h[3 * sp + b]);
+      p[3 * sp + a] = t;
+    }
 }
 
 // Per-thread sums for the epilogue reductions, kept in the compute type: GB300 runs
@@ -128,9 +173,14 @@ __device__ __forceinline__ void acc_norm(Acc<T>& a, const cpx<T>& z) {
   a.add(z.i, z.i);
 }
 
-template <int MU, int PIN, int PL, bool RO, typename T>
+// FP64 takes the two hops of a direction together (accumulate_pair): that kernel is bound by FP64
+// operations, 840 per site instead of 912 (12 systems of 16^3 x 32 2.82 -> 2.60 ms). For FP32 the
+// registers it holds across the second product cost more than the additions it saves (12-system
+// sign 20.2 -> 20.7 ms). FIRST: this hop starts the sum (saves 24 additions).
+template <int MU, int PIN, int PL, bool RO, typename T, bool FIRST = false>
 __device__ __forceinline__ void hop_dir(const Geom& g, const LinkRef& L, const SpinorRef& in, int rhs, int s,
                                         const int x[4], int stride, cpx<T> acc[12]) {
+  constexpr bool PAIRED = std::is_same<T, double>::value;
   cpx<T> psi[12], h[6], w[6], u[9];
   // forward neighbour: (1 - gamma_mu) U_mu(x) psi(x + mu)
   {
@@ -144,7 +194,18 @@ __device__ __forceinline__ void hop_dir(const Geom& g, const LinkRef& L, const S
     }
     load_link<PL, T>(L, MU, s, u);
     su3_mul(u, h, w);
-    accumulate<MU, -1>(acc, w);
+    if constexpr (FIRST && !PAIRED) {
+      static_assert(MU == 0, "the first direction");
+#pragma unroll
+      for (int k = 0; k < 6; ++k) acc[k] = w[k];
+#pragma unroll
+      for (int c = 0; c < 3; ++c) {
+        acc[6 + c] = timesI(w[3 + c]);
+        acc[9 + c] = timesI(w[c]);
+      }
+    } else if constexpr (!PAIRED) {
+      accumulate<MU, -1>(acc, w);
+    }
   }
   // backward neighbour: (1 + gamma_mu) U_mu(x - mu)^dag psi(x - mu)
   {
@@ -157,8 +218,14 @@ __device__ __forceinline__ void hop_dir(const Geom& g, const LinkRef& L, const S
       for (int k = 0; k < 6; ++k) h[k] = -h[k];
     }
     load_link<PL, T>(L, MU, sb, u);
-    su3_dag_mul(u, h, w);
-    accumulate<MU, +1>(acc, w);
+    if constexpr (PAIRED) {
+      cpx<T> p[6];
+      su3_dag_mul_add(u, h, w, p);
+      accumulate_pair<MU, MU == 0>(acc, p, w);
+    } else {
+      su3_dag_mul(u, h, w);
+      accumulate<MU, +1>(acc, w);
+    }
   }
 }
 
@@ -526,7 +593,7 @@ struct LzpBody32 {
     site_coords(a.g, s, x);
     const int sy = a.g.L[0], sz = sy * a.g.L[1], st = sz * a.g.L[2];
     const int dir = NS == 1 ? -1 : (threadIdx.x >> 5) % NS;
-    if (NS == 1 || dir == 0) hop_dir<0, P32, P32, false, float>(a.g, a.links, in, fin, s, x, 1, acc);
+    if (NS == 1 || dir == 0) hop_dir<0, P32, P32, false, float, true>(a.g, a.links, in, fin, s, x, 1, acc);
     if (NS == 1 || dir == 1) hop_dir<1, P32, P32, false, float>(a.g, a.links, in, fin, s, x, sy, acc);
     if (NS == 1 || dir == 2) hop_dir<2, P32, P32, false, float>(a.g, a.links, in, fin, s, x, sz, acc);
     if (NS == 1 || dir == 3) hop_dir<3, P32, P32, false, float>(a.g, a.links, in, fin, s, x, st, acc);
