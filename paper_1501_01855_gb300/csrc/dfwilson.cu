@@ -465,7 +465,7 @@ struct LzpBodyDf {
         hop_pair<(G >= 4)>(pair_at(in, fblk, h.nbr), link_at(a.links, i, n), half, h, up, low);
         h = nx;
       }
-      if (n == min(n1 - 1, 3)) {   // as in df_wilson_kernel: the same for a warp, or for G = 8 its two hops
+      if (n == min(n1 - 1, 3)) {   // as in df_wilson_kernel; with P = 8 both groups of a warp come here in the same turn
 #pragma unroll
         for (int c = 0; c < 3; ++c)
 #pragma unroll
@@ -541,12 +541,15 @@ bool lzp_df(LzPersist& p, int nsm, cudaStream_t st) {
 
 }  // namespace
 
-// Eight groups on 8 pairs while the SMs hold every tile at 96 registers or more (9728 sites x
-// systems on 152 SMs; 80 registers spill: 8^3 x 16 2.2 instead of 2.1 ms), two groups on 16 pairs up
-// to 34048.
+// A phase is mostly the latency of the hops that a thread takes one after the other: eight groups on
+// 8 pairs while the SMs hold every tile at 96 registers or more (9728 sites x systems on 152 SMs; 80
+// registers spill: 8^3 x 16 2.2 instead of 2.1 ms), four groups on 8 pairs up to 21888 (9 tiles at 96
+// registers), two on 16 pairs up to 34048. Sign to 1e-10 with four / two groups, ms: 10080 sites 2.60 /
+// 3.82, 12288 2.62 / 3.68, 16384 2.99 / 3.87, 20000 3.92 / 4.15, 20480 3.95 / 4.05. Requesting the
+// epilogue's operands before the hops made every size slower (4^4 1.35 -> 1.39 ms).
 bool launch_lz_persistent_df(LzPersist& p, int nsm, cudaStream_t st) {
-  return lzp_df<8, 8, 3>(p, nsm, st) || lzp_df<8, 8, 4>(p, nsm, st) || lzp_df<2, 16, 5>(p, nsm, st) ||
-         lzp_df<2, 16, 7>(p, nsm, st);
+  return lzp_df<8, 8, 3>(p, nsm, st) || lzp_df<8, 8, 4>(p, nsm, st) || lzp_df<4, 8, 7>(p, nsm, st) ||
+         lzp_df<4, 8, 9>(p, nsm, st) || lzp_df<2, 16, 5>(p, nsm, st) || lzp_df<2, 16, 7>(p, nsm, st);
 }
 
 // Two threads per pair and system, times 1, 2, 4 or 8 groups. One group is the cheapest form

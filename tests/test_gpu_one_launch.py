@@ -64,3 +64,18 @@ def test_one_launch_iteration_limit_is_reported(prec):
     assert e.value.status == B.OVL_ENOCONV
     o = np.zeros_like(v)
     c.sign_apply(v, o, eta=0.5, prec=prec)     # the context stays usable
+
+
+@pytest.mark.parametrize("dims,n", [((10, 6, 14, 12), 1), ((6, 10, 14, 4), 4), ((10, 10, 10, 20), 1)])
+def test_one_launch_four_groups(dims, n):
+    """Double-float tiles of 8 pairs in four groups: up to 7 and up to 9 tiles per SM."""
+    eta = 1e-9
+    v = synth.gaussian_source(dims, 85, nvec=n)
+    outs = []
+    for c in _pair(dims):
+        o = np.zeros_like(v)
+        c.sign_apply(v, o, eta=eta, prec=3)
+        outs.append(o)
+        c.close()
+    for j in range(n):
+        assert rel(outs[0][j], outs[1][j]) <= 2 * eta
