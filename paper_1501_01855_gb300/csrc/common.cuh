@@ -108,14 +108,10 @@ template <typename T> __host__ __device__ __forceinline__ cpx<T> operator*(cpx<T
   return {a.r * b.r - a.i * b.i, a.r * b.i + a.i * b.r};
 }
 template <typename T> __host__ __device__ __forceinline__ cpx<T> operator*(T s, cpx<T> a) { return {s * a.r, s * a.i}; }
-// t += a b, t += conj(a) b: four multiply-adds
+// t += a b: four multiply-adds
 template <typename T> __device__ __forceinline__ void cmac(cpx<T>& t, cpx<T> a, cpx<T> b) {
   t.r = fma(-a.i, b.i, fma(a.r, b.r, t.r));
   t.i = fma(a.i, b.r, fma(a.r, b.i, t.i));
-}
-template <typename T> __device__ __forceinline__ void cmacc(cpx<T>& t, cpx<T> a, cpx<T> b) {
-  t.r = fma(a.i, b.i, fma(a.r, b.r, t.r));
-  t.i = fma(-a.i, b.r, fma(a.r, b.i, t.i));
 }
 // conj(a) * b
 template <typename T> __host__ __device__ __forceinline__ cpx<T> cmulc(cpx<T> a, cpx<T> b) {

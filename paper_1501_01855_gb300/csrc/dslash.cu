@@ -96,66 +96,31 @@ __device__ __forceinline__ void accumulate(cpx<T> acc[12], const cpx<T> w[6]) {
   }
 }
 
-// Both hops of a direction: upper spins + (wf + wb), lower spins + the S = +1 expansion of
-// wb - wf; p = wf + wb comes out of the backward product's chain of multiply-adds, wb - wf = p - 2 wf.
-// FIRST: nothing accumulated yet.
-template <int MU, bool FIRST, typename T>
-__device__ __forceinline__ void accumulate_pair(cpx<T> acc[12], const cpx<T> p[6], const cpx<T> wf[6]) {
-  cpx<T> low[6];
-#pragma unroll
-  for (int c = 0; c < 3; ++c) {
-    const cpx<T> m0 = {fma(T(-2), wf[c].r, p[c].r), fma(T(-2), wf[c].i, p[c].i)};
-    const cpx<T> m1 = {fma(T(-2), wf[3 + c].r, p[3 + c].r), fma(T(-2), wf[3 + c].i, p[3 + c].i)};
-    low[c] = MU == 0 ? timesMinusI(m1) : MU == 1 ? m1 : MU == 2 ? timesMinusI(m0) : m0;
-    low[3 + c] = MU == 0 ? timesMinusI(m0) : MU == 1 ? -m0 : MU == 2 ? timesI(m1) : m1;
-  }
-#pragma unroll
-  for (int k = 0; k < 6; ++k) {
-    acc[k] = FIRST ? p[k] : acc[k] + p[k];
-    acc[6 + k] = FIRST ? low[k] : acc[6 + k] + low[k];
-  }
+// The six products of a real number as two chains of multiply-adds of three and their sum: 7
+// operations (a sum of three complex products takes 8) with partial sums no larger than there; one
+// chain of six takes 6 but rounds larger partial sums, and its error against 64 bits was
+// larger than before (FP64 K 1.5e-16 against 1.4e-16). S = +1: a b, -1: conj(a) b.
+template <int S, typename T>
+__device__ __forceinline__ cpx<T> dot3(cpx<T> a0, cpx<T> b0, cpx<T> a1, cpx<T> b1, cpx<T> a2, cpx<T> b2) {
+  const T i0 = S > 0 ? a0.i : -a0.i, i1 = S > 0 ? a1.i : -a1.i, i2 = S > 0 ? a2.i : -a2.i;
+  return {fma(a1.r, b1.r, fma(-i0, b0.i, a0.r * b0.r)) + fma(-i2, b2.i, fma(a2.r, b2.r, -i1 * b1.i)),
+          fma(a1.r, b1.i, fma(i0, b0.r, a0.r * b0.i)) + fma(i2, b2.r, fma(a2.r, b2.i, i1 * b1.r))};
 }
-
-// Sums of products as one chain of multiply-adds: written as a sum of complex products every
-// product ended in an addition of its own (8 instead of 6 operations per real number). FP32 signs
-// 21.3 -> 20.2 ms (16^3 x 32, 12 systems), 2.08 -> 1.89 ms (one).
 template <typename T>
 __device__ __forceinline__ void su3_mul(const cpx<T> u[9], const cpx<T> h[6], cpx<T> w[6]) {
 #pragma unroll
   for (int sp = 0; sp < 2; ++sp)
 #pragma unroll
-    for (int a = 0; a < 3; ++a) {
-      cpx<T> t = u[3 * a] * h[3 * sp];
-      cmac(t, u[3 * a + 1], h[3 * sp + 1]);
-      cmac(t, u[3 * a + 2], h[3 * sp + 2]);
-      w[3 * sp + a] = t;
-    }
+    for (int a = 0; a < 3; ++a)
+      w[3 * sp + a] = dot3<1>(u[3 * a], h[3 * sp], u[3 * a + 1], h[3 * sp + 1], u[3 * a + 2], h[3 * sp + 2]);
 }
 template <typename T>
 __device__ __forceinline__ void su3_dag_mul(const cpx<T> u[9], const cpx<T> h[6], cpx<T> w[6]) {
 #pragma unroll
   for (int sp = 0; sp < 2; ++sp)
 #pragma unroll
-    for (int a = 0; a < 3; ++a) {
-      cpx<T> t = cmulc(u[a], h[3 * sp]);
-      cmacc(t, u[3 + a], h[3 * sp + 1]);
-      cmacc(t, u[6 + a], h[3 * sp + 2]);
-      w[3 * sp + a] = t;
-    }
-}
-
-// p = wf + U^dag h
-template <typename T>
-__device__ __forceinline__ void su3_dag_mul_add(const cpx<T> u[9], const cpx<T> h[6], const cpx<T> wf[6], cpx<T> p[6]) {
-#pragma unroll
-  for (int sp = 0; sp < 2; ++sp)
-#pragma unroll
-    for (int a = 0; a < 3; ++a) {
-      cpx<T> t = wf[3 * sp + a];
-#pragma unroll
-      for (int b = 0; b < 3; ++b) cmacc(t, u[3 * b + a], h[3 * sp + b]);
-      p[3 * sp + a] = t;
-    }
+    for (int a = 0; a < 3; ++a)
+      w[3 * sp + a] = dot3<-1>(u[a], h[3 * sp], u[3 + a], h[3 * sp + 1], u[6 + a], h[3 * sp + 2]);
 }
 
 // Per-thread sums for the epilogue reductions, kept in the compute type: GB300 runs
@@ -173,14 +138,10 @@ __device__ __forceinline__ void acc_norm(Acc<T>& a, const cpx<T>& z) {
   a.add(z.i, z.i);
 }
 
-// FP64 takes the two hops of a direction together (accumulate_pair): that kernel is bound by FP64
-// operations, 840 per site instead of 912 (12 systems of 16^3 x 32 2.82 -> 2.60 ms). For FP32 the
-// registers it holds across the second product cost more than the additions it saves (12-system
-// sign 20.2 -> 20.7 ms). FIRST: this hop starts the sum (saves 24 additions).
+// FIRST: this hop starts the sum (saves 24 additions).
 template <int MU, int PIN, int PL, bool RO, typename T, bool FIRST = false>
 __device__ __forceinline__ void hop_dir(const Geom& g, const LinkRef& L, const SpinorRef& in, int rhs, int s,
                                         const int x[4], int stride, cpx<T> acc[12]) {
-  constexpr bool PAIRED = std::is_same<T, double>::value;
   cpx<T> psi[12], h[6], w[6], u[9];
   // forward neighbour: (1 - gamma_mu) U_mu(x) psi(x + mu)
   {
@@ -194,7 +155,7 @@ __device__ __forceinline__ void hop_dir(const Geom& g, const LinkRef& L, const S
     }
     load_link<PL, T>(L, MU, s, u);
     su3_mul(u, h, w);
-    if constexpr (FIRST && !PAIRED) {
+    if constexpr (FIRST) {
       static_assert(MU == 0, "the first direction");
 #pragma unroll
       for (int k = 0; k < 6; ++k) acc[k] = w[k];
@@ -203,7 +164,7 @@ __device__ __forceinline__ void hop_dir(const Geom& g, const LinkRef& L, const S
         acc[6 + c] = timesI(w[3 + c]);
         acc[9 + c] = timesI(w[c]);
       }
-    } else if constexpr (!PAIRED) {
+    } else {
       accumulate<MU, -1>(acc, w);
     }
   }
@@ -218,14 +179,8 @@ __device__ __forceinline__ void hop_dir(const Geom& g, const LinkRef& L, const S
       for (int k = 0; k < 6; ++k) h[k] = -h[k];
     }
     load_link<PL, T>(L, MU, sb, u);
-    if constexpr (PAIRED) {
-      cpx<T> p[6];
-      su3_dag_mul_add(u, h, w, p);
-      accumulate_pair<MU, MU == 0>(acc, p, w);
-    } else {
-      su3_dag_mul(u, h, w);
-      accumulate<MU, +1>(acc, w);
-    }
+    su3_dag_mul(u, h, w);
+    accumulate<MU, +1>(acc, w);
   }
 }
 
