@@ -120,7 +120,8 @@ typedef struct {
                            projections of the deflated starts, Sec. 4): 0 (default) on the
                            tensor cores with FP64-level accuracy (operands split into six
                            7-bit digits, exact BF16 products, exact FP32 sums over 512 reals,
-                           double-float and FP64 above) for FP64 and FP32 fields, else as 1;
+                           double-float and FP64 above) for two FP64 or two FP32 fields, else
+                           as 1;
                            1 CUDA-core kernel with FP32 products and FP64 sums              */
   void*  stream;        /* cudaStream_t for all work; NULL = legacy default stream              */
 } ovl_params;

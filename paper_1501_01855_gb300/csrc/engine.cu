@@ -552,8 +552,8 @@ static ovl_status kd_project(ovl_ctx* c, const Field& v, int voff, int n, const 
 static ovl_status kd_add_low(ovl_ctx* c, Field& y, int n, const std::vector<cd>& C) {
   if (C.empty()) return OVL_OK;
   const int nk = c->kd_n;
-  const Field* y64 = &y;
-  if (y.prec != P64 && y.prec != P32) {
+  const Field* y64 = &y;   // the tensor-core block takes two fields of one precision
+  if (y.prec != P64) {
     Field* t;
     OVL_TRY(get_field(c, "kd_ty", P64, n, &t));
     OVL_TRY(copy_convert(c, y, 0, *t, 0, n));

@@ -253,7 +253,7 @@ __global__ void __launch_bounds__(256) tc_gram_exp_kernel(const void* X, size_t 
 
 // grid: (splits of the K range, A tiles x B tiles). partial: per CTA 2 x 64 x 64 doubles
 // (Re rows, then Im rows), scaled by 2^(e_i + e_j).
-template <int PA, int PB>
+template <int P>
 __global__ void __launch_bounds__(TG_THREADS, 1)
     tc_gram_kernel(const void* A, int na, const void* B, int nb, size_t nq, int g5q, const int* exa, const int* exb,
                    double* partial, int* err) {
@@ -272,8 +272,8 @@ __global__ void __launch_bounds__(TG_THREADS, 1)
   const size_t st0 = nstage_all * split / nsplit, st1 = nstage_all * (split + 1) / nsplit;
   const int nst = (int)(st1 - st0);
 
-  if (tid < TG_NA) ea_s[tid] = a0 + tid < na ? tg_exponent<PA>(exa[a0 + tid]) : TG_EXP_ZERO;
-  else if (tid < TG_NA + TG_NB) eb_s[tid - TG_NA] = b0 + tid - TG_NA < nb ? tg_exponent<PB>(exb[b0 + tid - TG_NA]) : TG_EXP_ZERO;
+  if (tid < TG_NA) ea_s[tid] = a0 + tid < na ? tg_exponent<P>(exa[a0 + tid]) : TG_EXP_ZERO;
+  else if (tid < TG_NA + TG_NB) eb_s[tid - TG_NA] = b0 + tid - TG_NA < nb ? tg_exponent<P>(exb[b0 + tid - TG_NA]) : TG_EXP_ZERO;
   if (tid == 0) {
     abort_flag = 0;
     for (int b = 0; b < TG_BUF; ++b) {
@@ -387,7 +387,7 @@ __global__ void __launch_bounds__(TG_THREADS, 1)
       if (task >= 64 || it >= nst) return;
       const int tt = task & 31, r = (tt >> 2) * 8 + rl;
       const size_t q = (st0 + it) * TG_KC + (tt & 3) * 4 + kp;
-      raw[i] = task < 32 ? tg_load<PA>(A, na, a0 + r, nq, q) : tg_load<PB>(B, nb, b0 + r, nq, q);
+      raw[i] = task < 32 ? tg_load<P>(A, na, a0 + r, nq, q) : tg_load<P>(B, nb, b0 + r, nq, q);
     };
 #pragma unroll
     for (int i = 0; i < TG_TASKS; ++i) load(i, 0);
@@ -408,7 +408,7 @@ __global__ void __launch_bounds__(TG_THREADS, 1)
         load(i, it + 1);
         uint32_t pd[TG_S];   // digit s of (re, im) as a BF16 pair
         if (task < 32) {
-          tg_digits<PA>(w, ea_s[r], false, pd);
+          tg_digits<P>(w, ea_s[r], false, pd);
           // A row r and A' row 64 + r: (re, im) and (-im, re)
           const uint32_t off = (uint32_t)((kc * 16 + rg) * 128 + rl * 16 + kp * 4);
 #pragma unroll
@@ -417,7 +417,7 @@ __global__ void __launch_bounds__(TG_THREADS, 1)
             *reinterpret_cast<uint32_t*>(stA + d * TG_TILE_A + off + 8 * 128) = __byte_perm(pd[d], 0u, 0x1032) ^ 0x8000u;
           }
         } else {
-          tg_digits<PB>(w, eb_s[r], g5q && q0 + j >= (size_t)g5q, pd);
+          tg_digits<P>(w, eb_s[r], g5q && q0 + j >= (size_t)g5q, pd);
           const uint32_t off = (uint32_t)((kc * 8 + rg) * 128 + rl * 16 + kp * 4);
 #pragma unroll
           for (int d = 0; d < TG_S; ++d) *reinterpret_cast<uint32_t*>(stB + d * TG_TILE_B + off) = pd[d];
@@ -479,7 +479,9 @@ __global__ void tc_gram_reduce_kernel(const double* partial, int na, int nb, int
   G[2 * e + 1] += im;
 }
 
-bool tc_gram_supported(int pa, int pb) { return (pa == P64 || pa == P32) && (pb == P64 || pb == P32); }
+// Both sides of one precision: an FP64 field holds one component per 16-byte chunk and an FP32 field
+// two, so element q of the one is not the component and site of element q of the other.
+bool tc_gram_supported(int pa, int pb) { return pa == pb && (pa == P64 || pa == P32); }
 
 int tc_gram_splits(int na, int nb, int V, int nsm) {
   const int tiles = ((na + TG_NA - 1) / TG_NA) * ((nb + TG_NB - 1) / TG_NB);
@@ -498,13 +500,13 @@ size_t tc_gram_work_doubles(int na, int nb, int nsplit) {
   return tiles * nsplit * 2 * TG_NA * TG_NB;
 }
 
-// A (na vectors), B (nb vectors): fields of precision pa / pb (P64 or P32), 12 V complex
-// elements each in the library layout (the element order is the same for both, and
-// gamma5 negates the elements from 6 V on). G: na x nb complex FP64 (device), accumulated.
+// A (na vectors), B (nb vectors): fields of precision p (P64 or P32), 12 V complex elements
+// each in the library layout (gamma5 negates the elements from 6 V on). G: na x nb complex
+// FP64 (device), accumulated.
 // partial: tc_gram_work_doubles doubles; ex: na + nb ints; err: device int set to 1 when a
 // bounded wait gives up.
-void launch_tc_gram(int pa, const void* A, int na, int pb, const void* B, int nb, int V, int g5, int nsplit,
-                    double* G, double* partial, int* ex, int* err, cudaStream_t st) {
+void launch_tc_gram(int p, const void* A, int na, const void* B, int nb, int V, int g5, int nsplit, double* G,
+                    double* partial, int* ex, int* err, cudaStream_t st) {
   const size_t nq = (size_t)12 * V;
   int* exa = ex;
   int* exb = ex + na;
@@ -513,22 +515,18 @@ void launch_tc_gram(int pa, const void* A, int na, int pb, const void* B, int nb
   auto blocks = [&](int n) {
     return (unsigned)std::max<size_t>(1, std::min<size_t>((1216 + n - 1) / n, (nq + 4095) / 4096));
   };
-  if (pa == P64) tc_gram_exp_kernel<P64><<<dim3(na, blocks(na)), 256, 0, st>>>(A, nq, exa);
-  else tc_gram_exp_kernel<P32><<<dim3(na, blocks(na)), 256, 0, st>>>(A, nq, exa);
-  if (pb == P64) tc_gram_exp_kernel<P64><<<dim3(nb, blocks(nb)), 256, 0, st>>>(B, nq, exb);
-  else tc_gram_exp_kernel<P32><<<dim3(nb, blocks(nb)), 256, 0, st>>>(B, nq, exb);
   const int tiles = ((na + TG_NA - 1) / TG_NA) * ((nb + TG_NB - 1) / TG_NB);
   dim3 grid((unsigned)nsplit, (unsigned)tiles);
   const int g5q = g5 ? (int)(6 * (size_t)V) : 0;
-#define TG(X, Y)                                                                                   \
+#define TG(P)                                                                                      \
   do {                                                                                             \
-    cudaFuncSetAttribute(tc_gram_kernel<X, Y>, cudaFuncAttributeMaxDynamicSharedMemorySize, TG_SMEM); \
-    tc_gram_kernel<X, Y><<<grid, TG_THREADS, TG_SMEM, st>>>(A, na, B, nb, nq, g5q, exa, exb, partial, err); \
+    tc_gram_exp_kernel<P><<<dim3(na, blocks(na)), 256, 0, st>>>(A, nq, exa);                       \
+    tc_gram_exp_kernel<P><<<dim3(nb, blocks(nb)), 256, 0, st>>>(B, nq, exb);                       \
+    cudaFuncSetAttribute(tc_gram_kernel<P>, cudaFuncAttributeMaxDynamicSharedMemorySize, TG_SMEM); \
+    tc_gram_kernel<P><<<grid, TG_THREADS, TG_SMEM, st>>>(A, na, B, nb, nq, g5q, exa, exb, partial, err); \
   } while (0)
-  if (pa == P64 && pb == P64) TG(P64, P64);
-  else if (pa == P32 && pb == P32) TG(P32, P32);
-  else if (pa == P64) TG(P64, P32);
-  else TG(P32, P64);
+  if (p == P64) TG(P64);
+  else TG(P32);
 #undef TG
   const int nn = na * nb;
   tc_gram_reduce_kernel<<<(nn + 255) / 256, 256, 0, st>>>(partial, na, nb, nsplit, G);
