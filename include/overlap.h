@@ -177,6 +177,11 @@ const char* overlap_last_error(const ovl_ctx* ctx);
  * allocates what it needs again. Synchronises the context stream. */
 ovl_status ovl_trim(ovl_ctx* ctx);
 
+/* Limit of the bounded waits inside kernels, in seconds (0..3600; 2 in a new context): those of
+ * the tensor-core Gram block, whose calls return OVL_ETIMEOUT when one gives up (the context
+ * stays usable). 0 makes every such wait give up at once. */
+ovl_status ovl_set_wait_limit(ovl_ctx* ctx, double seconds);
+
 /* Host-only (no GPU needed): the Zolotarev rational of order n on a < |x| < b
  * (Sec. 3), eps(x) = sum_i omega_i x / (x^2 + sigma_i), sigma ascending, and its
  * maximum error delta, from Jacobi elliptic functions (AGM / descending Landen). */

@@ -82,6 +82,7 @@ _SIGS = {
     "overlap_destroy": (None, [P]),
     "overlap_last_error": (ctypes.c_char_p, [P]),
     "ovl_trim": (I, [P]),
+    "ovl_set_wait_limit": (I, [P, D]),
     "overlap_zolotarev": (I, [P, DP, DP, DP, DP, DP]),
     "ovl_wilson_apply": (I, [P, P, P, I, I, I, I]),
     "ovl_wilson_apply_noalloc": (I, [P, P, P, I, I, I]),
@@ -373,6 +374,10 @@ class Overlap:
     def trim(self):
         """Release the workspaces and graphs the context caches between calls."""
         _check(load().ovl_trim(self.h), self.h)
+
+    def set_wait_limit(self, seconds):
+        """Limit of the bounded waits inside kernels (2 s in a new context; 0: give up at once)."""
+        _check(load().ovl_set_wait_limit(self.h, float(seconds)), self.h)
 
     def close(self):
         if getattr(self, "h", None):

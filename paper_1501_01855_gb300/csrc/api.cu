@@ -58,6 +58,13 @@ extern "C" ovl_status ovl_params_default(ovl_params* p) {
 
 extern "C" const char* overlap_last_error(const ovl_ctx* c) { return c ? c->err.c_str() : "null context"; }
 
+extern "C" ovl_status ovl_set_wait_limit(ovl_ctx* c, double seconds) {
+  if (!c) return OVL_EINVAL;
+  if (!(seconds >= 0.0 && seconds <= 3600.0)) return set_err(c, OVL_EINVAL, "the wait limit must lie in 0..3600 s");
+  c->wait_ns = (unsigned long long)(seconds * 1e9);
+  return OVL_OK;
+}
+
 extern "C" ovl_status ovl_trim(ovl_ctx* c) {
   if (!c) return OVL_EINVAL;
   trim_workspaces(c);

@@ -87,6 +87,7 @@ struct ovl_ctx {
   unsigned int* lzp_bar = nullptr;  // barrier and flags of the one-launch Lanczos iteration
   double* lzp_part = nullptr;       // its blocks' partial sums
   int nsm = 0;                      // SMs of the device
+  unsigned long long wait_ns = 2000000000ull;   // limit of the bounded waits inside kernels
   void* lz_pool = nullptr;       // stored Lanczos bases of every sign precision (one at a time)
   size_t lz_pool_bytes = 0;
   bool lz_pool_busy = false;     // a sign application holds a view of the pool

@@ -235,12 +235,12 @@ void launch_gram(int pa, SpinorRef A, int na, int pb, SpinorRef B, int nb, int V
 // The same block on the tensor cores, FP64-accurate (operands split into 7-bit digits with
 // exact BF16 products and exact FP32 sums; both sides P64 or both P32). ex: na + nb ints;
 // partial: tc_gram_work_doubles(na, nb, nsplit) doubles; err set to 1 on a bounded wait that
-// gave up.
+// gave up after wait_ns.
 bool tc_gram_supported(int pa, int pb);
 int tc_gram_splits(int na, int nb, int V, int nsm);
 size_t tc_gram_work_doubles(int na, int nb, int nsplit);
 void launch_tc_gram(int p, const void* A, int na, const void* B, int nb, int V, int g5, int nsplit, double* G,
-                    double* partial, int* ex, int* err, cudaStream_t st);
+                    double* partial, int* ex, int* err, unsigned long long wait_ns, cudaStream_t st);
 // Y_j (+)= sum_i A_i C[i, j] for j < ny (C na x ny row-major complex, device); Y distinct
 // from A. add = 1 accumulates into Y.
 void launch_combine(int pa, SpinorRef A, int na, const double* C, int py, SpinorRef Y, int ny, int V, int add,

@@ -120,7 +120,7 @@ ovl_status gram_device(ovl_ctx* c, const Field& A, int aoff, int na, const Field
     *derr = ex + na + nb;
     OVL_CUDA(c, cudaMemsetAsync(*derr, 0, sizeof(int), c->st));
     launch_tc_gram(A.prec, A.ref(aoff).data, na, B.ref(boff).data, nb, c->V, g5, nsplit, dG, c->dwork, ex, *derr,
-                   c->st);
+                   c->wait_ns, c->st);
   } else {
     launch_gram(A.prec, A.ref(aoff), na, B.prec, B.ref(boff), nb, c->V, dG, c->dwork, c->dwork_n - gsz, g5, c->st);
   }

@@ -35,8 +35,8 @@
 // other 3.5 cycles per issued instruction. Bound now by the ALU pipe of the slicing (57% busy,
 // tensor pipe 35%). FP64 fields, 16^3 x 32: 128 x 128 17.6 -> 7.3 ms, 64 x 64 8.7 -> 2.1, 64 x 12 8.6 -> 1.7
 // (more than half of that was the exponent pass, below).
-// Waits are bounded by a 2 s deadline: one that gives up sets the error flag, the CTA skips the
-// rest, waits once more (again bounded) for the MMAs it has committed, frees its tensor memory
+// Waits are bounded (wait_ns, 2 s by default): one that gives up sets the error flag, the CTA skips the
+// rest, warp by warp (warp_wait), waits once more (again bounded) for the MMAs it has committed, frees its tensor memory
 // and returns, and the host reports OVL_ETIMEOUT.
 #include <limits.h>
 #include <stdint.h>
@@ -69,7 +69,7 @@ constexpr int TG_TASKS = (64 + TG_SLICERS - 1) / TG_SLICERS;   // slicing tasks 
 constexpr int TG_TMEM_COLS = 512;
 static_assert(TG_G * TG_NB <= TG_TMEM_COLS, "group accumulators exceed the tensor-memory allocation");                // 7 groups x 64 columns, rounded to a power of 2
 constexpr int TG_EXP_ZERO = -4000;               // scale exponent of an all-zero vector
-constexpr unsigned long long TG_WAIT_NS = 2000000000ull;
+constexpr unsigned long long TG_DRAIN_NS = 2000000000ull;   // the exit's wait for MMAs in flight
 
 __device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
 
@@ -89,11 +89,12 @@ __device__ __forceinline__ uint64_t smem_desc(uint32_t saddr, uint32_t lbo, uint
   return d;
 }
 
-// true once the barrier's phase with this parity has completed, false after the deadline or when
-// another thread has given up (*gave_up)
-__device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatile int* gave_up) {
+// true once the barrier's phase with this parity has completed, false after the limit or when
+// another thread has given up (*gave_up). A limit of zero gives up without a look.
+__device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatile int* gave_up,
+                                          unsigned long long limit) {
   const unsigned long long t0 = global_ns();
-  for (;;) {
+  while (limit != 0) {
     uint32_t ok;
     asm volatile(
         "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, p;\n}\n"
@@ -102,11 +103,18 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatil
         : "memory");
     if (ok) return true;
     if (gave_up != nullptr && *gave_up) return false;
-    if (global_ns() - t0 > TG_WAIT_NS) {
-      if (gave_up != nullptr) *gave_up = 1;
-      return false;
-    }
+    if (global_ns() - t0 > limit) break;
   }
+  if (gave_up != nullptr) *gave_up = 1;
+  return false;
+}
+// The wait of a whole warp: true when every lane saw the phase complete. Lanes poll for
+// themselves and may disagree when the time runs out; what follows (warp barriers, tcgen05.ld,
+// the way out) takes the warp as one, so they vote first.
+__device__ __forceinline__ bool warp_wait(uint32_t bar, uint32_t parity, volatile int* gave_up,
+                                          unsigned long long limit) {
+  const bool ok = mbar_wait(bar, parity, gave_up, limit);
+  return __all_sync(0xffffffffu, ok) != 0;
 }
 
 __device__ __forceinline__ void mma_bf16(uint32_t tmem, uint64_t da, uint64_t db, uint32_t idesc, uint32_t acc) {
@@ -256,7 +264,7 @@ __global__ void __launch_bounds__(256) tc_gram_exp_kernel(const void* X, size_t 
 template <int P>
 __global__ void __launch_bounds__(TG_THREADS, 1)
     tc_gram_kernel(const void* A, int na, const void* B, int nb, size_t nq, int g5q, const int* exa, const int* exb,
-                   double* partial, int* err) {
+                   double* partial, int* err, unsigned long long wait_ns) {
   extern __shared__ unsigned char sm_raw[];
   unsigned char* sm = reinterpret_cast<unsigned char*>(((uintptr_t)sm_raw + 1023) & ~(uintptr_t)1023);
   __shared__ uint32_t tmem_base;
@@ -307,8 +315,7 @@ __global__ void __launch_bounds__(TG_THREADS, 1)
   // One accumulation chunk's group sums are exact integers in FP32: add them, scaled, in
   // double-float. Every warp, once the chunk's MMAs are done (fbar); false when a wait gave up.
   auto flush = [&](int chunk) -> bool {
-    if (!mbar_wait(smem_u32(&fbar), (uint32_t)chunk & 1u, &abort_flag)) return false;
-    __syncwarp();   // tcgen05.ld is warp-collective
+    if (!warp_wait(smem_u32(&fbar), (uint32_t)chunk & 1u, &abort_flag, wait_ns)) return false;
     asm volatile("tcgen05.fence::after_thread_sync;");
 #pragma unroll
     for (int g = 0; g < TG_G; ++g) {
@@ -343,11 +350,11 @@ __global__ void __launch_bounds__(TG_THREADS, 1)
   if (warp == 0) {
     for (int it = 0; ok && it < nst; ++it) {
       const int s = it % TG_BUF, cs = it % TG_CHUNK;
-      ok = mbar_wait(smem_u32(&full[s]), (uint32_t)(it / TG_BUF) & 1u, &abort_flag);
+      ok = warp_wait(smem_u32(&full[s]), (uint32_t)(it / TG_BUF) & 1u, &abort_flag, wait_ns);
       // the accumulators restart: the last chunk must have been read out
       if (ok && cs == 0 && it > 0) ok = flush(it / TG_CHUNK - 1);
-      if (ok && cs == 0 && it > 0) ok = mbar_wait(smem_u32(&flushed), (uint32_t)(it / TG_CHUNK - 1) & 1u, &abort_flag);
-      ok = __all_sync(0xffffffffu, ok);
+      if (ok && cs == 0 && it > 0)
+        ok = warp_wait(smem_u32(&flushed), (uint32_t)(it / TG_CHUNK - 1) & 1u, &abort_flag, wait_ns);
       if (!ok) break;
       if (lane == 0) {
         asm volatile("tcgen05.fence::after_thread_sync;");
@@ -393,8 +400,7 @@ __global__ void __launch_bounds__(TG_THREADS, 1)
     for (int i = 0; i < TG_TASKS; ++i) load(i, 0);
     for (int it = 0; ok && it < nst; ++it) {
       const int s = it % TG_BUF;
-      if (it >= TG_BUF) ok = mbar_wait(smem_u32(&empty[s]), (uint32_t)(it / TG_BUF - 1) & 1u, &abort_flag);
-      ok = __all_sync(0xffffffffu, ok);
+      if (it >= TG_BUF) ok = warp_wait(smem_u32(&empty[s]), (uint32_t)(it / TG_BUF - 1) & 1u, &abort_flag, wait_ns);
       if (!ok) break;
       unsigned char* stA = sm + s * TG_STAGE;
       unsigned char* stB = stA + TG_S * TG_TILE_A;
@@ -439,7 +445,7 @@ __global__ void __launch_bounds__(TG_THREADS, 1)
   // wait for a commit that covers all of them
   if (abort_flag && tid == 0) {
     mma_commit(smem_u32(&drain));
-    mbar_wait(smem_u32(&drain), 0u, nullptr);
+    mbar_wait(smem_u32(&drain), 0u, nullptr, TG_DRAIN_NS);
   }
   __syncthreads();
   if (abort_flag && tid == 0) atomicExch(err, 1);
@@ -504,9 +510,9 @@ size_t tc_gram_work_doubles(int na, int nb, int nsplit) {
 // each in the library layout (gamma5 negates the elements from 6 V on). G: na x nb complex
 // FP64 (device), accumulated.
 // partial: tc_gram_work_doubles doubles; ex: na + nb ints; err: device int set to 1 when a
-// bounded wait gives up.
+// bounded wait gives up (after wait_ns).
 void launch_tc_gram(int p, const void* A, int na, const void* B, int nb, int V, int g5, int nsplit, double* G,
-                    double* partial, int* ex, int* err, cudaStream_t st) {
+                    double* partial, int* ex, int* err, unsigned long long wait_ns, cudaStream_t st) {
   const size_t nq = (size_t)12 * V;
   int* exa = ex;
   int* exb = ex + na;
@@ -523,7 +529,7 @@ void launch_tc_gram(int p, const void* A, int na, const void* B, int nb, int V, 
     tc_gram_exp_kernel<P><<<dim3(na, blocks(na)), 256, 0, st>>>(A, nq, exa);                       \
     tc_gram_exp_kernel<P><<<dim3(nb, blocks(nb)), 256, 0, st>>>(B, nq, exb);                       \
     cudaFuncSetAttribute(tc_gram_kernel<P>, cudaFuncAttributeMaxDynamicSharedMemorySize, TG_SMEM); \
-    tc_gram_kernel<P><<<grid, TG_THREADS, TG_SMEM, st>>>(A, na, B, nb, nq, g5q, exa, exb, partial, err); \
+    tc_gram_kernel<P><<<grid, TG_THREADS, TG_SMEM, st>>>(A, na, B, nb, nq, g5q, exa, exb, partial, err, wait_ns); \
   } while (0)
   if (p == P64) TG(P64);
   else TG(P32);
