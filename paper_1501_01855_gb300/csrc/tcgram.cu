@@ -11,9 +11,9 @@
 // others in [-64, 64]), x = 2^e_i sum_s a_s 2^(-7 s) up to 2^(e_i - 43), by FP32 arithmetic
 // (tg_digits). Digits are exact in BF16 and
 // their products exact in the tensor core; for each group g = s + t (2 .. 8) the products
-// a_s b_t summed over 512 reals stay below 2^24 in magnitude, so the FP32 accumulator holds
+// a_s b_t summed over 512 reals stay within 2^24 in magnitude, so the FP32 accumulator holds
 // that sum exactly. Every 512 reals the seven group sums are read from tensor memory and
-// added, scaled by 2^(-7 g), into a double-float (hi + lo FP32) accumulator per output;
+// added, scaled by 2^(-7 g), into a normalised double-float (hi + lo FP32) accumulator per output;
 // the partial results of the CTAs that split the sum are added in FP64 in a fixed order.
 // The last digit is rounded to nearest; the pairs with s + t > 8 (weight 2^-63 and below) are left out.
 // The error is then that of representing each operand to 2^(e_i - 43): on Gaussian data
@@ -115,6 +115,14 @@ __device__ __forceinline__ bool warp_wait(uint32_t bar, uint32_t parity, volatil
                                           unsigned long long limit) {
   const bool ok = mbar_wait(bar, parity, gave_up, limit);
   return __all_sync(0xffffffffu, ok) != 0;
+}
+
+// a <- fl(a + b); the rounding error
+__device__ __forceinline__ float two_sum(float& a, float b) {
+  const float s = __fadd_rn(a, b), v = __fsub_rn(s, a);
+  const float e = __fadd_rn(__fsub_rn(a, __fsub_rn(s, v)), __fsub_rn(b, v));
+  a = s;
+  return e;
 }
 
 __device__ __forceinline__ void mma_bf16(uint32_t tmem, uint64_t da, uint64_t db, uint32_t idesc, uint32_t acc) {
@@ -312,32 +320,45 @@ __global__ void __launch_bounds__(TG_THREADS, 1)
 #pragma unroll
   for (int c = 0; c < TG_CPT; ++c) acc_h[c] = acc_l[c] = 0.f;
 
-  // One accumulation chunk's group sums are exact integers in FP32: add them, scaled, in
-  // double-float. Every warp, once the chunk's MMAs are done (fbar); false when a wait gave up.
+  // One accumulation chunk's group sums are exact integers in FP32: summed, scaled, in
+  // double-float from the smallest weight up, then one double-float addition to the running sum,
+  // which stays normalised (|low| <= half an ulp of high): however many chunks a CTA sums, each
+  // adds one rounding of 2^-48. Every warp, once the chunk's MMAs are done (fbar); false when a
+  // wait gave up.
   auto flush = [&](int chunk) -> bool {
     if (!warp_wait(smem_u32(&fbar), (uint32_t)chunk & 1u, &abort_flag, wait_ns)) return false;
     asm volatile("tcgen05.fence::after_thread_sync;");
+    constexpr int NC = 8;   // columns at a time (registers)
 #pragma unroll
-    for (int g = 0; g < TG_G; ++g) {
-      uint32_t v[TG_CPT];
-      static_assert(TG_CPT == 16, "the flush reads 16 columns per thread");
-      const uint32_t ta_ = tmem + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)(g * TG_NB + cbase);
-      asm volatile(
-          "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
-          : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]),
-            "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]), "=r"(v[15])
-          : "r"(ta_));
-      asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-      const float w = __int_as_float((127 - 7 * (g + 2)) << 23);   // 2^(-7 (g + 2))
+    for (int c0 = 0; c0 < TG_CPT; c0 += NC) {
+      float ch[NC], cl[NC];
 #pragma unroll
-      for (int c = 0; c < TG_CPT; ++c) {
-        // TwoSum of acc_h and the exactly scaled group sum
-        const float x = __uint_as_float(v[c]) * w;
-        const float sum = acc_h[c] + x;
-        const float bb = sum - acc_h[c];
-        const float e = (acc_h[c] - (sum - bb)) + (x - bb);
-        acc_h[c] = sum;
-        acc_l[c] += e;
+      for (int g = TG_G - 1; g >= 0; --g) {
+        uint32_t v[NC];
+        const uint32_t ta_ = tmem + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)(g * TG_NB + cbase + c0);
+        asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+                     : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7])
+                     : "r"(ta_));
+        asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+        const float w = __int_as_float((127 - 7 * (g + 2)) << 23);   // 2^(-7 (g + 2))
+#pragma unroll
+        for (int c = 0; c < NC; ++c) {
+          const float x = __uint_as_float(v[c]) * w;   // exact
+          if (g == TG_G - 1) {
+            ch[c] = x;
+            cl[c] = 0.f;
+          } else {
+            cl[c] += two_sum(ch[c], x);
+          }
+        }
+      }
+#pragma unroll
+      for (int c = 0; c < NC; ++c) {
+        float &h = acc_h[c0 + c], &l = acc_l[c0 + c];
+        l = __fadd_rn(two_sum(h, ch[c]), __fadd_rn(l, cl[c]));
+        const float r = __fadd_rn(h, l);
+        l = __fsub_rn(l, __fsub_rn(r, h));
+        h = r;
       }
     }
     asm volatile("tcgen05.fence::before_thread_sync;");
