@@ -8,8 +8,8 @@
 // matrix multiplication", 2012), with BF16 slices and FP32 accumulation in tensor memory.
 // Every vector i gets a power-of-two scale 2^e_i above its largest element; each real
 // element x is written in six balanced base-128 digits a_1 .. a_6 (a_1 in [-128, 128], the
-// others in [-64, 64]), x = 2^e_i sum_s a_s 2^(-7 s) up to 2^(e_i - 43), by FP32 arithmetic
-// (tg_digits). Digits are exact in BF16 and
+// others in [-64, 64]), x = 2^e_i sum_s a_s 2^(-7 s) up to 9/8 2^(e_i - 43), without bias, by FP32
+// arithmetic (tg_digits). Digits are exact in BF16 and
 // their products exact in the tensor core; for each group g = s + t (2 .. 8) the products
 // a_s b_t summed over 512 reals stay within 2^24 in magnitude, so the FP32 accumulator holds
 // that sum exactly. Every 512 reals the seven group sums are read from tensor memory and
@@ -162,11 +162,15 @@ struct TgLoad<P32> {
 // others in [-64, 64], and x 2^-e = sum_s d_s 2^(-7 (s + 1)) up to 2^-43. A digit is an integer of
 // at most 8 bits, so the upper half of its float is its exact BF16.
 // FP32 operands: r by two power-of-two factors. FP64 operands, from their bits (conversions from
-// FP64 are slow): r is the float of the leading 24 bits, and the next 23 bits, a second float,
-// join the remainder after three digits, when 21 of the leading bits are spent (rounded there
-// at 2^-46; the third digit is chosen with them, so that the fourth stays in its range). About 75 instructions per element, against 270 for taking the digits out of a 64-bit
-// fixed-point integer: a 64 x 64 tile on 16^4 1.43 -> 0.81 ms with the
-// pipeline below.
+// FP64 are slow): r is the float of the leading 24 bits; the next 22 bits, with a last bit that says
+// whether any bit below them is set (rounding to odd), are a second float that joins the remainder
+// after three digits, when 21 of the leading bits are spent (the third digit is chosen with them, so
+// that the fourth stays in its range). That sum is exact in FP32 for elements above 2^(e-1), but for a
+// remainder that the choice of the third digit left past one half, and is rounded at 2^-47 or finer
+// below, so the last digit's rounding, at 2^-43, is that of all 53 bits up to 9/8 of it and has no bias;
+// cutting the low bits off instead put 1.0e-14 on every diagonal entry of Gaussian data. About 80
+// instructions per element, against 270 for taking the digits out of a 64-bit fixed-point integer: a
+// 64 x 64 tile on 16^4 1.43 -> 0.81 ms with the pipeline below.
 __device__ __forceinline__ float tg_pow2(int k) { return __int_as_float((127 + k) << 23); }
 // the digit of s (r itself, or r and what follows it, rounded); r becomes its remainder
 __device__ __forceinline__ uint32_t tg_digit(f2 s, f2& r) {
@@ -182,7 +186,8 @@ __device__ __forceinline__ void tg_split64(uint2 w, int e, int thr, uint32_t fli
   const uint32_t sg = (w.y ^ flip) & 0x80000000u;
   const int ex = t - 896 - e;   // exponent field of the float, <= 126
   const uint32_t m = __funnelshift_l(w.x, w.y, 3) & 0x7FFFFFu;
-  const uint32_t v = (w.x >> 6) & 0x7FFFFFu;   // the next 23 bits: v 2^(t - 1023 - 46 - e), times 2^21 in lo
+  // the next 22 bits, and 1 when any bit below them is set: v 2^(t - 1023 - 46 - e), times 2^21 in lo
+  const uint32_t v = ((w.x >> 6) & 0x7FFFFEu) | ((w.x & 0x7Fu) != 0u ? 1u : 0u);
   const bool z = t < thr;
   hi = __uint_as_float(z ? 0u : ((uint32_t)ex << 23) | m | sg);
   const float f = __fsub_rn(__uint_as_float(0x4B000000u | v), 8388608.0f);
