@@ -337,6 +337,7 @@ static ovl_status create_impl(ovl_ctx* c, const int dims[4], const double* links
   c->eps_sign = eps_sign;
   c->st = (cudaStream_t)c->P.stream;
   OVL_CUDA(c, cudaGetDevice(&c->device));
+  OVL_CUDA(c, cudaDeviceGetAttribute(&c->nsm, cudaDevAttrMultiProcessorCount, c->device));
   OVL_CUDA(c, cudaMallocHost((void**)&c->hpin, sizeof(double) * 64 * 4096));
   OVL_CUDA(c, cudaMalloc((void**)&c->dscal, sizeof(double) * 64 * 4096));
   OVL_CUDA(c, cudaMalloc((void**)&c->dred, sizeof(double) * NVRED * 4096));

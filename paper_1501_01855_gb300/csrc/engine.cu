@@ -10,6 +10,7 @@
 #include <algorithm>
 #include <cmath>
 
+#include "bufferset.h"
 #include "context.h"
 #include "hostmath.h"
 #include "solver.h"
@@ -104,56 +105,47 @@ ovl_status get_field(ovl_ctx* c, const std::string& name, int prec, int n, Field
   return OVL_OK;
 }
 
+// a set of device buffers, all or none
+static ovl_status renew_device(ovl_ctx* c, std::initializer_list<BufferSlot> set, const char* what) {
+  cudaStreamSynchronize(c->st);
+  const int e = renew_all(set, [](void** p, size_t n) { return cudaMalloc(p, n); }, [](void* p) { cudaFree(p); });
+  return e == 0 ? OVL_OK : cuda_check(c, static_cast<cudaError_t>(e), what);
+}
+template <typename T>
+static BufferSlot slot(T** p, size_t count) {
+  return {reinterpret_cast<void**>(p), sizeof(T) * count};
+}
+
 ovl_status ensure_partials(ovl_ctx* c, int nrhs) {
   const size_t need = (size_t)nrhs * ((c->V + BX - 1) / BX) * NVRED;
   if (need <= c->partials_n) return OVL_OK;
-  if (c->partials) {
-    cudaStreamSynchronize(c->st);
-    cudaFree(c->partials);
-  }
-  OVL_CUDA(c, cudaMalloc((void**)&c->partials, need * sizeof(double)));
+  c->partials_n = 0;
+  OVL_TRY(renew_device(c, {slot(&c->partials, need)}, "cudaMalloc(partial sums)"));
   c->partials_n = need;
   return OVL_OK;
 }
 
 ovl_status ensure_ms(ovl_ctx* c, int nrhs) {
   if (nrhs <= c->ms_n) return OVL_OK;
-  if (c->ms) {
-    cudaStreamSynchronize(c->st);
-    cudaFree(c->ms);
-  }
-  OVL_CUDA(c, cudaMalloc((void**)&c->ms, sizeof(MsRhs) * nrhs));
+  c->ms_n = 0;
+  OVL_TRY(renew_device(c, {slot(&c->ms, nrhs)}, "cudaMalloc(multi-shift states)"));
   c->ms_n = nrhs;
   return OVL_OK;
 }
 
 ovl_status ensure_lz(ovl_ctx* c, int nrhs, int cap) {
   if (nrhs <= c->lz_n && cap <= c->lz_cap) return OVL_OK;
-  const int n = std::max(nrhs, c->lz_n), k = std::max(cap, c->lz_cap);
-  cudaStreamSynchronize(c->st);
-  if (c->lz) cudaFree(c->lz);
-  if (c->lz_hist) cudaFree(c->lz_hist);
-  if (c->lz_Y) cudaFree(c->lz_Y);
-  if (c->lz_coefW) cudaFree(c->lz_coefW);
-  if (c->lz_ctr) cudaFree(c->lz_ctr);
-  c->lz = nullptr;
-  c->lz_hist = c->lz_Y = c->lz_coefW = nullptr;
-  c->lz_ctr = nullptr;
+  const size_t n = std::max(nrhs, c->lz_n), k = std::max(cap, c->lz_cap);
   c->lz_n = c->lz_cap = 0;
-  OVL_CUDA(c, cudaMalloc((void**)&c->lz, sizeof(LzRhs) * n));
-  OVL_CUDA(c, cudaMalloc((void**)&c->lz_ctr, sizeof(unsigned int) * n));
+  // lz_Y is sized for the largest pole count (kernel deflation can change the count later)
+  OVL_TRY(renew_device(c,
+                       {slot(&c->lz, n), slot(&c->lz_ctr, n), slot(&c->lz_hist, 2 * n * k),
+                        slot(&c->lz_Y, n * NPMAX * 2 * k), slot(&c->lz_coefW, n * k), slot(&c->lzp_bar, LZP_WORDS),
+                        slot(&c->lzp_part, 2 * LZP_SYS * LZP_BLOCKS)},
+                       "cudaMalloc(Lanczos states)"));
   OVL_CUDA(c, cudaMemsetAsync(c->lz_ctr, 0, sizeof(unsigned int) * n, c->st));
-  OVL_CUDA(c, cudaMalloc((void**)&c->lz_hist, sizeof(double) * 2 * (size_t)n * k));
-  // sized for the largest pole count (kernel deflation can change the count later)
-  OVL_CUDA(c, cudaMalloc((void**)&c->lz_Y, sizeof(double) * (size_t)n * NPMAX * 2 * k));
-  OVL_CUDA(c, cudaMalloc((void**)&c->lz_coefW, sizeof(double) * (size_t)n * k));
-  if (!c->lzp_bar) {
-    OVL_CUDA(c, cudaMalloc((void**)&c->lzp_bar, sizeof(unsigned int) * LZP_WORDS));
-    OVL_CUDA(c, cudaMalloc((void**)&c->lzp_part, sizeof(double) * 2 * LZP_SYS * LZP_BLOCKS));
-    OVL_CUDA(c, cudaDeviceGetAttribute(&c->nsm, cudaDevAttrMultiProcessorCount, c->device));
-  }
-  c->lz_n = n;
-  c->lz_cap = k;
+  c->lz_n = (int)n;
+  c->lz_cap = (int)k;
   return OVL_OK;
 }
 
@@ -198,20 +190,18 @@ ovl_status ensure_stage(ovl_ctx* c, size_t bytes) {
   if (bytes <= c->hstage_bytes) return OVL_OK;
   // the last copy out of the old buffer must be done before it goes back
   if (c->hstage) OVL_CUDA(c, cudaEventSynchronize(c->stage_ev));
-  if (c->hstage) cudaFreeHost(c->hstage);
-  c->hstage = nullptr;
-  OVL_CUDA(c, cudaMallocHost(&c->hstage, bytes));
+  c->hstage_bytes = 0;
+  const int e = renew_all({{&c->hstage, bytes}}, [](void** p, size_t n) { return cudaMallocHost(p, n); },
+                          [](void* p) { cudaFreeHost(p); });
+  if (e != 0) return cuda_check(c, static_cast<cudaError_t>(e), "cudaMallocHost(staging)");
   c->hstage_bytes = bytes;
   return OVL_OK;
 }
 
 ovl_status ensure_work(ovl_ctx* c, size_t nd) {
   if (nd <= c->dwork_n) return OVL_OK;
-  if (c->dwork) {
-    cudaStreamSynchronize(c->st);
-    cudaFree(c->dwork);
-  }
-  OVL_CUDA(c, cudaMalloc((void**)&c->dwork, nd * sizeof(double)));
+  c->dwork_n = 0;
+  OVL_TRY(renew_device(c, {slot(&c->dwork, nd)}, "cudaMalloc(Gram work buffer)"));
   c->dwork_n = nd;
   return OVL_OK;
 }
