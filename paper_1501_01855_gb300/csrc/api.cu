@@ -289,8 +289,7 @@ extern "C" void overlap_destroy(ovl_ctx* c) {
   if (c->hpin) cudaFreeHost(c->hpin);
   if (c->hstage) cudaFreeHost(c->hstage);
   if (c->stage_ev) cudaEventDestroy(c->stage_ev);
-  for (auto& g : c->graphs)
-    if (g.exec) cudaGraphExecDestroy(g.exec);
+  drop_graphs(c);
   if (c->cap_st) cudaStreamDestroy(c->cap_st);
   for (auto& q : c->prof.pending) {
     cudaEventDestroy(q.a);
@@ -403,7 +402,8 @@ ovl_status ovl::set_poles(ovl_ctx* c, int n_poles, double a, double b) {
     P.omega[i] = c->omega[i];
     P.gbound[i] = pole_gbound(c->sigma[i], a, b);
   }
-  if (c->st) cudaStreamSynchronize(c->st);
+  cudaStreamSynchronize(c->st);
+  drop_graphs(c);
   OVL_CUDA(c, cudaMemcpy(c->dpoles, &P, sizeof(Poles), cudaMemcpyHostToDevice));
   // step counts seen so far belong to the old rational
   memset(c->lz_kmax, 0, sizeof(c->lz_kmax));

@@ -160,6 +160,7 @@ ovl_status lz_pool_field(ovl_ctx* c, int prec, int n, Field* out);
 // free every cached workspace, graph and pool of the context (what the next call needs is
 // allocated again)
 void trim_workspaces(ovl_ctx* c);
+void drop_graphs(ovl_ctx* c);
 ovl_status ensure_stage(ovl_ctx* c, size_t bytes);
 ovl_status ensure_work(ovl_ctx* c, size_t ndoubles);
 

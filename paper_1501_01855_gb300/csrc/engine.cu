@@ -49,6 +49,14 @@ ovl_status check_launch(ovl_ctx* c, const char* where) {
 
 static size_t spinor_bytes(int prec) { return (size_t)spinor_site_bytes(prec); }
 
+// The cached graphs, with the stream idle: whenever something that their launches captured and
+// their keys do not name changes (the base shift, buffers that are released).
+void drop_graphs(ovl_ctx* c) {
+  for (auto& g : c->graphs)
+    if (g.exec) cudaGraphExecDestroy(g.exec);
+  c->graphs.clear();
+}
+
 void free_field(Field& f) {
   if (f.data) cudaFree(f.data);
   if (f.norm) cudaFree(f.norm);
@@ -81,9 +89,7 @@ ovl_status get_field(ovl_ctx* c, const std::string& name, int prec, int n, Field
       cudaFree(c->lz_pool);
       c->lz_pool = nullptr;
       c->lz_pool_bytes = 0;
-      for (auto& g : c->graphs)
-        if (g.exec) cudaGraphExecDestroy(g.exec);
-      c->graphs.clear();
+      drop_graphs(c);
       if (cudaMalloc(&f.data, bytes) != cudaSuccess) {
         cudaGetLastError();
         f.data = nullptr;
@@ -121,6 +127,7 @@ ovl_status ensure_partials(ovl_ctx* c, int nrhs) {
   if (need <= c->partials_n) return OVL_OK;
   c->partials_n = 0;
   OVL_TRY(renew_device(c, {slot(&c->partials, need)}, "cudaMalloc(partial sums)"));
+  drop_graphs(c);
   c->partials_n = need;
   return OVL_OK;
 }
@@ -129,6 +136,7 @@ ovl_status ensure_ms(ovl_ctx* c, int nrhs) {
   if (nrhs <= c->ms_n) return OVL_OK;
   c->ms_n = 0;
   OVL_TRY(renew_device(c, {slot(&c->ms, nrhs)}, "cudaMalloc(multi-shift states)"));
+  drop_graphs(c);
   c->ms_n = nrhs;
   return OVL_OK;
 }
@@ -143,6 +151,7 @@ ovl_status ensure_lz(ovl_ctx* c, int nrhs, int cap) {
                         slot(&c->lz_Y, n * NPMAX * 2 * k), slot(&c->lz_coefW, n * k), slot(&c->lzp_bar, LZP_WORDS),
                         slot(&c->lzp_part, 2 * LZP_SYS * LZP_BLOCKS)},
                        "cudaMalloc(Lanczos states)"));
+  drop_graphs(c);
   OVL_CUDA(c, cudaMemsetAsync(c->lz_ctr, 0, sizeof(unsigned int) * n, c->st));
   c->lz_n = (int)n;
   c->lz_cap = (int)k;
@@ -181,9 +190,7 @@ void trim_workspaces(ovl_ctx* c) {
   if (c->lz_pool) cudaFree(c->lz_pool);
   c->lz_pool = nullptr;
   c->lz_pool_bytes = 0;
-  for (auto& g : c->graphs)
-    if (g.exec) cudaGraphExecDestroy(g.exec);
-  c->graphs.clear();
+  drop_graphs(c);
 }
 
 ovl_status ensure_stage(ovl_ctx* c, size_t bytes) {
