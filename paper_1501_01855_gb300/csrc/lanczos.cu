@@ -170,7 +170,11 @@ __global__ void lz_start_kernel(LzRhs* lz, const double* partials, int nsb, cons
   const int rhs = blockIdx.x;
   LzRhs& L = lz[rhs];
   const double nn = lz_sum_partials(partials, nsb, rhs);
-  if (!first && (L.finished || L.status != 3)) return;
+  if (!first && (L.finished || L.status != 3)) {
+    // done in an earlier cycle, whose part is in y: nothing of it is combined again
+    if (threadIdx.x == 0) L.j = 0;
+    return;
+  }
   const double n0 = sqrt(nn);
   for (int i = threadIdx.x; i < P->n; i += blockDim.x) {
     if (first) L.w[i] = P->omega[i];
