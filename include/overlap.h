@@ -495,6 +495,14 @@ ovl_status ovl_bench_fp32(ovl_ctx* ctx, double* fma_per_s);
 ovl_status ovl_wilson_tuning(const ovl_ctx* ctx, int prec, int* variant, double* ms_thread_per_site,
                              double* ms_split, double* ms_tiled, double* ms_pair);
 
+/* Cycles of the stored-basis Lanczos (sign_method 0 and 2) since the context was created: run as
+ * one cooperative launch (double-float and FP32 signs of up to 4 systems on lattices that the SMs
+ * hold at once, with wilson_variant = -1 and use_graphs = 1), and run by launches per step.
+ * groups, tiles: the shape of the last one-launch cycle (thread groups per tile, tiles per
+ * block; 0 when there was none). Any output pointer may be NULL. */
+ovl_status ovl_lanczos_cycles(const ovl_ctx* ctx, long long* one_launch, long long* stepped, int* groups,
+                              int* tiles);
+
 /* Library version string. */
 const char* ovl_version(void);
 

@@ -105,6 +105,7 @@ _SIGS = {
     "ovl_profile_units": (I, [P, I, DP]),
     "ovl_bench_wilson": (I, [P, I, I, I, DP, DP]),
     "ovl_wilson_tuning": (I, [P, I, ctypes.POINTER(I), DP, DP, DP, DP]),
+    "ovl_lanczos_cycles": (I, [P, LLP, LLP, ctypes.POINTER(I), ctypes.POINTER(I)]),
     "ovl_bench_fp32": (I, [P, DP]),
     "ovl_gram": (I, [P, P, I, P, I, I, I, I, I, I, DP]),
     "ovl_bench_gram": (I, [P, I, I, I, I, I, DP]),
@@ -558,6 +559,15 @@ class Overlap:
         t = [ctypes.c_double() for _ in range(4)]
         _check(load().ovl_wilson_tuning(self.h, int(prec), ctypes.byref(v), *[ctypes.byref(x) for x in t]), self.h)
         return (v.value,) + tuple(x.value for x in t)
+
+    def lanczos_cycles(self):
+        """(cycles as one launch, cycles by launches per step, thread groups and tiles per block of the
+        last one-launch cycle) of the stored-basis Lanczos since the context was created."""
+        n1, n2 = ctypes.c_longlong(), ctypes.c_longlong()
+        g, t = ctypes.c_int(), ctypes.c_int()
+        _check(load().ovl_lanczos_cycles(self.h, ctypes.byref(n1), ctypes.byref(n2), ctypes.byref(g),
+                                         ctypes.byref(t)), self.h)
+        return n1.value, n2.value, g.value, t.value
 
     def bench_fp32(self):
         """Measured FP32 FMA instructions per second of the context's device."""

@@ -1278,6 +1278,16 @@ extern "C" ovl_status ovl_wilson_tuning(const ovl_ctx* c, int prec, int* variant
   return OVL_OK;
 }
 
+extern "C" ovl_status ovl_lanczos_cycles(const ovl_ctx* c, long long* one_launch, long long* stepped, int* groups,
+                                         int* tiles) {
+  if (!c) return OVL_EINVAL;
+  if (one_launch) *one_launch = c->lz_cycles[0];
+  if (stepped) *stepped = c->lz_cycles[1];
+  if (groups) *groups = c->lz_cycles[0] ? c->lzp_shape.groups : 0;
+  if (tiles) *tiles = c->lz_cycles[0] ? c->lzp_shape.tiles : 0;
+  return OVL_OK;
+}
+
 extern "C" ovl_status ovl_profile_units(ovl_ctx* c, int cls, double* units) {
   if (!c || cls < 0 || cls >= OVL_PROF_CLASSES || !units) return OVL_EINVAL;
   prof_flush(c);

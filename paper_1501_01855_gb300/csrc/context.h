@@ -86,6 +86,8 @@ struct ovl_ctx {
   int lz_cap = 0;
   unsigned int* lzp_bar = nullptr;  // barrier and flags of the one-launch Lanczos iteration
   double* lzp_part = nullptr;       // its blocks' partial sums
+  ovl::LzpShape lzp_shape;          // shape of the last one
+  long long lz_cycles[2] = {0, 0};  // Lanczos cycles as one launch, by launches per step
   int nsm = 0;                      // SMs of the device
   unsigned long long wait_ns = 2000000000ull;   // limit of the bounded waits inside kernels
   void* lz_pool = nullptr;       // stored Lanczos bases of every sign precision (one at a time)

@@ -532,11 +532,12 @@ __global__ void __launch_bounds__(2 * P * G * TB + 32, 1) lz_persistent_df_kerne
   lzp_run(p, body, sh);
 }
 template <int G, int P, int TB>
-bool lzp_df(LzPersist& p, int nsm, cudaStream_t st) {
+bool lzp_df(LzPersist& p, LzpShape* shape, int nsm, cudaStream_t st) {
   p.ntile = ((p.a.g.V >> 1) + P - 1) / P * p.a.nrhs;
   p.tb = (p.ntile + nsm - 1) / nsm;
+  *shape = {G, p.tb};
   return p.tb <= TB && lzp_launch(lz_persistent_df_kernel<G, P, TB>, p, 2 * P * G / 32,
-                                  sizeof(ulonglong2) * G * 12 * 2 * P, nsm, st);
+                                  sizeof(ulonglong2) * G * 12 * 2 * P, TB, nsm, st);
 }
 
 }  // namespace
@@ -547,9 +548,10 @@ bool lzp_df(LzPersist& p, int nsm, cudaStream_t st) {
 // registers), two on 16 pairs up to 34048. Sign to 1e-10 with four / two groups, ms: 10080 sites 2.60 /
 // 3.82, 12288 2.62 / 3.68, 16384 2.99 / 3.87, 20000 3.92 / 4.15, 20480 3.95 / 4.05. Requesting the
 // epilogue's operands before the hops made every size slower (4^4 1.35 -> 1.39 ms).
-bool launch_lz_persistent_df(LzPersist& p, int nsm, cudaStream_t st) {
-  return lzp_df<8, 8, 3>(p, nsm, st) || lzp_df<8, 8, 4>(p, nsm, st) || lzp_df<4, 8, 7>(p, nsm, st) ||
-         lzp_df<4, 8, 9>(p, nsm, st) || lzp_df<2, 16, 5>(p, nsm, st) || lzp_df<2, 16, 7>(p, nsm, st);
+bool launch_lz_persistent_df(LzPersist& p, LzpShape* shape, int nsm, cudaStream_t st) {
+  return lzp_df<8, 8, 3>(p, shape, nsm, st) || lzp_df<8, 8, 4>(p, shape, nsm, st) ||
+         lzp_df<4, 8, 7>(p, shape, nsm, st) || lzp_df<4, 8, 9>(p, shape, nsm, st) ||
+         lzp_df<2, 16, 5>(p, shape, nsm, st) || lzp_df<2, 16, 7>(p, shape, nsm, st);
 }
 
 // Two threads per pair and system, times 1, 2, 4 or 8 groups. One group is the cheapest form

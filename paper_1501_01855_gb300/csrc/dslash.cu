@@ -642,7 +642,8 @@ static DArgs base_args(const Geom& g, double kappa, LinkRef links, int nrhs) {
 }
 
 bool launch_lz_persistent(int prec, const Geom& g, double kappa, LinkRef links, SpinorRef W, SpinorRef t, int nrhs,
-                          const LzCtl& ctl, double* part, unsigned int* bar, int nsm, cudaStream_t st) {
+                          const LzCtl& ctl, double* part, unsigned int* bar, LzpShape* shape, int nsm,
+                          cudaStream_t st) {
   if (nrhs > LZP_SYS) return false;
   LzPersist p;
   p.a = base_args(g, kappa, links, nrhs);
@@ -658,14 +659,17 @@ bool launch_lz_persistent(int prec, const Geom& g, double kappa, LinkRef links, 
   p.t = t;
   p.part = part;
   p.bar = bar;
-  if (prec == P64E) return launch_lz_persistent_df(p, nsm, st);
+  if (prec == P64E) return launch_lz_persistent_df(p, shape, nsm, st);
   if (prec != P32) return false;
   // FP32: every tile has its warps at once, up to 27 per SM (72 registers; up to 19: 102)
   p.ntile = (g.V + 31) / 32 * nrhs;
   p.tb = (p.ntile + nsm - 1) / nsm;
-  if (4 * p.tb <= 19) return lzp_launch(lz_persistent_f32_kernel<4, 20>, p, 4, 4 * 12 * 32 * sizeof(cpx<float>), nsm, st);
-  if (p.tb <= 19) return lzp_launch(lz_persistent_f32_kernel<1, 20>, p, 1, 0, nsm, st);
-  if (p.tb <= LZP_WARPS - 1) return lzp_launch(lz_persistent_f32_kernel<1, LZP_WARPS>, p, 1, 0, nsm, st);
+  *shape = {4 * p.tb <= 19 ? 4 : 1, p.tb};
+  if (4 * p.tb <= 19)
+    return lzp_launch(lz_persistent_f32_kernel<4, 20>, p, 4, 4 * 12 * 32 * sizeof(cpx<float>), 4, nsm, st);
+  if (p.tb <= 19) return lzp_launch(lz_persistent_f32_kernel<1, 20>, p, 1, 0, 19, nsm, st);
+  if (p.tb <= LZP_WARPS - 1)
+    return lzp_launch(lz_persistent_f32_kernel<1, LZP_WARPS>, p, 1, 0, LZP_WARPS - 1, nsm, st);
   return false;
 }
 

@@ -684,10 +684,13 @@ static ovl_status sign_op_batch_lz(ovl_ctx* c, int mode, const Field& v, int vof
   for (int cycle = 0;; ++cycle) {
     int chunk = 8;
     if (persist) {
+      LzpShape shape;
       OVL_CUDA(c, cudaMemsetAsync(c->lzp_bar, 0, sizeof(unsigned int) * LZP_WORDS, c->st));
       persist = launch_lz_persistent(PL, c->g, c->kappa, L, W->ref(), t->ref(), n, ctl, c->lzp_part, c->lzp_bar,
-                                     c->nsm, c->st);
+                                     &shape, c->nsm, c->st);
+      if (persist) c->lzp_shape = shape;
     }
+    ++c->lz_cycles[persist ? 0 : 1];
     if (persist) {
       OVL_TRY(check_launch(c, __func__));
       OVL_CUDA(c, cudaMemcpyAsync(hlzp, c->lzp_bar + 1, sizeof(unsigned int), cudaMemcpyDeviceToHost, c->st));

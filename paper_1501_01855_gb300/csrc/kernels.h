@@ -149,8 +149,13 @@ struct LzCtl {
 constexpr int LZP_SYS = 4;         // systems
 constexpr int LZP_BLOCKS = 512;
 constexpr int LZP_WORDS = 2 + 2 * LZP_SYS;
+struct LzpShape {      // what was launched
+  int groups = 0;      // groups of threads (FP32: warps) that share the hops of a tile
+  int tiles = 0;       // tiles per block
+};
 bool launch_lz_persistent(int prec, const Geom& g, double kappa, LinkRef links, SpinorRef W, SpinorRef t, int nrhs,
-                          const LzCtl& ctl, double* part, unsigned int* bar, int nsm, cudaStream_t st);
+                          const LzCtl& ctl, double* part, unsigned int* bar, LzpShape* shape, int nsm,
+                          cudaStream_t st);
 void launch_wilson_lzK(int pw, int plink, int pt, const Geom& g, double kappa, LinkRef links, SpinorRef W,
                        SpinorRef t, int nrhs, double* partials, const LzCtl& ctl, cudaStream_t st);
 void launch_wilson_lzL(int pt, int plink, int pw, const Geom& g, double kappa, LinkRef links, SpinorRef t,

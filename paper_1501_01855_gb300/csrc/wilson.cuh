@@ -496,22 +496,28 @@ __device__ __forceinline__ void lzp_run(const LzPersist& p, Body& body, LzpShare
 // MODE_OVL (P64 or P32), P64E otherwise.
 void run_wilson_df(int mode, int pio, DArgs a, cudaStream_t st);
 // Its Lanczos iteration in one launch; false when the launch is too large for it.
-bool launch_lz_persistent_df(LzPersist& p, int nsm, cudaStream_t st);
+bool launch_lz_persistent_df(LzPersist& p, LzpShape* shape, int nsm, cudaStream_t st);
 // Cooperative launch of p.tb tiles of tw warps per block (and one warp more); false when the blocks
-// do not fit at once.
+// do not fit at once (a block takes each of its tiles once, so none may be missing). max_tiles: the most
+// tiles a block of this kernel takes; its shared memory is the limit that is set, the same on every
+// call, since contexts in other threads launch the same kernel with other sizes.
 template <typename K>
-bool lzp_launch(K kernel, LzPersist& p, int tw, size_t smem_tile, int nsm, cudaStream_t st) {
+bool lzp_launch(K kernel, LzPersist& p, int tw, size_t smem_tile, int max_tiles, int nsm, cudaStream_t st) {
   const int threads = 32 * (p.tb * tw + 1);
   const size_t smem = smem_tile * p.tb;
-  int grid = (p.ntile + p.tb - 1) / p.tb;
-  if (smem > 40 * 1024) cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  const int grid = (p.ntile + p.tb - 1) / p.tb;
+  if (smem_tile * max_tiles > 40 * 1024 &&
+      cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(smem_tile * max_tiles)) !=
+          cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
   int per = 0;
   if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, kernel, threads, smem) != cudaSuccess) {
     cudaGetLastError();
     return false;
   }
-  grid = grid < per * nsm ? grid : per * nsm;
-  if (grid < 1 || grid > LZP_BLOCKS || grid < p.a.nrhs) return false;
+  if (grid < p.a.nrhs || grid > LZP_BLOCKS || grid > per * nsm) return false;
   void* args[] = {&p};
   if (cudaLaunchCooperativeKernel((const void*)kernel, dim3((unsigned)grid), dim3((unsigned)threads), args, smem, st) !=
       cudaSuccess) {
