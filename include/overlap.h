@@ -179,7 +179,9 @@ ovl_status ovl_trim(ovl_ctx* ctx);
 
 /* Limit of the bounded waits inside kernels, in seconds (0..3600; 2 in a new context): those of
  * the tensor-core Gram block, whose calls return OVL_ETIMEOUT when one gives up (the context
- * stays usable). 0 makes every such wait give up at once. */
+ * stays usable), and those between the blocks of a one-launch Lanczos cycle (see
+ * ovl_lanczos_cycles), which is then done again by launches per step. 0 makes every such wait
+ * give up at once. */
 ovl_status ovl_set_wait_limit(ovl_ctx* ctx, double seconds);
 
 /* Host-only (no GPU needed): the Zolotarev rational of order n on a < |x| < b
@@ -497,7 +499,8 @@ ovl_status ovl_wilson_tuning(const ovl_ctx* ctx, int prec, int* variant, double*
 
 /* Cycles of the stored-basis Lanczos (sign_method 0 and 2) since the context was created: run as
  * one cooperative launch (double-float and FP32 signs of up to 4 systems on lattices that the SMs
- * hold at once, with wilson_variant = -1 and use_graphs = 1), and run by launches per step.
+ * hold at once, with wilson_variant = -1 and use_graphs = 1; either switch turns it off), and
+ * run by launches per step.
  * groups, tiles: the shape of the last one-launch cycle (thread groups per tile, tiles per
  * block; 0 when there was none). Any output pointer may be NULL. */
 ovl_status ovl_lanczos_cycles(const ovl_ctx* ctx, long long* one_launch, long long* stepped, int* groups,

@@ -642,8 +642,8 @@ static DArgs base_args(const Geom& g, double kappa, LinkRef links, int nrhs) {
 }
 
 bool launch_lz_persistent(int prec, const Geom& g, double kappa, LinkRef links, SpinorRef W, SpinorRef t, int nrhs,
-                          const LzCtl& ctl, double* part, unsigned int* bar, LzpShape* shape, int nsm,
-                          cudaStream_t st) {
+                          const LzCtl& ctl, double* part, unsigned int* bar, unsigned long long wait_ns,
+                          LzpShape* shape, int nsm, cudaStream_t st) {
   if (nrhs > LZP_SYS) return false;
   LzPersist p;
   p.a = base_args(g, kappa, links, nrhs);
@@ -659,6 +659,7 @@ bool launch_lz_persistent(int prec, const Geom& g, double kappa, LinkRef links, 
   p.t = t;
   p.part = part;
   p.bar = bar;
+  p.wait_ns = wait_ns;
   if (prec == P64E) return launch_lz_persistent_df(p, shape, nsm, st);
   if (prec != P32) return false;
   // FP32: every tile has its warps at once, up to 27 per SM (72 registers; up to 19: 102)

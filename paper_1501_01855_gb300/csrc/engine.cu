@@ -681,13 +681,14 @@ static ovl_status sign_op_batch_lz(ovl_ctx* c, int mode, const Field& v, int vof
   int itmax = 0;
   double comb_bytes = 0.0;
   std::vector<int> it(n, 0), stt(n, 0);
+  std::vector<LzState> before;   // the systems' states after the cycle before
   for (int cycle = 0;; ++cycle) {
     int chunk = 8;
     if (persist) {
       LzpShape shape;
       OVL_CUDA(c, cudaMemsetAsync(c->lzp_bar, 0, sizeof(unsigned int) * LZP_WORDS, c->st));
       persist = launch_lz_persistent(PL, c->g, c->kappa, L, W->ref(), t->ref(), n, ctl, c->lzp_part, c->lzp_bar,
-                                     &shape, c->nsm, c->st);
+                                     c->wait_ns, &shape, c->nsm, c->st);
       if (persist) c->lzp_shape = shape;
     }
     ++c->lz_cycles[persist ? 0 : 1];
@@ -723,7 +724,8 @@ static ovl_status sign_op_batch_lz(ovl_ctx* c, int mode, const Field& v, int vof
     }
     // this cycle's part of y
     prof_begin(c, 5, &pp);
-    launch_lz_coef(c->lz, ahist, bhist, hcap, c->dpoles, c->lz_Y, c->lz_coefW, n, c->st);
+    launch_lz_coef(c->lz, ahist, bhist, hcap, c->dpoles, c->lz_Y, c->lz_coefW, persist ? c->lzp_bar + 1 : nullptr, n,
+                   c->st);
     prof_end(c, &pp, 0.0);
     prof_begin(c, 3, &pp);
     launch_lz_combine(PB, PR, W->ref(), y->ref(), c->lz_coefW, c->lz, hcap, n, V, c->st);
@@ -732,8 +734,23 @@ static ovl_status sign_op_batch_lz(ovl_ctx* c, int mode, const Field& v, int vof
     OVL_CUDA(c, cudaMemcpy2DAsync(hs, sizeof(LzState), c->lz, sizeof(LzRhs), sizeof(LzState), n, cudaMemcpyDeviceToHost,
                                   c->st));
     OVL_CUDA(c, cudaStreamSynchronize(c->st));
-    if (persist && *hlzp)
-      return set_err(c, OVL_ETIMEOUT, "Lanczos iteration of the sign: a bounded wait between its blocks gave up");
+    if (persist && *hlzp) {
+      // A wait between its blocks gave up (another program held the GPU for seconds). Nothing of the
+      // cycle is in y, its first vectors and their norms are as they were: it is done again from
+      // there, and the rest of this sign, by launches per step, which wait for nothing.
+      persist = false;
+      --c->lz_cycles[0];
+      if (cycle > 0) {
+        std::copy(before.begin(), before.end(), hs);
+        OVL_CUDA(c, cudaMemcpy2DAsync(c->lz, sizeof(LzRhs), hs, sizeof(LzState), sizeof(LzState), n,
+                                      cudaMemcpyHostToDevice, c->st));
+      }
+      launch_lz_start(c->lz, c->partials, sh.nsb, n, c->dpoles, d_eta, c->P.mscg_max, cap, cycle == 0, c->st);
+      OVL_TRY(check_launch(c, __func__));
+      --cycle;
+      continue;
+    }
+    before.assign(hs, hs + n);
     bool more = false;
     double cb = (double)n * 2.0 * rbytes;   // y, and the basis vectors of this cycle per system
     for (int j = 0; j < n; ++j) {

@@ -143,8 +143,8 @@ struct LzCtl {
 };
 // A whole cycle of the iteration in one cooperative launch, for launches too small to hide the
 // tail and the dispatch of two launches per step (see lzp_run in wilson.cuh). part: 2 nrhs
-// LZP_BLOCKS doubles; bar: LZP_WORDS zeroed words, word 1 of which is set when a bounded wait gave
-// up. False (nothing launched): this precision or size has no such form, or the device cannot hold
+// LZP_BLOCKS doubles; bar: LZP_WORDS zeroed words, word 1 of which is set when a wait gave up after
+// wait_ns (the cycle's vectors past the first and its systems' states are then unfinished). False (nothing launched): this precision or size has no such form, or the device cannot hold
 // its blocks at once.
 constexpr int LZP_SYS = 4;         // systems
 constexpr int LZP_BLOCKS = 512;
@@ -154,8 +154,8 @@ struct LzpShape {      // what was launched
   int tiles = 0;       // tiles per block
 };
 bool launch_lz_persistent(int prec, const Geom& g, double kappa, LinkRef links, SpinorRef W, SpinorRef t, int nrhs,
-                          const LzCtl& ctl, double* part, unsigned int* bar, LzpShape* shape, int nsm,
-                          cudaStream_t st);
+                          const LzCtl& ctl, double* part, unsigned int* bar, unsigned long long wait_ns,
+                          LzpShape* shape, int nsm, cudaStream_t st);
 void launch_wilson_lzK(int pw, int plink, int pt, const Geom& g, double kappa, LinkRef links, SpinorRef W,
                        SpinorRef t, int nrhs, double* partials, const LzCtl& ctl, cudaStream_t st);
 void launch_wilson_lzL(int pt, int plink, int pw, const Geom& g, double kappa, LinkRef links, SpinorRef t,
@@ -168,9 +168,10 @@ void launch_lz_start(LzRhs* lz, const double* partials, int nsb, int nrhs, const
                      const double* eta, int maxit, int cap, int first, cudaStream_t st);
 // coefficients of the stored vectors in y = sum_i w_i x_i (per system, cap doubles) from
 // the tridiagonal solves; Y is scratch of nrhs * npoles * 2 cap doubles. For a system whose
-// cycle filled up, the weights of the next cycle are set too.
+// cycle filled up, the weights of the next cycle are set too. gave_up (may be null): word 1 of a
+// one-launch cycle's bar; when it is set nothing is formed and the combination adds nothing.
 void launch_lz_coef(LzRhs* lz, const double* ahist, const double* bhist, int cap, const Poles* poles, double* Y,
-                    double* coefW, int nrhs, cudaStream_t st);
+                    double* coefW, const unsigned int* gave_up, int nrhs, cudaStream_t st);
 // y += sum_l coefW[l] W_l for every system with basis vectors this cycle
 void launch_lz_combine(int pw, int py, SpinorRef W, SpinorRef y, const double* coefW, const LzRhs* lz, int cap,
                        int nrhs, int V, cudaStream_t st);

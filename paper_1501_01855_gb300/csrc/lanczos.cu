@@ -223,11 +223,16 @@ void launch_lz_start(LzRhs* lz, const double* partials, int nsb, int nrhs, const
 // A serial chain per pole, so what counts is its latency: one FP64 division per step (160 ns; a
 // multiply-add 31) with the reciprocal kept, T in shared memory, and the backward pass' loads
 // eight at a time ahead of its chain. 115 steps, 20 poles: 180 -> 60 us.
+// gave_up (may be null): set when the one-launch form of the cycle gave up, of which nothing is used.
 __global__ void lz_coef_kernel(LzRhs* lz, const double* ahist, const double* bhist, int cap, const Poles* P,
-                               double* Y, double* coefW) {
+                               double* Y, double* coefW, const unsigned int* gave_up) {
   extern __shared__ double tri[];   // alpha, beta: cap each
   const int rhs = blockIdx.x;
   LzRhs& L = lz[rhs];
+  if (gave_up != nullptr && *gave_up != 0u) {
+    if (threadIdx.x == 0) L.j = 0;   // no vectors to combine
+    return;
+  }
   const int k = L.j;
   const int np = P->n;
   double *al = tri, *be = tri + cap;
@@ -289,8 +294,8 @@ __global__ void lz_coef_kernel(LzRhs* lz, const double* ahist, const double* bhi
 }
 
 void launch_lz_coef(LzRhs* lz, const double* ahist, const double* bhist, int cap, const Poles* poles, double* Y,
-                    double* coefW, int nrhs, cudaStream_t st) {
-  lz_coef_kernel<<<nrhs, 128, 2 * sizeof(double) * (size_t)cap, st>>>(lz, ahist, bhist, cap, poles, Y, coefW);
+                    double* coefW, const unsigned int* gave_up, int nrhs, cudaStream_t st) {
+  lz_coef_kernel<<<nrhs, 128, 2 * sizeof(double) * (size_t)cap, st>>>(lz, ahist, bhist, cap, poles, Y, coefW, gave_up);
 }
 
 // ---------------------------------------------------------------- combine

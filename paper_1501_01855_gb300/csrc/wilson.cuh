@@ -256,6 +256,7 @@ struct LzPersist {
   double* part;        // [phase][system][block]
   unsigned int* bar;   // arrivals, error, stop flags set in K phases, in L phases (each read in the other)
   int tb, ntile;       // tiles a block holds at a time, tiles of the launch
+  unsigned long long wait_ns;   // limit of a barrier's wait
 };
 struct LzCoef {        // what the epilogues take from LzRhs
   float2 fn, fa, fb;
@@ -274,8 +275,12 @@ __device__ __forceinline__ unsigned int lzp_acquire(const unsigned int* p) {
   return v;
 }
 // One lane of the block: arrive and wait for the k-th barrier of the grid. The wait ends after
-// 2 s, or when another block has given up; the launch then ends everywhere.
-__device__ __forceinline__ int lzp_barrier(unsigned int* bar, unsigned int target) {
+// the limit (zero: at once), or when another block has given up; the launch then ends everywhere.
+__device__ __forceinline__ int lzp_barrier(unsigned int* bar, unsigned int target, unsigned long long limit) {
+  if (limit == 0) {
+    atomicExch(bar + 1, 1u);
+    return 0;
+  }
   __threadfence();
   atomicAdd(bar, 1u);
   unsigned long long t0 = 0;
@@ -286,7 +291,7 @@ __device__ __forceinline__ int lzp_barrier(unsigned int* bar, unsigned int targe
       asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
       if (t0 == 0) t0 = t;
       if (lzp_acquire(bar + 1) != 0u) return 0;
-      if (t - t0 > 2000000000ull) {
+      if (t - t0 > limit) {
         atomicExch(bar + 1, 1u);
         return 0;
       }
@@ -484,7 +489,7 @@ __device__ __forceinline__ void lzp_run(const LzPersist& p, Body& body, LzpShare
           for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
           if (lane == 0) __stcg(p.part + (size_t)(phase * n + s) * LZP_BLOCKS + blockIdx.x, v);
         }
-        if (lane == 0) sh.ok = lzp_barrier(p.bar, target);
+        if (lane == 0) sh.ok = lzp_barrier(p.bar, target, p.wait_ns);
       }
       lzp_block_barrier();
       if (!sh.ok) return;
