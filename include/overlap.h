@@ -489,11 +489,13 @@ ovl_status ovl_bench_wilson(ovl_ctx* ctx, int prec, int n, int iters, double* ms
 ovl_status ovl_bench_fp32(ovl_ctx* ctx, double* fma_per_s);
 
 /* Wilson-kernel autotuner result for one storage precision (OVL_PREC_*): the variant
- * in use (0 one thread per site, 1 one thread per site and direction, 2 4D tiles, 3 two
- * threads per site, one per half spinor, double-float only) and the measured
- * milliseconds per launch of each on this lattice (zero when the variant was forced, does
- * not apply to the precision or, for tiles, when the lattice does not divide into them).
- * Any output pointer may be NULL. */
+ * in use for launches of fewer than 4 systems (0 one thread per site, 1 one thread per site and
+ * direction, 2 4D tiles; double-float: 0, 3, 2, 1 for 1, 2, 4, 8 thread groups per pair of sites)
+ * and the measured milliseconds per launch of one system of each on this lattice (zero when the
+ * variant was forced, does not apply to the precision or, for tiles, when the lattice does not
+ * divide into them). The double-float kernel takes its groups from the size of each launch: its
+ * variant is the one for one system, its times are for information. Any output pointer may be
+ * NULL. */
 ovl_status ovl_wilson_tuning(const ovl_ctx* ctx, int prec, int* variant, double* ms_thread_per_site,
                              double* ms_split, double* ms_tiled, double* ms_pair);
 

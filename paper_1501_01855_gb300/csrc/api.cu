@@ -150,7 +150,8 @@ static ovl_status autotune_wilson(ovl_ctx* c) {
   OVL_CUDA(c, cudaEventCreate(&e1));
   for (int p = 0; p < 4; ++p) {
     if (forced >= 0 && forced <= 3) {
-      c->wvar[p] = (forced == 2 && !wilson_tiles_fit(c->g)) || (forced == 3 && p != P64E) ? 0 : forced;
+      // double-float: numbers of thread groups, on any lattice; else tiles that fit, and no variant 3
+      c->wvar[p] = p != P64E && ((forced == 2 && !wilson_tiles_fit(c->g)) || forced == 3) ? 0 : forced;
       c->wvar_multi[p] = c->wvar[p];
       continue;
     }
@@ -168,7 +169,6 @@ static ovl_status autotune_wilson(ovl_ctx* c) {
         break;
       }
       for (int v = 0; v < nv; ++v) {
-        if (v == 2 && !wilson_tiles_fit(c->g)) continue;
         LinkRef L = links_of(c, p);
         L.variant = L.variant_multi = v;
         const int reps = p == P64 ? 3 : bucket == 0 ? 8 : 4;
