@@ -119,8 +119,8 @@ __device__ __forceinline__ bool warp_wait(uint32_t bar, uint32_t parity, volatil
 
 // a <- fl(a + b); the rounding error
 __device__ __forceinline__ float two_sum(float& a, float b) {
-  const float s = __fadd_rn(a, b), v = __fsub_rn(s, a);
-  const float e = __fadd_rn(__fsub_rn(a, __fsub_rn(s, v)), __fsub_rn(b, v));
+  const float s = a + b, v = s - a;
+  const float e = (a - (s - v)) + (b - v);
   a = s;
   return e;
 }
@@ -162,15 +162,14 @@ struct TgLoad<P32> {
 // others in [-64, 64], and x 2^-e = sum_s d_s 2^(-7 (s + 1)) up to 2^-43. A digit is an integer of
 // at most 8 bits, so the upper half of its float is its exact BF16.
 // FP32 operands: r by two power-of-two factors. FP64 operands, from their bits (conversions from
-// FP64 are slow): r is the float of the leading 24 bits; the next 22 bits, with a last bit that says
-// whether any bit below them is set (rounding to odd), are a second float that joins the remainder
-// after three digits, when 21 of the leading bits are spent (the third digit is chosen with them, so
-// that the fourth stays in its range). That sum is exact in FP32 for elements above 2^(e-1), but for a
-// remainder that the choice of the third digit left past one half, and is rounded at 2^-47 or finer
-// below, so the last digit's rounding, at 2^-43, is that of all 53 bits up to 9/8 of it and has no bias;
-// cutting the low bits off instead put 1.0e-14 on every diagonal entry of Gaussian data. About 80
-// instructions per element, against 270 for taking the digits out of a 64-bit fixed-point integer: a
-// 64 x 64 tile on 16^4 1.43 -> 0.81 ms with the pipeline below.
+// FP64 are slow): r is the float of the leading 24 bits; the other 29, rounded to a second float
+// (a 32-bit integer conversion, on a pipe that is idle otherwise), join the remainder after three
+// digits, when 21 of the leading bits are spent (the third digit is chosen with them, so that the
+// fourth stays in its range; that sum is rounded at 2^-46 or finer). Every rounding is to nearest, so
+// an element is off by 2^-43, in rare cases up to 9/8 of that, without bias; cutting at 47 bits instead
+// put 1.0e-14 on every diagonal entry of Gaussian data. About 75 instructions per element, against
+// 270 for taking the digits out of a 64-bit fixed-point integer: a 64 x 64 tile on 16^4 1.43 -> 0.81 ms
+// with the pipeline below.
 __device__ __forceinline__ float tg_pow2(int k) { return __int_as_float((127 + k) << 23); }
 // the digit of s (r itself, or r and what follows it, rounded); r becomes its remainder
 __device__ __forceinline__ uint32_t tg_digit(f2 s, f2& r) {
@@ -186,12 +185,11 @@ __device__ __forceinline__ void tg_split64(uint2 w, int e, int thr, uint32_t fli
   const uint32_t sg = (w.y ^ flip) & 0x80000000u;
   const int ex = t - 896 - e;   // exponent field of the float, <= 126
   const uint32_t m = __funnelshift_l(w.x, w.y, 3) & 0x7FFFFFu;
-  // the next 22 bits, and 1 when any bit below them is set: v 2^(t - 1023 - 46 - e), times 2^21 in lo
-  const uint32_t v = ((w.x >> 6) & 0x7FFFFEu) | ((w.x & 0x7Fu) != 0u ? 1u : 0u);
   const bool z = t < thr;
   hi = __uint_as_float(z ? 0u : ((uint32_t)ex << 23) | m | sg);
-  const float f = __fsub_rn(__uint_as_float(0x4B000000u | v), 8388608.0f);
-  lo = __fmul_rn(f, __uint_as_float(z || ex <= 25 ? 0u : ((uint32_t)(ex - 25) << 23) | sg));
+  // the other 29 bits v, rounded to 24: v 2^(t - 1023 - 52 - e), times 2^21 in lo
+  const float f = __uint2float_rn(w.x & 0x1FFFFFFFu);
+  lo = __fmul_rn(f, __uint_as_float(z || ex <= 31 ? 0u : ((uint32_t)(ex - 31) << 23) | sg));
 }
 template <int P>
 __device__ __forceinline__ void tg_digits(uint4 w4, int e, bool neg, uint32_t pd[TG_S]) {
@@ -325,46 +323,40 @@ __global__ void __launch_bounds__(TG_THREADS, 1)
 #pragma unroll
   for (int c = 0; c < TG_CPT; ++c) acc_h[c] = acc_l[c] = 0.f;
 
-  // One accumulation chunk's group sums are exact integers in FP32: summed, scaled, in
-  // double-float from the smallest weight up, then one double-float addition to the running sum,
-  // which stays normalised (|low| <= half an ulp of high): however many chunks a CTA sums, each
-  // adds one rounding of 2^-48. Every warp, once the chunk's MMAs are done (fbar); false when a
-  // wait gave up.
+  // One accumulation chunk's group sums are exact integers in FP32: add them, scaled, in
+  // double-float, and normalise the sum (|low| <= half an ulp of high), so that a low word never
+  // holds more than the errors of one chunk: however many chunks a CTA sums, each adds roundings of
+  // about 2^-48. Every warp, once the chunk's MMAs are done (fbar); false when a wait gave up.
   auto flush = [&](int chunk) -> bool {
     if (!warp_wait(smem_u32(&fbar), (uint32_t)chunk & 1u, &abort_flag, wait_ns)) return false;
     asm volatile("tcgen05.fence::after_thread_sync;");
-    constexpr int NC = 8;   // columns at a time (registers)
 #pragma unroll
-    for (int c0 = 0; c0 < TG_CPT; c0 += NC) {
-      float ch[NC], cl[NC];
+    for (int g = 0; g < TG_G; ++g) {
+      uint32_t v[TG_CPT];
+      static_assert(TG_CPT == 16, "the flush reads 16 columns per thread");
+      const uint32_t ta_ = tmem + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)(g * TG_NB + cbase);
+      asm volatile(
+          "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
+          : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]),
+            "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]), "=r"(v[15])
+          : "r"(ta_));
+      // the wait names the registers: nothing that uses them moves above it
+      asm volatile("tcgen05.wait::ld.sync.aligned;"
+                   : "+r"(v[0]), "+r"(v[1]), "+r"(v[2]), "+r"(v[3]), "+r"(v[4]), "+r"(v[5]), "+r"(v[6]), "+r"(v[7]),
+                     "+r"(v[8]), "+r"(v[9]), "+r"(v[10]), "+r"(v[11]), "+r"(v[12]), "+r"(v[13]), "+r"(v[14]),
+                     "+r"(v[15])::"memory");
+      const float w = __int_as_float((127 - 7 * (g + 2)) << 23);   // 2^(-7 (g + 2))
 #pragma unroll
-      for (int g = TG_G - 1; g >= 0; --g) {
-        uint32_t v[NC];
-        const uint32_t ta_ = tmem + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)(g * TG_NB + cbase + c0);
-        asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
-                     : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7])
-                     : "r"(ta_));
-        asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-        const float w = __int_as_float((127 - 7 * (g + 2)) << 23);   // 2^(-7 (g + 2))
-#pragma unroll
-        for (int c = 0; c < NC; ++c) {
-          const float x = __uint_as_float(v[c]) * w;   // exact
-          if (g == TG_G - 1) {
-            ch[c] = x;
-            cl[c] = 0.f;
-          } else {
-            cl[c] += two_sum(ch[c], x);
-          }
-        }
+      for (int c = 0; c < TG_CPT; ++c) {
+        const float x = __uint_as_float(v[c]) * w;   // exact
+        acc_l[c] += two_sum(acc_h[c], x);
       }
+    }
 #pragma unroll
-      for (int c = 0; c < NC; ++c) {
-        float &h = acc_h[c0 + c], &l = acc_l[c0 + c];
-        l = __fadd_rn(two_sum(h, ch[c]), __fadd_rn(l, cl[c]));
-        const float r = __fadd_rn(h, l);
-        l = __fsub_rn(l, __fsub_rn(r, h));
-        h = r;
-      }
+    for (int c = 0; c < TG_CPT; ++c) {
+      const float h = acc_h[c] + acc_l[c];
+      acc_l[c] -= h - acc_h[c];
+      acc_h[c] = h;
     }
     asm volatile("tcgen05.fence::before_thread_sync;");
     __syncwarp();

@@ -1,7 +1,6 @@
 """FP64 operands of the tensor-core Gram blocks are rounded, not cut, to their six digits: a host
-model of the splitting (leading 24 bits, the next 22 with a last bit that says whether anything lies
-below them, digits by FP32 arithmetic) over many elements at once. Elements on the grid are exact, an
-element is off by at most 9/8 2^-43 of its vector's scale, by the mean of a rounding (no bias; cutting
+model of the splitting (leading 24 bits, the other 29 rounded to 24, digits by FP32 arithmetic) over
+many elements at once. Elements on the grid are exact, an element is off by at most 9/8 2^-43 of its vector's scale, by the mean of a rounding (no bias; cutting
 gives 2^-47), digits stay in the ranges of the exact FP32 sums. On the GPU: diagonal entries of
 Gaussian vectors have no common offset."""
 import numpy as np
@@ -24,8 +23,8 @@ def split64(x, e):
     zero = t < max(e + 897, 1)
     ex = np.where(zero, 1, t - 896 - e)
     h = ((ex << 23).astype(np.uint32) | ((b >> np.uint64(29)) & np.uint64(0x7fffff)).astype(np.uint32) | sg).view(F)
-    v = ((lo >> np.uint64(6)) & np.uint64(0x7ffffe)).astype(F) + ((lo & np.uint64(0x7f)) != 0).astype(F)
-    scale = np.where(ex <= 25, np.uint32(0), (np.maximum(ex - 25, 0) << 23).astype(np.uint32) | sg).view(F)
+    v = (lo & np.uint64(0x1fffffff)).astype(F)
+    scale = np.where(ex <= 31, np.uint32(0), (np.maximum(ex - 31, 0) << 23).astype(np.uint32) | sg).view(F)
     return np.where(zero, F(0), h), np.where(zero, F(0), v * scale)
 
 
