@@ -10,6 +10,7 @@
 // leaves its half of the lattice.
 #pragma once
 #include "common.cuh"
+#include "threeword.h"
 
 namespace ovl {
 
@@ -158,6 +159,19 @@ __device__ __forceinline__ double dot2p_get(dot2p d) {
   double a, b;
   dd2_to({d.s, d.c}, a, b);
   return a + b;
+}
+
+// the sum of a warp's pairs, both lanes of each, on lane 0: a fixed tree in three words
+__device__ __forceinline__ double dot2p_warp_sum(dot2p d) {
+  float s0, s1, c0, c1;
+  upk(d.s, s0, s1);
+  upk(d.c, c0, c1);
+  ThreeWord v = ThreeWord{s0, c0, 0.f} + ThreeWord{s1, c1, 0.f};
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1)
+    v = v + ThreeWord{__shfl_down_sync(0xffffffffu, v.a, o), __shfl_down_sync(0xffffffffu, v.b, o),
+                      __shfl_down_sync(0xffffffffu, v.c, o)};
+  return to_double(v);
 }
 
 // real number r (0 re, 1 im) of complex component k of the pair (i, i + V/2) of field fld;

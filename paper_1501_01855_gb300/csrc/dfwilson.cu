@@ -234,7 +234,7 @@ __global__ void __launch_bounds__(2 * P * G, df_resident(G, P)) df_wilson_kernel
   constexpr int NR = nred(MODE);
   extern __shared__ ulonglong2 part[];   // G > 1: [z][component (6 x re, im)][thread x]
   constexpr int NW = 2 * P * G / 32;   // warps
-  __shared__ float2 red[NW][NR];
+  __shared__ double red[NW][NR];
   const int half = threadIdx.x & 1;
   const int grp = G > 1 ? threadIdx.z : 0;
   const int sb = blockIdx.x / a.nrhs;   // the systems of one site block together: they share its links in L1 / L2
@@ -357,25 +357,19 @@ __global__ void __launch_bounds__(2 * P * G, df_resident(G, P)) df_wilson_kernel
     }
   }
   if (a.partials != nullptr) {
-    // lanes in double-float, a fixed tree; then FP64 over the warps in the order z, x
+    // lanes in three words, a fixed tree; then FP64 over the warps in the order z, x
     const int lin = threadIdx.z * 2 * P + threadIdx.x;
 #pragma unroll
     for (int q = 0; q < NR; ++q) {
-      float s0, s1, c0, c1;
-      upk(d[q].s, s0, s1);
-      upk(d[q].c, c0, c1);
-      df v = df(s0, c0) + df(s1, c1);
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1)
-        v = v + df(__shfl_down_sync(0xffffffffu, v.hi, o), __shfl_down_sync(0xffffffffu, v.lo, o));
-      if ((lin & 31) == 0) red[lin >> 5][q] = make_float2(v.hi, v.lo);
+      const double v = dot2p_warp_sum(d[q]);
+      if ((lin & 31) == 0) red[lin >> 5][q] = v;
     }
     __syncthreads();
     if (threadIdx.x == 0 && threadIdx.z == 0) {
       double tot[NVRED] = {0.0, 0.0, 0.0, 0.0};
 #pragma unroll
       for (int q = 0; q < NR; ++q)
-        for (int w = 0; w < NW; ++w) tot[q] += (double)red[w][q].x + (double)red[w][q].y;
+        for (int w = 0; w < NW; ++w) tot[q] += red[w][q];
       store_partials<MODE>(a, rhs, sb, tot);
     }
   }
@@ -514,14 +508,8 @@ struct LzpBodyDf {
                                    q < 3 ? 3 * half + q : 3 + 3 * half + q, i, t, d);
       }
     }
-    float s0, s1, c0, c1;
-    upk(d[0].s, s0, s1);
-    upk(d[0].c, c0, c1);
-    df v = df(s0, c0) + df(s1, c1);
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1)
-      v = v + df(__shfl_down_sync(0xffffffffu, v.hi, o), __shfl_down_sync(0xffffffffu, v.lo, o));
-    if (lane_id() == 0) sh.acc[threadIdx.x >> 5][rhs] = (double)v;
+    const double v = dot2p_warp_sum(d[0]);
+    if (lane_id() == 0) sh.acc[threadIdx.x >> 5][rhs] = v;
   }
 };
 template <int G, int P, int TB>
