@@ -315,17 +315,17 @@ struct LinkRef {
   int variant_multi; // the variant chosen for launches of 4 or more systems
 };
 
-// row 3 = conj(row 1 x row 2)
+// row 3 = conj(row 1 x row 2); the product with a diagonal entry last, of which the real parts' last (the
+// largest on smooth fields: the fewest roundings of the size of the result)
 template <typename T>
 __device__ __forceinline__ void reconstruct_row3(cpx<T> u[9]) {
-  auto minor = [](cpx<T> a, cpx<T> b, cpx<T> c, cpx<T> d) {   // conj(a b - c d)
-    cpx<T> t = a * b;
-    cmac(t, -c, d);
-    return conj(t);
+  auto minor = [](cpx<T> a, cpx<T> b, cpx<T> c, cpx<T> d) {   // conj(c d - a b)
+    const cpx<T> t = -a * b;
+    return cmk(fma(c.r, d.r, fma(-c.i, d.i, t.r)), fma(-c.r, d.i, fma(-c.i, d.r, -t.i)));
   };
-  u[6] = minor(u[1], u[5], u[2], u[4]);
-  u[7] = minor(u[2], u[3], u[0], u[5]);
-  u[8] = minor(u[0], u[4], u[1], u[3]);
+  u[6] = minor(-u[1], u[5], -u[2], u[4]);
+  u[7] = minor(-u[2], u[3], -u[0], u[5]);
+  u[8] = minor(u[1], u[3], u[0], u[4]);
 }
 
 template <int P> struct LinkIO;

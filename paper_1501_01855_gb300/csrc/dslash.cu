@@ -98,30 +98,37 @@ __device__ __forceinline__ void accumulate(cpx<T> acc[12], const cpx<T> w[6]) {
 
 // The six products of a real number as two chains of multiply-adds of three and their sum: 7
 // operations (a sum of three complex products takes 8) with partial sums no larger than there; one
-// chain of six takes 6 but rounds larger partial sums, and its error against 64 bits was
-// larger than before (FP64 K 1.5e-16 against 1.4e-16). With the stored third row: K of 12 FP64 systems on
-// 16^3 x 32 4.16 -> 3.15 ms, FP32 sign of 12 systems 21.3 -> 20.7 ms. S = +1: a b, -1: conj(a) b.
+// chain of six takes 6 but rounds larger partial sums (error of FP64 K against 64 bits 1.5e-16
+// against 1.4e-16). The diagonal entry of the row comes last in both chains: on smooth fields it is
+// nearly one and the others are small, so that only two of the seven roundings are of the size of
+// the sum, three on average in the order of the columns: FP32 K on 24^3 x 48 5.45e-8 of the norm,
+// 5.70e-8 in the order of the columns, 5.65e-8 as three products. With the stored third row: K of 12 FP64 systems on 16^3 x 32 4.16 -> 3.15 ms,
+// FP32 sign of 12 systems 21.3 -> 20.7 ms. S = +1: a b, -1: conj(a) b; (a2, b2) the diagonal entry's.
 template <int S, typename T>
 __device__ __forceinline__ cpx<T> dot3(cpx<T> a0, cpx<T> b0, cpx<T> a1, cpx<T> b1, cpx<T> a2, cpx<T> b2) {
   const T i0 = S > 0 ? a0.i : -a0.i, i1 = S > 0 ? a1.i : -a1.i, i2 = S > 0 ? a2.i : -a2.i;
-  return {fma(a1.r, b1.r, fma(-i0, b0.i, a0.r * b0.r)) + fma(-i2, b2.i, fma(a2.r, b2.r, -i1 * b1.i)),
-          fma(a1.r, b1.i, fma(i0, b0.r, a0.r * b0.i)) + fma(i2, b2.r, fma(a2.r, b2.i, i1 * b1.r))};
+  return {fma(a2.r, b2.r, fma(-i0, b0.i, a0.r * b0.r)) + fma(-i2, b2.i, fma(-i1, b1.i, a1.r * b1.r)),
+          fma(a2.r, b2.i, fma(i0, b0.r, a0.r * b0.i)) + fma(i2, b2.r, fma(i1, b1.r, a1.r * b1.i))};
 }
 template <typename T>
 __device__ __forceinline__ void su3_mul(const cpx<T> u[9], const cpx<T> h[6], cpx<T> w[6]) {
 #pragma unroll
   for (int sp = 0; sp < 2; ++sp)
 #pragma unroll
-    for (int a = 0; a < 3; ++a)
-      w[3 * sp + a] = dot3<1>(u[3 * a], h[3 * sp], u[3 * a + 1], h[3 * sp + 1], u[3 * a + 2], h[3 * sp + 2]);
+    for (int a = 0; a < 3; ++a) {
+      const int b = (a + 1) % 3, c = (a + 2) % 3;
+      w[3 * sp + a] = dot3<1>(u[3 * a + b], h[3 * sp + b], u[3 * a + c], h[3 * sp + c], u[4 * a], h[3 * sp + a]);
+    }
 }
 template <typename T>
 __device__ __forceinline__ void su3_dag_mul(const cpx<T> u[9], const cpx<T> h[6], cpx<T> w[6]) {
 #pragma unroll
   for (int sp = 0; sp < 2; ++sp)
 #pragma unroll
-    for (int a = 0; a < 3; ++a)
-      w[3 * sp + a] = dot3<-1>(u[a], h[3 * sp], u[3 + a], h[3 * sp + 1], u[6 + a], h[3 * sp + 2]);
+    for (int a = 0; a < 3; ++a) {
+      const int b = (a + 1) % 3, c = (a + 2) % 3;
+      w[3 * sp + a] = dot3<-1>(u[3 * b + a], h[3 * sp + b], u[3 * c + a], h[3 * sp + c], u[4 * a], h[3 * sp + a]);
+    }
 }
 
 // Per-thread sums for the epilogue reductions, kept in the compute type: GB300 runs
