@@ -466,8 +466,9 @@ ovl_status ovl_bench_gram(ovl_ctx* ctx, int prec, int na, int nb, int method, in
  * enabled: per kernel class, launches, total milliseconds and algorithmic bytes.
  * Classes: 0 Wilson FP64, 1 Wilson FP32, 2 Wilson FP16-storage, 3 multi-shift
  * update, 4 vector ops, 5 reductions/scalars, 6 Gram/rotate, 7 force, 8 Wilson
- * double-float. While enabled, the multi-shift iterations are launched one by one
- * (not as CUDA graphs) so that every launch can be timed. */
+ * double-float. While enabled, iterations that otherwise run as CUDA graphs are launched one by
+ * one so that every launch can be timed; a one-launch Lanczos cycle (ovl_lanczos_cycles) stays one
+ * launch of its Wilson class. */
 enum { OVL_PROF_CLASSES = 9 };
 ovl_status ovl_profile_enable(ovl_ctx* ctx, int on);
 ovl_status ovl_profile_reset(ovl_ctx* ctx);

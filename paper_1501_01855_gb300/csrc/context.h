@@ -169,6 +169,7 @@ ovl_status ensure_work(ovl_ctx* c, size_t ndoubles);
 // profiling
 void prof_begin(ovl_ctx* c, int cls, ProfPair* p);
 void prof_end(ovl_ctx* c, ProfPair* p, double bytes);
+void prof_cancel(ovl_ctx* c, ProfPair* p);   // nothing was launched since prof_begin
 void prof_flush(ovl_ctx* c);
 
 LinkRef links_of(const ovl_ctx* c, int prec);

@@ -250,6 +250,12 @@ void prof_end(ovl_ctx* c, ProfPair* p, double bytes) {
   if (c->prof.pending.size() > 4096) prof_flush(c);
 }
 
+void prof_cancel(ovl_ctx* c, ProfPair* p) {
+  if (!c->prof.on) return;
+  c->prof.pool.push_back(p->a);
+  c->prof.pool.push_back(p->b);
+}
+
 void prof_flush(ovl_ctx* c) {
   if (c->prof.pending.empty()) return;
   cudaEventSynchronize(c->prof.pending.back().b);
@@ -649,7 +655,7 @@ static ovl_status sign_op_batch_lz(ovl_ctx* c, int mode, const Field& v, int vof
 
   // A small sign runs each cycle as one cooperative launch; a larger one, one with a forced launch
   // shape, or one on a device that cannot hold its blocks, as cached graphs of kGraphIters steps.
-  bool persist = !c->prof.on && c->P.use_graphs && c->P.wilson_variant < 0 && n <= LZP_SYS;
+  bool persist = c->P.use_graphs && c->P.wilson_variant < 0 && n <= LZP_SYS;
   unsigned int* hlzp = reinterpret_cast<unsigned int*>(c->hpin + 12288 + 4096);
   cudaGraphExec_t gexec = nullptr;
   auto get_graph = [&]() -> ovl_status {
@@ -687,9 +693,15 @@ static ovl_status sign_op_batch_lz(ovl_ctx* c, int mode, const Field& v, int vof
     if (persist) {
       LzpShape shape;
       OVL_CUDA(c, cudaMemsetAsync(c->lzp_bar, 0, sizeof(unsigned int) * LZP_WORDS, c->st));
+      prof_begin(c, wcls, &pp);
       persist = launch_lz_persistent(PL, c->g, c->kappa, L, W->ref(), t->ref(), n, ctl, c->lzp_part, c->lzp_bar,
                                      c->wait_ns, &shape, c->nsm, c->st);
-      if (persist) c->lzp_shape = shape;
+      if (persist) {
+        prof_end(c, &pp, 0.0);
+        c->lzp_shape = shape;
+      } else {
+        prof_cancel(c, &pp);
+      }
     }
     ++c->lz_cycles[persist ? 0 : 1];
     if (persist) {
