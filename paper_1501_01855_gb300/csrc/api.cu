@@ -1324,7 +1324,7 @@ extern "C" ovl_status ovl_bench_wilson(ovl_ctx* c, int prec, int n, int iters, d
   cudaEventDestroy(e1);
   OVL_TRY(check_launch(c, __func__));
   const double sb = prec == P16 ? 52 : spinor_site_bytes(prec);
-  const double lb = prec == P64E ? 576 : prec == P64 ? 384 : prec == P32 ? 192 : 96;   // algorithmic
+  const double lb = link_site_bytes(prec);
   if (ms_per_launch) *ms_per_launch = ms / iters;
   if (bytes_per_launch) *bytes_per_launch = (double)c->V * (2.0 * sb * n + lb);
   return OVL_OK;

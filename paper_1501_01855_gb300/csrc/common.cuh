@@ -133,6 +133,11 @@ template <> struct Real<P64> { using T = double; };
 template <> struct Real<P64E> { using T = df; };
 
 __host__ __device__ constexpr int spinor_site_bytes(int p) { return p == P32 ? 96 : p == P16 ? 48 : 192; }
+// Algorithmic link bytes per site of a launch: the four 12-real links (18-real in double-float) each
+// read once. That FP64 keeps the third row and double-float a slot per hop are choices of layout, not work.
+__host__ __device__ constexpr int link_site_bytes(int p) {
+  return p == P64E ? 4 * 18 * 8 : 4 * 12 * (p == P64 ? 8 : p == P32 ? 4 : 2);
+}
 // double-float: blocks of 32 pairs of sites, the last one padded
 __host__ __device__ constexpr int df_blocks(int V) { return (V / 2 + 31) / 32; }
 // bytes of one spinor field (F16: without its scales)

@@ -633,7 +633,7 @@ static ovl_status sign_op_batch_lz(ovl_ctx* c, int mode, const Field& v, int vof
   OVL_TRY(upload_eta_coef(c, n, eta, coef, &d_eta, &d_coef));
   const LinkRef L = links_of(c, PL);
   const int wcls = PL == P64E ? 8 : PL;
-  const double lbytes = (PL == P64E || PL == P64 ? 576.0 : PL == P32 ? 192.0 : 96.0) * V;
+  const double lbytes = (double)link_site_bytes(PL) * V;
   const double sbytes = (double)spinor_bytes(PB) * V, rbytes = (double)spinor_bytes(PR) * V;
   double* ahist = c->lz_hist;
   double* bhist = c->lz_hist + (size_t)c->lz_n * c->lz_cap;
@@ -854,10 +854,7 @@ static ovl_status sign_op_batch(ovl_ctx* c, int mode, const Field& v, int voff, 
   OVL_TRY(upload_eta_coef(c, n, eta, coef, &d_eta, &d_coef));
   const LinkRef L = links_of(c, PL);
   const int wcls = PL == P64E ? 8 : PL;  // profiler class of the Wilson launches
-  // algorithmic link bytes per site and launch: four 18-real links in FP64 and for the
-  // double-float kernel (its eight-slot field stores each link twice, forward and
-  // transposed, which is a layout choice, not work), four 12-real links otherwise
-  const double lbytes = (PL == P64E || PL == P64 ? 576.0 : PL == P32 ? 192.0 : 96.0) * V;
+  const double lbytes = (double)link_site_bytes(PL) * V;
   const double sbytes = (double)spinor_bytes(PP) * V, rbytes = (double)spinor_bytes(PR) * V;
   ProfPair pp;
 
