@@ -102,8 +102,10 @@ __device__ __forceinline__ void accumulate(cpx<T> acc[12], const cpx<T> w[6]) {
 // against 1.4e-16). The diagonal entry of the row comes last in both chains: on smooth fields it is
 // nearly one and the others are small, so that only two of the seven roundings are of the size of
 // the sum, three on average in the order of the columns: FP32 K on 24^3 x 48 5.45e-8 of the norm,
-// 5.70e-8 in the order of the columns, 5.65e-8 as three products. With the stored third row: K of 12 FP64 systems on 16^3 x 32 4.16 -> 3.15 ms,
-// FP32 sign of 12 systems 21.3 -> 20.7 ms. S = +1: a b, -1: conj(a) b; (a2, b2) the diagonal entry's.
+// 5.70e-8 in the order of the columns, 5.65e-8 as three products; FP64 K on 16^3 x 32 1.344e-16,
+// 1.376e-16 and 1.369e-16. With the stored third row: K of 12 FP64 systems on 16^3 x 32 4.16 -> 3.15 ms,
+// FP32 sign of 12 systems 21.3 -> 20.8 ms (20.7 in the order of the columns). S = +1: a b, -1: conj(a) b;
+// (a2, b2) the diagonal entry's.
 template <int S, typename T>
 __device__ __forceinline__ cpx<T> dot3(cpx<T> a0, cpx<T> b0, cpx<T> a1, cpx<T> b1, cpx<T> a2, cpx<T> b2) {
   const T i0 = S > 0 ? a0.i : -a0.i, i1 = S > 0 ? a1.i : -a1.i, i2 = S > 0 ? a2.i : -a2.i;
@@ -116,7 +118,7 @@ __device__ __forceinline__ void su3_mul(const cpx<T> u[9], const cpx<T> h[6], cp
   for (int sp = 0; sp < 2; ++sp)
 #pragma unroll
     for (int a = 0; a < 3; ++a) {
-      const int b = (a + 1) % 3, c = (a + 2) % 3;
+      const int b = a == 0 ? 1 : 0, c = a == 2 ? 1 : 2;   // the other two, ascending
       w[3 * sp + a] = dot3<1>(u[3 * a + b], h[3 * sp + b], u[3 * a + c], h[3 * sp + c], u[4 * a], h[3 * sp + a]);
     }
 }
@@ -126,7 +128,7 @@ __device__ __forceinline__ void su3_dag_mul(const cpx<T> u[9], const cpx<T> h[6]
   for (int sp = 0; sp < 2; ++sp)
 #pragma unroll
     for (int a = 0; a < 3; ++a) {
-      const int b = (a + 1) % 3, c = (a + 2) % 3;
+      const int b = a == 0 ? 1 : 0, c = a == 2 ? 1 : 2;   // the other two, ascending
       w[3 * sp + a] = dot3<-1>(u[3 * b + a], h[3 * sp + b], u[3 * c + a], h[3 * sp + c], u[4 * a], h[3 * sp + a]);
     }
 }
