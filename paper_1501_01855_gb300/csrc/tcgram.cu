@@ -16,9 +16,10 @@
 // added, scaled by 2^(-7 g), into a normalised double-float (hi + lo FP32) accumulator per output;
 // the partial results of the CTAs that split the sum are added in FP64 in a fixed order.
 // The last digit is rounded to nearest; the pairs with s + t > 8 (weight 2^-63 and below) are left out.
-// The error is then that of representing each operand to 2^(e_i - 43): on Gaussian data
-// about 1e-14 of |A_i| |B_j| at 4096 reals and less on longer vectors, the level of an
-// FP64 dot product of the same length.
+// The error is then that of the representation and one rounding of 2^-48 of the running sum per 512
+// reals: on Gaussian data at most 4e-14 of |A_i| |B_j| over 70 x 70 vectors of 6144 reals with scales
+// 1e-30 to 1e30, 1e-15 for FP32 fields, and 1.3e-13 on the diagonal of vectors of 1.6 M reals that one
+// CTA sums whole (640 x 640; 7.6e-11 when the low word was not normalised).
 //
 // Complex arithmetic: vectors are read as interleaved (re, im) reals. With the A operand
 // rows [A_i (64 vectors); A'_i] where A' = (-im, re) per complex element, one MMA of
@@ -32,8 +33,8 @@
 // barrier that frees it (empty). All warps read a chunk's sums out of tensor memory once its
 // MMAs are done (fbar), two stages into the next chunk, whose MMAs wait for that (flushed). With
 // block barriers instead (two per stage, operands staged by cp.async) the warps waited for each
-// other 3.5 cycles per issued instruction. Bound now by the ALU pipe of the slicing (57% busy,
-// tensor pipe 35%). FP64 fields, 16^3 x 32: 128 x 128 17.6 -> 7.3 ms, 64 x 64 8.7 -> 2.1, 64 x 12 8.6 -> 1.7
+// other 3.5 cycles per issued instruction. Bound now by the ALU pipe of the slicing (55% busy,
+// tensor pipe 34%). FP64 fields, 16^3 x 32: 128 x 128 17.6 -> 7.3 ms, 64 x 64 8.7 -> 2.1, 64 x 12 8.6 -> 1.7
 // (more than half of that was the exponent pass, below).
 // Waits are bounded (wait_ns, 2 s by default): one that gives up sets the error flag, the CTA skips the
 // rest, warp by warp (warp_wait), waits once more (again bounded) for the MMAs it has committed, frees its tensor memory
@@ -323,40 +324,47 @@ __global__ void __launch_bounds__(TG_THREADS, 1)
 #pragma unroll
   for (int c = 0; c < TG_CPT; ++c) acc_h[c] = acc_l[c] = 0.f;
 
-  // One accumulation chunk's group sums are exact integers in FP32: add them, scaled, in
-  // double-float, and normalise the sum (|low| <= half an ulp of high), so that a low word never
-  // holds more than the errors of one chunk: however many chunks a CTA sums, each adds roundings of
-  // about 2^-48. Every warp, once the chunk's MMAs are done (fbar); false when a wait gave up.
+  // One accumulation chunk's group sums are exact integers in FP32: the three smallest weights added
+  // plainly (at most 2^-18: off by 2^-42 of a chunk whose digits are all at their bounds), the others in
+  // double-float, then one double-float addition to the running sum, which stays normalised (|low| <=
+  // half an ulp of high): however many chunks a CTA sums, each adds one rounding of 2^-48. Every
+  // warp, once the chunk's MMAs are done (fbar); false when a wait gave up.
   auto flush = [&](int chunk) -> bool {
     if (!warp_wait(smem_u32(&fbar), (uint32_t)chunk & 1u, &abort_flag, wait_ns)) return false;
     asm volatile("tcgen05.fence::after_thread_sync;");
+    constexpr int NC = 4;   // columns at a time: every group's sums loaded before one wait
 #pragma unroll
-    for (int g = 0; g < TG_G; ++g) {
-      uint32_t v[TG_CPT];
-      static_assert(TG_CPT == 16, "the flush reads 16 columns per thread");
-      const uint32_t ta_ = tmem + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)(g * TG_NB + cbase);
-      asm volatile(
-          "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
-          : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]),
-            "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]), "=r"(v[15])
-          : "r"(ta_));
+    for (int c0 = 0; c0 < TG_CPT; c0 += NC) {
+      uint32_t v[TG_G][NC];
+      const uint32_t at = tmem + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)(cbase + c0);
+#pragma unroll
+      for (int g = 0; g < TG_G; ++g)
+        asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0,%1,%2,%3}, [%4];"
+                     : "=r"(v[g][0]), "=r"(v[g][1]), "=r"(v[g][2]), "=r"(v[g][3])
+                     : "r"(at + (uint32_t)(g * TG_NB)));
       // the wait names the registers: nothing that uses them moves above it
+      static_assert(TG_G == 7 && NC == 4, "the wait below lists 28 registers");
       asm volatile("tcgen05.wait::ld.sync.aligned;"
-                   : "+r"(v[0]), "+r"(v[1]), "+r"(v[2]), "+r"(v[3]), "+r"(v[4]), "+r"(v[5]), "+r"(v[6]), "+r"(v[7]),
-                     "+r"(v[8]), "+r"(v[9]), "+r"(v[10]), "+r"(v[11]), "+r"(v[12]), "+r"(v[13]), "+r"(v[14]),
-                     "+r"(v[15])::"memory");
-      const float w = __int_as_float((127 - 7 * (g + 2)) << 23);   // 2^(-7 (g + 2))
+                   : "+r"(v[0][0]), "+r"(v[0][1]), "+r"(v[0][2]), "+r"(v[0][3]), "+r"(v[1][0]), "+r"(v[1][1]),
+                     "+r"(v[1][2]), "+r"(v[1][3]), "+r"(v[2][0]), "+r"(v[2][1]), "+r"(v[2][2]), "+r"(v[2][3]),
+                     "+r"(v[3][0]), "+r"(v[3][1]), "+r"(v[3][2]), "+r"(v[3][3]), "+r"(v[4][0]), "+r"(v[4][1]),
+                     "+r"(v[4][2]), "+r"(v[4][3]), "+r"(v[5][0]), "+r"(v[5][1]), "+r"(v[5][2]), "+r"(v[5][3]),
+                     "+r"(v[6][0]), "+r"(v[6][1]), "+r"(v[6][2]), "+r"(v[6][3])::"memory");
 #pragma unroll
-      for (int c = 0; c < TG_CPT; ++c) {
-        const float x = __uint_as_float(v[c]) * w;   // exact
-        acc_l[c] += two_sum(acc_h[c], x);
+      for (int c = 0; c < NC; ++c) {
+        auto x = [&](int g) {   // exact: times 2^(-7 (g + 2))
+          return __uint_as_float(v[g][c]) * __int_as_float((127 - 7 * (g + 2)) << 23);
+        };
+        float ch = x(3), cl = (x(6) + x(5)) + x(4);
+        cl += two_sum(ch, x(2));
+        cl += two_sum(ch, x(1));
+        cl += two_sum(ch, x(0));
+        float &h = acc_h[c0 + c], &l = acc_l[c0 + c];
+        l = two_sum(h, ch) + (l + cl);
+        const float r = h + l;
+        l -= r - h;
+        h = r;
       }
-    }
-#pragma unroll
-    for (int c = 0; c < TG_CPT; ++c) {
-      const float h = acc_h[c] + acc_l[c];
-      acc_l[c] -= h - acc_h[c];
-      acc_h[c] = h;
     }
     asm volatile("tcgen05.fence::before_thread_sync;");
     __syncwarp();
