@@ -57,17 +57,18 @@ NVEC = 16
 LINK_SEED, SRC_SEED = 1002, 2002
 WILSON_FLOPS_PER_SITE = 1320          # conventional count of the hopping term
 FP64_NOMINAL_TFLOPS = 1.25            # GB300 FP64 (nominal; the ALU roofline of the FP64 kernel)
-# FP32 operations one double-float site application needs by construction: per neighbour
-# 12 lazy double-float sums for the projection (8 each), 12 link-product components as
-# 6-term Dot2 sums (4 + 5 x 12 each) and 24 lazy sums into the accumulator (8 each) =
-# 1056; x 8 neighbours, plus the diagonal term in - kappa hop (24 x (7 + 11)). Loads,
-# index arithmetic, phase selects and the epilogue reductions are not counted.
-DF64_FP32_OPS_PER_SITE = 8 * (12 * 8 + 12 * (4 + 5 * 12) + 24 * 8) + 24 * (7 + 11)
+# FP32 operations one double-float site application needs by construction (a packed operation
+# counts two, one per site of its pair): per neighbour 12 lazy double-float sums for the projection
+# (8 each), 18 negations of its words, 12 link-product components as 6-term compensated sums
+# (5 + 5 x 10 each) and 24 lazy sums into the accumulator (8 each) = 966; x 8 neighbours, plus 24
+# renormalisations (3 each) and the diagonal term in - kappa hop (24 x (8 + 11)). Loads, index
+# arithmetic and the epilogue reductions are not counted.
+DF64_FP32_OPS_PER_SITE = 8 * (12 * 8 + 18 + 12 * (5 + 5 * 10) + 24 * 8) + 24 * 3 + 24 * (8 + 11)
 # DRAM bytes (read + write) per launch of the double-float Wilson kernel in this step: the
 # mean of the first six timed launches (three of each Lanczos mode) in one ncu capture of
 # this command (profiles/launches_overlap_apply_lanczos_df64_16x16x16x32.md); each mode moves
-# 1.18-1.19 x its algorithmic bytes.
-TRAFFIC_WILSON_DF64 = 1.44e9
+# 1.71-1.77 x its algorithmic bytes.
+TRAFFIC_WILSON_DF64 = 2.11e9
 # Algorithmic bytes of one Wilson launch, per site: every system reads its input spinor
 # and writes its output (K mode) or also reads p and r and writes r (r-update mode); the
 # four 18-real FP64 links of the site (576 B) are read once per launch.
@@ -359,7 +360,7 @@ def run_ours(args, ws, rank, local):
     d = prof[dom]
     avg_ms = d["ms"] / max(1, d["launches"])
     ach = d["bytes"] / (d["ms"] * 1e-3) / 1e9
-    names = {"wilson_f64e": "wilson_kernel (double-float; the Lanczos K and three-term-recurrence launches + "
+    names = {"wilson_f64e": "df_wilson_kernel (double-float; the Lanczos K and three-term-recurrence launches + "
                             "the final overlap epilogue)",
              "mscg_update": "lz_combine_df_kernel (y from the stored Lanczos basis)"}
     roof = {"kernel": names.get(dom, dom), "bound": "hbm", "achieved": ach, "peak": hbm, "unit": "GB/s",
