@@ -90,9 +90,12 @@ typedef struct {
                            thread per site on 8x4x4x2 tiles (needs extents divisible by those),
                            3 as 0. Double-float (two threads per pair of sites, one per half
                            spinor): 0, 3, 2, 1 share the eight hops of a pair among 1, 2, 4, 8
-                           groups of threads; -1 takes the number by the size of each launch  */
-  int    use_graphs;    /* 1 (default): run the multi-shift CG iterations as cached CUDA graphs
-                           (not while profiling); 0: launch every kernel on the stream        */
+                           groups of threads; -1 takes the number by the size of each launch.
+                           Any but -1 also turns the one-launch Lanczos cycles off           */
+  int    use_graphs;    /* 1 (default): run small Lanczos cycles as one launch (see
+                           ovl_lanczos_cycles) and the other sign iterations as cached CUDA
+                           graphs (these not while profiling); 0: launch every kernel on the
+                           stream                                                             */
   int    verify;        /* 1: after a solve, recompute ||b - D x|| / ||b|| with an FP64 sign at
                            eps_sign (one more sign application per system); 0: report the
                            GMRESR recursive residual. Default 1                                 */

@@ -15,9 +15,9 @@
 // leaves the instruction cache): a power of i only chooses which of the two chunks (re, im)
 // of the lower spin is loaded into which operand, and a sign, which rides on a multiply-add.
 //
-// What bounds it (ncu, 16^3 x 32, K): the FP32 pipes are busy 61% of the cycles (527 packed
-// operations per thread and hop), the rest is the latency of the loads that three warps per
-// scheduler do not cover. 168 registers (12 warps per SM) against 128 (16 warps, spilling and
+// What bounds it (ncu, 16^3 x 16, 6 systems, Lanczos modes): the FP32 pipes are busy 55% to 58% of the
+// cycles (527 packed operations per thread and hop), the rest is the latency of the loads that three
+// warps per scheduler do not cover. 168 registers (12 warps per SM) against 128 (16 warps, spilling and
 // scheduled with less overlap): 0.530 against 0.841 ms on 16^3 x 32 with 12 systems. Measured there
 // against the scalar kernel before it (one thread per site, 12 operations per product term):
 // K launch 0.678 -> 0.517 ms, on 24^3 x 48 2.61 ms (3.0 G site applications/s; 2.4 before), one
@@ -394,9 +394,10 @@ void run_m(const DArgs& a, cudaStream_t st) {
     case 3: run_g<MODE, PIO, 2>(a, st); break;
     case 2: run_g<MODE, PIO, 4>(a, st); break;
     default:
-      // small blocks where the caller does not read partial sums per 64 sites
+      // small blocks where the caller does not read partial sums per 64 sites and where blocks of 32
+      // pairs would leave half of the 152 SMs without one
       if constexpr (MODE == MODE_LZK || MODE == MODE_LZL || MODE == MODE_K) {
-        if ((long long)a.g.V * a.nrhs <= 4864 && (MODE != MODE_K || a.partials == nullptr)) {
+        if ((long long)a.g.V * a.nrhs <= 32 * 152 && (MODE != MODE_K || a.partials == nullptr)) {
           run_g<MODE, PIO, 8, 8>(a, st);
           break;
         }
@@ -544,7 +545,7 @@ bool launch_lz_persistent_df(LzPersist& p, LzpShape* shape, int nsm, cudaStream_
 
 // Two threads per pair and system, times 1, 2, 4 or 8 groups. One group is the cheapest form
 // (no exchange in shared memory) once its threads fill the SMs; below, the hops of a pair are
-// spread over more groups. K launches, us with 1 / 2 / 4 / 8 groups: 49152 threads (8^4, 12
+// spread over more groups. The lines are those of the 152 SMs they were measured on. K launches, us with 1 / 2 / 4 / 8 groups: 49152 threads (8^4, 12
 // systems) 24.6 / 24.7 / 30.8 / 32.9; 32768 (8^3 x 16, 4) 18.5 / 18.5 / 22.6 / 22.6; 20736 (12^4, 1)
 // 18.5 / 14.5 / 18.5 / 18.6; 16384 (8^4, 4) 14.4 / 12.4 / 12.4 / 12.6; 8192 (8^3 x 16, 1)
 // 14.4 / 10.3 / 8.3 / 8.3; 4096 (8^4, 1) 14.4 / 10.4 / 8.3 / 8.2.

@@ -17,7 +17,7 @@
 // the partial results of the CTAs that split the sum are added in FP64 in a fixed order.
 // The last digit is rounded to nearest; the pairs with s + t > 8 (weight 2^-63 and below) are left out.
 // The error is then that of the representation and one rounding of 2^-48 of the running sum per 512
-// reals: on Gaussian data at most 4e-14 of |A_i| |B_j| over 70 x 70 vectors of 6144 reals with scales
+// reals: on Gaussian data at most 4.2e-14 of |A_i| |B_j| over 70 x 70 vectors of 6144 reals with scales
 // 1e-30 to 1e30, 1e-15 for FP32 fields, and 1.3e-13 on the diagonal of vectors of 1.6 M reals that one
 // CTA sums whole (640 x 640; 7.6e-11 when the low word was not normalised).
 //
